@@ -779,10 +779,8 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
     // renamed into degree-class order
     for (int i = 0; i < slices; ++i) {
         KCHK2(cudaStreamWaitEvent(h->stream, ev[i], 0), "event");
-        KCHK2(remap_src_rows(rp64, col0, g.inv, rp_new, vcut[i], vcut[i + 1], n, row_warp, g.col, d_bad + 1,
-                             h->stream), "relabel rows");
-        KCHK2(remap_hub_chunks(rp64, col0, g.perm, g.inv, rp_new, g.chunk_row, g.chunk_first, row_warp, chunks_cap,
-                               vcut[i], vcut[i + 1], n, g.col, d_bad + 1, h->stream), "relabel hub rows");
+        KCHK2(remap_rows(rp64, col0, g.inv, rp_new, vcut[i], vcut[i + 1], acut[i], acut[i + 1], n, g.col, d_bad + 1,
+                         h->stream), "relabel rows");
     }
     // then the low-degree rows reordered inside their classes by anchor
     // (katz_opts.locality); the rows of degree > 16 keep their places, the

@@ -283,15 +283,10 @@ cudaError_t exclusive_scan_i64(const int64_t* in, int64_t n, int64_t* out, int64
 // new row offsets (int64, n+1) of the relabelled adjacency
 cudaError_t relabel_offsets(const int64_t* rowptr64, const int32_t* perm, int64_t n, int64_t* deg_new_scratch,
                             int64_t* rowptr_new, int64_t* sums_scratch, cudaStream_t st);
-// arcs of the original rows [v0, v1) that do not become CHUNK rows, renamed
-// into their new rows; then those of the CHUNK rows among them, chunk by chunk
-cudaError_t remap_src_rows(const int64_t* rowptr64, const int32_t* col, const int32_t* inv, const int64_t* rowptr_new,
-                           int64_t v0, int64_t v1, int64_t n, int64_t row_warp, int32_t* col_new,
-                           unsigned long long* bad, cudaStream_t st);
-cudaError_t remap_hub_chunks(const int64_t* rowptr64, const int32_t* col, const int32_t* perm, const int32_t* inv,
-                             const int64_t* rowptr_new, const int32_t* chunk_row, const int64_t* chunk_first,
-                             int64_t row_warp, int64_t chunks_cap, int64_t v0, int64_t v1, int64_t n,
-                             int32_t* col_new, unsigned long long* bad, cudaStream_t st);
+// arcs [a0, a1) = those of the original rows [v0, v1), renamed into their new rows
+cudaError_t remap_rows(const int64_t* rowptr64, const int32_t* col, const int32_t* inv, const int64_t* rowptr_new,
+                       int64_t v0, int64_t v1, int64_t a0, int64_t a1, int64_t n, int32_t* col_new,
+                       unsigned long long* bad, cudaStream_t st);
 // chunk table of the CHUNK rows from the new offsets: chunk_first (row_warp + 1
 // entries, exclusive scan of the chunk counts), chunk_row, and the largest count
 cudaError_t build_chunk_table(const int64_t* rowptr_new, int64_t row_warp, int64_t* cnt_scratch, int64_t* sums_scratch,
