@@ -188,9 +188,11 @@ enum {
  * Algorithm 1 (Sec. 3.2) with any stopping criterion of Sec. 3.1.
  * KATZ_CRIT_TOPK: the same as katz_rank_static(h, alpha, k, eps, info).
  * The others run on FP64 handles and keep every node active:
- *   KATZ_CRIT_RANKING: each iteration sorts all n nodes by (l desc, id asc)
- *     and checks every adjacent pair (Eq. 3); afterwards katz_get_ranking
- *     returns the full certified order (k up to n);
+ *   KATZ_CRIT_RANKING: every pair of nodes must be separated (Eq. 3).  An
+ *     iteration with an unseparated pair among those first looked at (the
+ *     neighbours in the last sorted order) ends there; else all n nodes are
+ *     sorted by (l desc, id asc) and every adjacent pair is checked.
+ *     Afterwards katz_get_ranking returns the full certified order (k up to n);
  *   KATZ_CRIT_SCORE: stops once u_r - l_r < eps at every node; the bounds
  *     (katz_get_bounds) then give every score to within eps, and there is
  *     no ranking (katz_get_ranking returns KATZ_ESTATE);

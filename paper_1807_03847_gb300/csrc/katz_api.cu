@@ -1020,7 +1020,6 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
         const int64_t cnt = 256 * radix_tiles(n);
         if ((e = dmalloc(h, &h->rank_ids, (size_t)n)) != cudaSuccess ||
             (e = dmalloc(h, &rs.hi[0], (size_t)n)) != cudaSuccess || (e = dmalloc(h, &rs.hi[1], (size_t)n)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.lo[0], (size_t)n)) != cudaSuccess || (e = dmalloc(h, &rs.lo[1], (size_t)n)) != cudaSuccess ||
             (e = dmalloc(h, &rs.val[0], (size_t)n)) != cudaSuccess ||
             (e = dmalloc(h, &rs.val[1], (size_t)n)) != cudaSuccess ||
             (e = dmalloc(h, &rs.counts, (size_t)cnt)) != cudaSuccess ||
@@ -1032,7 +1031,6 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     h->ranked = false;
     h->launches = 0;
     const int64_t spmv_kernels = h->g.layout.row_warp > 0 ? 2 : 1;
-    const int64_t check_kernels = criterion == KATZ_CRIT_RANKING ? 2 + 12 * 5 : 1;  // keys, 12 x (hist, scan 3, scatter), check
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
     if ((e = cudaMemsetAsync(h->b.ctrl, 0, sizeof(Ctrl), h->stream)) != cudaSuccess ||
         (e = launch_init_walk(h->g, h->b, p, false, h->stream)) != cudaSuccess ||
@@ -1040,22 +1038,37 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
         (e = launch_crit_init(h->b, h->stream)) != cudaSuccess)
         return cuda_fail(h, e, "init");
     h->launches += 3;
-    for (int it = 0; it < p.r_max; ++it) {
-        // level 1 is the degree vector (A 1 = deg), one O(n) pass
-        e = it == 0 ? launch_degree_level(h->g, h->b, p, h->stream) : launch_spmv(h->g, h->b, p, false, h->stream);
-        if (e != cudaSuccess) return cuda_fail(h, e, "spmv");
-        if (criterion == KATZ_CRIT_RANKING)
-            e = launch_ranking_check(h->g, h->b, p, h->rs, h->rank_ids, h->stream);
-        else if (criterion == KATZ_CRIT_SCORE)
-            e = launch_score_check(h->b, p, h->stream);
-        else
-            e = launch_pair_check(h->g, h->b, p, oa, ob, h->stream);
-        if (e != cudaSuccess) return cuda_fail(h, e, "criterion");
-        if ((e = launch_finalize_crit(h->b, p, h->stream)) != cudaSuccess) return cuda_fail(h, e, "finalize");
-        h->launches += (it == 0 ? 1 : spmv_kernels) + check_kernels + 1;
-        if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
-            return cuda_fail(h, e, "sync");
+    // Levels are launched four at a time (a launch after the loop stopped, or
+    // paused for a sort, returns at once), the control block read in between.
+    const bool ranking = criterion == KATZ_CRIT_RANKING;
+    const int32_t* order = nullptr;  // the last sorted order (none yet: the internal one)
+    for (int it = 0;;) {
+        for (int q = 0; q < 4; ++q, ++it) {
+            // level 1 is the degree vector (A 1 = deg), one O(n) pass
+            e = it == 0 ? launch_degree_level(h->g, h->b, p, h->stream) : launch_spmv(h->g, h->b, p, false, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "spmv");
+            if (ranking)
+                e = launch_ranking_witness(h->g, h->b, p, order, h->stream);
+            else if (criterion == KATZ_CRIT_SCORE)
+                e = launch_score_check(h->b, p, h->stream);
+            else
+                e = launch_pair_check(h->g, h->b, p, oa, ob, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "criterion");
+            if ((e = launch_finalize_crit(h->b, p, ranking, h->stream)) != cudaSuccess)
+                return cuda_fail(h, e, "finalize");
+            h->launches += (it == 0 ? 1 : spmv_kernels) + 2;
+        }
+        for (;;) {
+            if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) !=
+                    cudaSuccess ||
+                (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
+                return cuda_fail(h, e, "sync");
+            if (h->h_ctrl->stop != STOP_SORT) break;
+            if ((e = launch_ranking_check(h->g, h->b, p, h->rs, h->rank_ids, &order, h->stream)) != cudaSuccess ||
+                (e = launch_finalize_crit(h->b, p, false, h->stream)) != cudaSuccess)
+                return cuda_fail(h, e, "ranking check");
+            h->launches += 3 + 8 * 5 + 1;  // resume, keys, 8 x (hist, scan 3, scatter), check, finalize
+        }
         if (h->h_ctrl->stop) break;
     }
     if ((e = cudaEventRecord(h->ev1, h->stream)) != cudaSuccess ||

@@ -27,6 +27,8 @@ constexpr int CHUNK_ARCS = 2048;  // arcs per warp for rows of degree > 2048
 constexpr int SELECT_CAP = KATZ_MAX_K;
 constexpr int SELECT_THREADS = 1024;
 
+constexpr int32_t STOP_SORT = 2;  // Ctrl::stop while a level waits for its sort
+
 enum : int32_t { DYN_E_INVAL = 1, DYN_E_ALPHA = 2 };  // batch validation failures
 
 // Iteration state kept on the device so that a captured graph can loop
@@ -34,7 +36,7 @@ enum : int32_t { DYN_E_INVAL = 1, DYN_E_ALPHA = 2 };  // batch validation failur
 struct Ctrl {
     int32_t r;           // iterations completed
     int32_t converged;   // result of the last converged() evaluation
-    int32_t stop;        // 1: leave the loop
+    int32_t stop;        // 1: leave the loop; STOP_SORT: paused for the ranking criterion's sort
     int32_t flags;       // reserved (0)
     unsigned long long n_cand;     // |{v in M : l_r(v) >= theta_{r-1}}|
     unsigned long long cnt_cross;  // active nodes outside the top-k with u_r - eps >= theta_r
@@ -232,7 +234,7 @@ struct RadixBuffers {
     int64_t* sums = nullptr;    // scan scratch
 };
 int64_t radix_tiles(int64_t n);
-cudaError_t radix_sort_passes(RadixBuffers& rs, int64_t n, int first, int last, int& cur, cudaStream_t st);
+cudaError_t radix_sort_passes(RadixBuffers& rs, int64_t n, int first, int last, bool lo, int& cur, cudaStream_t st);
 // anchor order of the low-degree rows (internal ids >= start) of a graph
 // already renamed into degree-class order; see katz_relabel.cu
 cudaError_t locality_order(int64_t n, int64_t nnz, int64_t start, const int64_t* rowptr1, int32_t* col1,
@@ -243,8 +245,10 @@ cudaError_t launch_score_check(const IterBuffers& b, const IterParams& p, cudaSt
 cudaError_t launch_pair_check(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int32_t oa, int32_t ob,
                               cudaStream_t st);
 cudaError_t launch_ranking_check(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, RadixBuffers& rs,
-                                 int32_t* rank_ids, cudaStream_t st);
-cudaError_t launch_finalize_crit(const IterBuffers& b, const IterParams& p, cudaStream_t st);
+                                 int32_t* rank_ids, const int32_t** order, cudaStream_t st);
+cudaError_t launch_ranking_witness(const DeviceGraph& g, const IterBuffers& b, const IterParams& p,
+                                   const int32_t* order, cudaStream_t st);
+cudaError_t launch_finalize_crit(const IterBuffers& b, const IterParams& p, bool witness, cudaStream_t st);
 
 cudaError_t dyn_validate(const DeviceGraph& g, const DynBuffers& d, int64_t m, int64_t D, cudaStream_t st);
 cudaError_t dyn_clear(const DeviceGraph& g, const DynBuffers& d, int64_t m, cudaStream_t st);

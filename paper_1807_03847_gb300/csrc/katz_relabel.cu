@@ -431,8 +431,8 @@ cudaError_t locality_order(int64_t n, int64_t nnz, int64_t start, const int64_t*
     tail_keys_kernel<<<grid_for(m, 256), 256, 0, st>>>(rowptr1, col1, perm, n, start, packed ? abits : 0, rs.hi[0],
                                                        rs.lo[0], rs.val[0]);
     int cur = 0;
-    cudaError_t e = packed ? radix_sort_passes(rs, m, 0, (abits + 3 + 7) / 8 - 1, cur, st)
-                           : radix_sort_passes(rs, m, 0, 4, cur, st);  // the anchor (4 digits), then the class
+    cudaError_t e = packed ? radix_sort_passes(rs, m, 0, (abits + 3 + 7) / 8 - 1, true, cur, st)
+                           : radix_sort_passes(rs, m, 0, 4, true, cur, st);  // the anchor (4 digits), then the class
     if (e != cudaSuccess) return e;
     const int32_t* sorted = rs.val[cur];
     int32_t* sigma = (int32_t*)rs.lo[1 - cur];
