@@ -12,24 +12,49 @@
 // array of fixed size, present on every device that loads the library.
 //
 // Its work is the selection and checking half of an iteration of the
-// library's main loop (a radix select of the k largest lower bounds, a
-// one-CTA sort of them, and the separation count), run over all n nodes.
+// library's main loop, run over all n nodes:
+//   groups   the nodes fall into 8192 groups by a hash of their id; the k-th
+//            largest of the groups' largest lower bounds, cut to its upper 32
+//            bits, is reached by at least k nodes, and by few more (about 1660
+//            for k = 1500, wherever the large bounds lie);
+//   compact  the nodes that reach it, the candidates;
+//   radix    only when they outgrow the candidate buffer (many equal bounds,
+//            k above 4096): a radix select of the k-th 96-bit key, in kernels
+//            that return at once otherwise (1 us each; one cooperative kernel
+//            instead took 190 us more per call when calls are queued);
+//   rank     each candidate's place by counting those before it;
+//   cross    the separation of the top-k from each other and from the rest.
+// Each of the three passes over the nodes reads one array of 8 n bytes.  A
+// radix select over all nodes with a sort in one block took 419 us at n = 4 M,
+// k = 1000 (230 of them in global atomics on the few bins that hold most
+// bounds); these kernels take 100 us, launches included.
 #include <cuda_runtime.h>
+#include <math_constants.h>
 #include <stdint.h>
 
 #include <mutex>
 
 #include "../../include/katz.h"
+#include "katz_grid.cuh"
 
 namespace {
 
+using katz::last_block;
+
 constexpr int NA_BINS = 65536;          // 16-bit digits
-constexpr int NA_CAP = KATZ_MAX_K;      // candidates sorted in one CTA
-constexpr int NA_THREADS = 1024;
+constexpr int NA_CAP = KATZ_MAX_K;      // candidates held
 constexpr int NA_MAX_DEVICES = 64;
+constexpr int NA_GROUPS = 8192;
+constexpr int NA_GROUP_THREADS = 512;
+constexpr int NA_GROUP_BLOCKS = 128;    // 65536 threads, eight for each group
+constexpr int NA_GROUP_MAX_K = NA_GROUPS / 2;  // above: more nodes than candidates would reach the k-th group
+constexpr int NA_RADIX_THREADS = 512;
 
 struct NoAllocScratch {
-    unsigned int hist[NA_BINS];
+    unsigned int hist[NA_BINS];    // radix: histogram; groups: largest bound of each thread; rank: the order
+    unsigned int ticket;           // last_block: zero between kernels
+    int use_radix;
+    unsigned int group_key;        // candidates: upper 32 key bits at or above it
     unsigned long long cand_count;
     unsigned long long cross;
     unsigned long long above;      // keys known to lie above the current bucket
@@ -37,14 +62,11 @@ struct NoAllocScratch {
     unsigned long long pre_hi;     // selected digits so far (96-bit key: hi 64, lo 32)
     unsigned int pre_lo;
     int done;                      // threshold found
-    int pairs_bad;
-    int pad;
     unsigned long long thr_hi;     // candidates: key >= (thr_hi, thr_lo)
     unsigned int thr_lo;
-    double theta;                  // k-th lower bound
-    int theta_id;
+    int theta_id;                  // k-th node
     unsigned long long theta_key;
-    double cand_l[NA_CAP];
+    unsigned long long cand_key[NA_CAP];
     double cand_u[NA_CAP];
     int cand_id[NA_CAP];
 };
@@ -67,13 +89,44 @@ __device__ __forceinline__ unsigned long long order_bits(double l) {
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
+__device__ __forceinline__ double bound_of(unsigned long long key) {  // the inverse
+    return __longlong_as_double((long long)((key >> 63) ? key & 0x7fffffffffffffffull : ~key));
+}
+
 __device__ __forceinline__ u128 key_of(double l, int v) {
     return ((u128)order_bits(l) << 32) | (u128)(0xffffffffu ^ (unsigned)v);
 }
 
-__global__ void na_reset(NoAllocScratch* S, long long k) {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NA_BINS; q += gridDim.x * blockDim.x) S->hist[q] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+// The largest lower bound (upper 32 key bits; 0: no node) of thread t's nodes
+// i 65536 + (t ^ mix(i)), i = 0, 1, ...; the last block takes the k-th largest
+// over the groups of eight threads s 8192 + (g ^ mix(s)).  Neighbouring large
+// bounds (a sorted array) fall into different groups, and so do those of ids
+// that differ in a few bits (the hubs of an R-MAT graph: 7700 candidates for k
+// = 1000 with groups v mod 8192).  A warp reads whole 256-byte segments.
+__device__ __forceinline__ unsigned int mix(unsigned int i) { return (i * 0x9E3779B1u) >> 16; }
+
+__global__ void __launch_bounds__(NA_GROUP_THREADS)
+na_groups(NoAllocScratch* S, const double* __restrict__ lower, long long n, long long k) {
+    constexpr unsigned int T = NA_GROUP_THREADS * NA_GROUP_BLOCKS;
+    static_assert(T == 65536, "mix() gives 16 bits");
+    constexpr int U = 16;
+    const int tid = threadIdx.x;
+    const unsigned int t = blockIdx.x * NA_GROUP_THREADS + tid;
+    const unsigned int rounds = (unsigned int)((n + T - 1) / T);
+    unsigned int m = 0;
+    for (unsigned int i = 0; i < rounds; i += U) {
+        double x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const long long v = (long long)(i + q) * T + (t ^ mix(i + q));
+            x[q] = v < n ? __ldg(lower + v) : -CUDART_INF;  // its key is below any other's
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) m = max(m, (unsigned int)(order_bits(x[q]) >> 32));
+    }
+    S->hist[t] = m;
+    if (!last_block(&S->ticket)) return;
+    if (tid == 0) {
         S->cand_count = 0;
         S->cross = 0;
         S->above = 0;
@@ -81,15 +134,153 @@ __global__ void na_reset(NoAllocScratch* S, long long k) {
         S->pre_hi = 0;
         S->pre_lo = 0;
         S->done = 0;
-        S->pairs_bad = 0;
+        S->use_radix = k > NA_GROUP_MAX_K && n > NA_CAP;
+        S->group_key = 0;  // unless the groups give one below: every node is taken
+    }
+    if (k > NA_GROUP_MAX_K || n <= NA_CAP) return;
+    __syncthreads();
+    constexpr int PER = NA_GROUPS / NA_GROUP_THREADS;
+    unsigned int g[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        unsigned int x = 0;
+#pragma unroll
+        for (unsigned int s = 0; s < T / NA_GROUPS; ++s)
+            x = max(x, __ldcg(&S->hist[s * NA_GROUPS + ((q * NA_GROUP_THREADS + tid) ^ (mix(s) % NA_GROUPS))]));
+        g[q] = x;
+    }
+    // the largest key that at least k groups reach, two bits a step
+    __shared__ int s_cnt[16][3];
+    if (tid < 48) (&s_cnt[0][0])[tid] = 0;
+    __syncthreads();
+    unsigned int key = 0;
+    for (int step = 0; step < 16; ++step) {
+        const int sh = 30 - 2 * step;
+        int c[3] = {0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+#pragma unroll
+            for (unsigned int d = 0; d < 3; ++d) c[d] += g[q] >= (key | ((d + 1) << sh));
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            c[d] = __reduce_add_sync(0xffffffffu, c[d]);
+            if ((tid & 31) == 0 && c[d]) atomicAdd(&s_cnt[step][d], c[d]);
+        }
+        __syncthreads();
+        unsigned int d = 3;
+        while (d > 0 && s_cnt[step][d - 1] < (int)k) --d;
+        key |= d << sh;
+    }
+    if (tid == 0) S->group_key = key;
+}
+
+// a candidate's place in the buffer, one atomic per warp; the buffer keeps the
+// first NA_CAP (more: the count says so, and the radix pass starts over)
+__device__ __forceinline__ void add_candidate(NoAllocScratch* S, bool take, double l, const double* upper,
+                                              long long v) {
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (!m) return;
+    const int lane = threadIdx.x & 31;
+    unsigned long long base = 0;
+    if (lane == __ffs(m) - 1) base = atomicAdd(&S->cand_count, (unsigned long long)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
+    const unsigned long long pos = base + __popc(m & ((1u << lane) - 1u));
+    if (take && pos < (unsigned long long)NA_CAP) {
+        S->cand_key[pos] = order_bits(l);
+        S->cand_u[pos] = upper[v];
+        S->cand_id[pos] = (int)v;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+na_compact(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper, long long n) {
+    if (S->use_radix) return;
+    const unsigned int gk = S->group_key;
+    constexpr int U = 4;
+    const long long tile = 256LL * U;
+    for (long long base = (long long)blockIdx.x * tile; base < n; base += gridDim.x * tile) {  // warp-uniform
+        double l[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const long long v = base + q * 256 + threadIdx.x;
+            l[q] = v < n ? __ldg(lower + v) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const long long v = base + q * 256 + threadIdx.x;
+            add_candidate(S, v < n && (unsigned int)(order_bits(l[q]) >> 32) >= gk, l[q], upper, v);
+        }
+    }
+}
+
+__device__ __forceinline__ bool radix_needed(const NoAllocScratch* S) {
+    return S->use_radix || S->cand_count > (unsigned long long)NA_CAP;
+}
+
+// pick the bucket that holds the k-th key (one block); stop once all keys from
+// that bucket up fit the candidate buffer
+__device__ void radix_find(NoAllocScratch* S, int pass) {
+    __shared__ unsigned long long part[NA_RADIX_THREADS];
+    __shared__ int sel;
+    __shared__ unsigned long long cum_sel;
+    const int tid = threadIdx.x;
+    constexpr int per = NA_BINS / NA_RADIX_THREADS;
+    // thread tid owns bins [NA_BINS-1 - tid*per - (per-1), NA_BINS-1 - tid*per], visited from the top
+    unsigned long long s = 0;
+    for (int q = 0; q < per; ++q) s += __ldcg(&S->hist[NA_BINS - 1 - tid * per - q]);
+    part[tid] = s;
+    if (tid == 0) sel = -1;
+    __syncthreads();
+    for (int off = 1; off < NA_RADIX_THREADS; off <<= 1) {
+        const unsigned long long a = tid >= off ? part[tid - off] : 0ull;
+        __syncthreads();
+        part[tid] += a;
+        __syncthreads();
+    }
+    const unsigned long long k = S->k_rem;
+    unsigned long long cum = tid ? part[tid - 1] : 0ull;
+    if (cum < k && part[tid] >= k) {
+        for (int q = 0; q < per; ++q) {
+            const int b = NA_BINS - 1 - tid * per - q;
+            const unsigned long long h = __ldcg(&S->hist[b]);
+            if (cum + h >= k) {
+                sel = b;
+                cum_sel = cum;
+                break;
+            }
+            cum += h;
+        }
+    }
+    __syncthreads();
+    const int b = sel;
+    const unsigned long long hb = b >= 0 ? __ldcg(&S->hist[b]) : 0ull;
+    __syncthreads();
+    for (int q = tid; q < NA_BINS; q += NA_RADIX_THREADS) S->hist[q] = 0;  // ready for the next pass
+    if (tid == 0 && b >= 0) {
+        const int shift = 80 - 16 * pass;
+        const u128 pre = (((u128)S->pre_hi << 32) | S->pre_lo) | ((u128)(unsigned)b << shift);
+        const unsigned long long above = S->above + cum_sel;
+        if (above + hb <= (unsigned long long)NA_CAP || pass == 5) {
+            S->done = 1;
+            S->thr_hi = (unsigned long long)(pre >> 32);
+            S->thr_lo = (unsigned int)pre;
+            S->cand_count = 0;  // na_radix_compact counts again
+        } else {
+            S->above = above;
+            S->k_rem = k - cum_sel;
+            S->pre_hi = (unsigned long long)(pre >> 32);
+            S->pre_lo = (unsigned int)pre;
+        }
     }
 }
 
 // histogram of digit `pass` (bits 95-16*pass .. 80-16*pass) of the keys that
 // share the digits chosen so far; the lanes of a warp that hit the same bin
-// (bounds of one magnitude share their top digits) add once
-__global__ void na_hist(NoAllocScratch* S, const double* __restrict__ lower, long long n, int pass) {
-    if (S->done) return;
+// (bounds of one magnitude share their top digits) add once.  The last block
+// picks the bucket.
+__global__ void __launch_bounds__(NA_RADIX_THREADS)
+na_radix(NoAllocScratch* S, const double* __restrict__ lower, long long n, int pass) {
+    if (!radix_needed(S) || S->done) return;
     const int shift = 80 - 16 * pass;
     const u128 pre = ((u128)S->pre_hi << 32) | S->pre_lo;
     const int lane = threadIdx.x & 31;
@@ -104,143 +295,86 @@ __global__ void na_hist(NoAllocScratch* S, const double* __restrict__ lower, lon
         const unsigned peers = __match_any_sync(0xffffffffu, bin);
         if (bin < 0x10000u && lane == __ffs(peers) - 1) atomicAdd(&S->hist[bin], (unsigned)__popc(peers));
     }
+    if (last_block(&S->ticket)) radix_find(S, pass);
 }
 
-// pick the bucket that holds the k-th key; stop once all keys from that
-// bucket up fit the candidate buffer
-__global__ void na_find(NoAllocScratch* S, int pass) {
-    __shared__ unsigned long long part[NA_THREADS];
-    __shared__ int sel;
-    __shared__ unsigned long long cum_sel;
-    if (S->done) return;
-    const int tid = threadIdx.x;
-    constexpr int per = NA_BINS / NA_THREADS;
-    // thread tid owns bins [NA_BINS-1 - tid*per - (per-1), NA_BINS-1 - tid*per], visited from the top
-    unsigned long long s = 0;
-    for (int q = 0; q < per; ++q) s += S->hist[NA_BINS - 1 - tid * per - q];
-    part[tid] = s;
-    if (tid == 0) sel = -1;
-    __syncthreads();
-    for (int off = 1; off < NA_THREADS; off <<= 1) {
-        const unsigned long long a = tid >= off ? part[tid - off] : 0ull;
-        __syncthreads();
-        part[tid] += a;
-        __syncthreads();
-    }
-    const unsigned long long k = S->k_rem;
-    unsigned long long cum = tid ? part[tid - 1] : 0ull;
-    if (cum < k && part[tid] >= k) {
-        for (int q = 0; q < per; ++q) {
-            const int b = NA_BINS - 1 - tid * per - q;
-            const unsigned long long h = S->hist[b];
-            if (cum + h >= k) {
-                sel = b;
-                cum_sel = cum;
-                break;
-            }
-            cum += h;
-        }
-    }
-    __syncthreads();
-    const int b = sel;
-    const unsigned long long hb = b >= 0 ? S->hist[b] : 0ull;
-    __syncthreads();
-    for (int q = tid; q < NA_BINS; q += NA_THREADS) S->hist[q] = 0;  // ready for the next pass
-    if (tid == 0 && b >= 0) {
-        const int shift = 80 - 16 * pass;
-        const u128 pre = (((u128)S->pre_hi << 32) | S->pre_lo) | ((u128)(unsigned)b << shift);
-        const unsigned long long above = S->above + cum_sel;
-        if (above + hb <= (unsigned long long)NA_CAP || pass == 5) {
-            S->done = 1;
-            S->thr_hi = (unsigned long long)(pre >> 32);
-            S->thr_lo = (unsigned int)pre;
-        } else {
-            S->above = above;
-            S->k_rem = k - cum_sel;
-            S->pre_hi = (unsigned long long)(pre >> 32);
-            S->pre_lo = (unsigned int)pre;
-        }
-    }
+// before the first pass: no counts
+__global__ void na_radix_reset(NoAllocScratch* S) {
+    if (!radix_needed(S)) return;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NA_BINS; q += gridDim.x * blockDim.x) S->hist[q] = 0;
 }
 
-__global__ void na_compact(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper,
-                           long long n) {
+// after the last pass: the candidates at or above the threshold
+__global__ void __launch_bounds__(256)
+na_radix_compact(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper, long long n) {
+    if (!S->done) return;
     const u128 thr = ((u128)S->thr_hi << 32) | S->thr_lo;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        if (key_of(lower[v], (int)v) >= thr) {
-            const unsigned long long pos = atomicAdd(&S->cand_count, 1ull);
-            if (pos < (unsigned long long)NA_CAP) {
-                S->cand_l[pos] = lower[v];
-                S->cand_u[pos] = upper[v];
-                S->cand_id[pos] = (int)v;
-            }
-        }
+    for (long long base = (long long)blockIdx.x * 256; base < n; base += (long long)gridDim.x * 256) {
+        const long long v = base + threadIdx.x;
+        const double l = v < n ? lower[v] : 0.0;
+        add_candidate(S, v < n && key_of(l, (int)v) >= thr, l, upper, v);
     }
 }
 
-struct Ent {
-    unsigned long long key;
-    int id;
-    int src;
-};
-
-__device__ __forceinline__ bool before(const Ent& a, const Ent& b) {
-    return a.key > b.key || (a.key == b.key && a.id < b.id);
-}
-
-// sort the candidates by (lower desc, id asc); the first k are the ranking,
-// the k-th gives theta; adjacent top-k pairs must be eps-separated
-__global__ void na_sort(NoAllocScratch* S, long long k, double eps, int32_t* ids_out) {
-    extern __shared__ Ent e[];
-    const int tid = threadIdx.x;
+// the candidates' places in the order (lower desc, id asc): the first k are
+// the ranking (and the order that na_cross checks), the k-th gives theta
+__global__ void __launch_bounds__(katz::RANK_THREADS) na_rank(NoAllocScratch* S, long long k, int32_t* ids_out) {
     const int cnt = (int)min((unsigned long long)NA_CAP, S->cand_count);
-    int P = 1;
-    while (P < cnt) P <<= 1;
-    for (int q = tid; q < P; q += NA_THREADS)
-        e[q] = q < cnt ? Ent{order_bits(S->cand_l[q]), S->cand_id[q], q} : Ent{0ull, 0x7fffffff, -1};
-    __syncthreads();
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int q = tid; q < (P >> 1); q += NA_THREADS) {
-                const int pos = 2 * q - (q & (stride - 1));
-                const Ent a = e[pos], b = e[pos + stride];
-                const bool up = (pos & size) == 0;
-                if (up ? before(b, a) : before(a, b)) {
-                    e[pos] = b;
-                    e[pos + stride] = a;
-                }
+    // i0 is the same for every thread of a block
+    for (int i0 = blockIdx.x * katz::RANK_PER_BLOCK; i0 < cnt; i0 += gridDim.x * katz::RANK_PER_BLOCK) {
+        const int i = i0 + threadIdx.x / katz::RANK_LANES;
+        const unsigned long long key = i < cnt ? S->cand_key[i] : 0ull;
+        const int id = i < cnt ? S->cand_id[i] : 0x7fffffff;
+        const int r = katz::rank_by_count(S->cand_key, S->cand_id, cnt, key, id);
+        if (i < cnt && r < k && threadIdx.x % katz::RANK_LANES == 0) {
+            ids_out[r] = id;
+            S->hist[r] = (unsigned int)i;
+            if (r == k - 1) {
+                S->theta_key = key;
+                S->theta_id = id;
             }
-            __syncthreads();
         }
-    }
-    const int kk = (int)min((long long)cnt, k);
-    for (int q = tid; q < kk; q += NA_THREADS) {
-        ids_out[q] = e[q].id;
-        if (q > 0 && __dsub_rn(S->cand_u[e[q].src], eps) >= S->cand_l[e[q - 1].src]) S->pairs_bad = 1;
-    }
-    if (tid == 0 && kk > 0) {
-        S->theta = S->cand_l[e[kk - 1].src];
-        S->theta_id = e[kk - 1].id;
-        S->theta_key = e[kk - 1].key;
     }
 }
 
-// every node outside the top-k must be eps-separated from the k-th
-__global__ void na_cross(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper,
-                         long long n, double eps) {
-    const double th = S->theta;
-    const u128 th_key = ((u128)S->theta_key << 32) | (u128)(0xffffffffu ^ (unsigned)S->theta_id);
+// every node outside the top-k must be eps-separated from the k-th (only the
+// nodes whose upper bound reaches theta need their lower bound looked at),
+// and adjacent top-k pairs from each other; the last block gives the verdict
+__global__ void __launch_bounds__(256)
+na_cross(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper, long long n,
+         long long k, double eps, int32_t* certified_out) {
+    const double th = bound_of(S->theta_key);
+    const unsigned long long th_bits = S->theta_key;
+    const u128 th_key = ((u128)th_bits << 32) | (u128)(0xffffffffu ^ (unsigned)S->theta_id);
     unsigned long long c = 0;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        const bool in_top = key_of(lower[v], (int)v) >= th_key;
-        if (!in_top && __dsub_rn(upper[v], eps) >= th) ++c;
+    constexpr int U = 4;
+    const long long tile = 256LL * U;
+    for (long long base = (long long)blockIdx.x * tile; base < n; base += gridDim.x * tile) {
+        double u[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const long long v = base + q * 256 + threadIdx.x;
+            u[q] = v < n ? __ldg(upper + v) : 0.0;
+        }
+        // u - eps >= theta needs u >= theta (eps > 0): an integer compare first;
+        // the FP64 pipe (narrow on this GPU: it took 20 us here) sees only the
+        // warps with a node that passes
+        bool near = false;
+#pragma unroll
+        for (int q = 0; q < U; ++q) near |= order_bits(u[q]) >= th_bits;
+        if (!__any_sync(0xffffffffu, near)) continue;
+        for (int q = 0; q < U; ++q) {
+            const long long v = base + q * 256 + threadIdx.x;
+            if (v < n && __dsub_rn(u[q], eps) >= th && key_of(lower[v], (int)v) < th_key) ++c;
+        }
     }
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    for (long long r = t + 1; r < k; r += (long long)gridDim.x * 256)
+        if (__dsub_rn(S->cand_u[S->hist[r]], eps) >= bound_of(S->cand_key[S->hist[r - 1]])) ++c;
     for (int off = 16; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&S->cross, c);
-}
-
-__global__ void na_finish(NoAllocScratch* S, int32_t* certified_out) {
-    *certified_out = (S->cross == 0 && !S->pairs_bad) ? 1 : 0;
+    if (last_block(&S->ticket) && threadIdx.x == 0)
+        *certified_out = __ldcg(&S->cross) == 0;
 }
 
 // Address of the scratch array on the current device and the device's
@@ -254,9 +388,6 @@ katz_status scratch_on_current_device(NoAllocScratch** out, int* sms) {
         int count = 0;
         if (cudaGetSymbolAddress(&p, g_noalloc) != cudaSuccess) return KATZ_ECUDA;
         if (cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || count < 1)
-            return KATZ_ECUDA;
-        if (cudaFuncSetAttribute(na_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 NA_CAP * (int)sizeof(Ent)) != cudaSuccess)
             return KATZ_ECUDA;
         g_sms[dev] = count;
         g_addr[dev] = (NoAllocScratch*)p;
@@ -282,16 +413,19 @@ extern "C" katz_status katz_certify_topk_noalloc(const double* lower, const doub
     katz_status st = scratch_on_current_device(&S, &sms);
     if (st != KATZ_OK) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    const long long nn = (long long)n, kk = (long long)k;
     const long long cap = 8LL * sms;  // eight 256-thread blocks per multiprocessor, grid-stride beyond
-    const int grid = (int)((n + 255) / 256 < cap ? (n + 255) / 256 : cap);
-    na_reset<<<64, 1024, 0, s>>>(S, (long long)k);
-    for (int pass = 0; pass < 6; ++pass) {
-        na_hist<<<grid, 256, 0, s>>>(S, lower, (long long)n, pass);
-        na_find<<<1, NA_THREADS, 0, s>>>(S, pass);
+    const int grid = (int)((n + 1023) / 1024 < cap ? (n + 1023) / 1024 : cap);
+    na_groups<<<NA_GROUP_BLOCKS, NA_GROUP_THREADS, 0, s>>>(S, lower, nn, kk);
+    na_compact<<<grid, 256, 0, s>>>(S, lower, upper, nn);
+    if (n > NA_CAP) {  // else every node fits
+        const int rgrid = (int)((n + NA_RADIX_THREADS - 1) / NA_RADIX_THREADS < cap / 2
+                                    ? (n + NA_RADIX_THREADS - 1) / NA_RADIX_THREADS : cap / 2);
+        na_radix_reset<<<64, 1024, 0, s>>>(S);
+        for (int pass = 0; pass < 6; ++pass) na_radix<<<rgrid, NA_RADIX_THREADS, 0, s>>>(S, lower, nn, pass);
+        na_radix_compact<<<grid, 256, 0, s>>>(S, lower, upper, nn);
     }
-    na_compact<<<grid, 256, 0, s>>>(S, lower, upper, (long long)n);
-    na_sort<<<1, NA_THREADS, NA_CAP * sizeof(Ent), s>>>(S, (long long)k, eps, ids_out);
-    na_cross<<<grid, 256, 0, s>>>(S, lower, upper, (long long)n, eps);
-    na_finish<<<1, 1, 0, s>>>(S, certified_out);
+    na_rank<<<NA_CAP / katz::RANK_PER_BLOCK, katz::RANK_THREADS, 0, s>>>(S, kk, ids_out);
+    na_cross<<<grid, 256, 0, s>>>(S, lower, upper, nn, kk, eps, certified_out);
     return cudaGetLastError() == cudaSuccess ? KATZ_OK : KATZ_ECUDA;
 }
