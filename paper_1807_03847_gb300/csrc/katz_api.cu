@@ -77,7 +77,6 @@ cudaMemPool_t library_pool(int dev) {
 katz_status init_handle_runtime(katz_handle* h) {
     cudaError_t e;
     if ((e = cudaGetDevice(&h->dev)) != cudaSuccess) return cuda_fail(h, e, "cudaGetDevice");
-    if ((e = prepare_kernels()) != cudaSuccess) return cuda_fail(h, e, "prepare kernels");
     if (h->opts.cuda_stream) {
         h->stream = (cudaStream_t)h->opts.cuda_stream;
         h->own_stream = false;
@@ -118,6 +117,9 @@ void free_iter(katz_handle* h) {
     dfree(h, b.cand_l);
     dfree(h, b.cand_u);
     dfree(h, b.cand_id);
+    dfree(h, b.sel.key);
+    dfree(h, b.sel.id);
+    dfree(h, b.sel.src);
     dfree(h, b.topk_id);
     dfree(h, b.topk_l);
     dfree(h, b.topk_u);
@@ -161,8 +163,18 @@ katz_status ensure_iter_buffers(katz_handle* h) {
     KALLOC(b.topk_l, KATZ_MAX_K);
     KALLOC(b.topk_u, KATZ_MAX_K);
     KALLOC(b.trace, h->opts.r_max + 2);
-    KALLOC(b.ctrl, 1);
+    KALLOC(b.sel.key, SELECT_CAP);
+    KALLOC(b.sel.id, SELECT_CAP);
+    KALLOC(b.sel.src, SELECT_CAP);
+    char* ctrl = nullptr;
+    KALLOC(ctrl, CTRL_SPAN);
 #undef KALLOC
+    b.ctrl = (Ctrl*)ctrl;
+    b.sel.state = (SelectState*)(ctrl + CTRL_SPAN - 256);
+    if ((e = cudaMemsetAsync(ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess) {
+        free_iter(h);
+        return cuda_fail(h, e, "memset ctrl");
+    }
     b.cand_cap = n;
     h->walk_slots = slots;
     h->walk_esz = esz;
@@ -170,17 +182,15 @@ katz_status ensure_iter_buffers(katz_handle* h) {
     return KATZ_OK;
 }
 
-// One iteration of Algorithm 1 (five kernels, no host synchronisation).
+// One iteration of Algorithm 1 (four kernels, five with hub rows; no host synchronisation).
 // ev_pair: optional events recorded around the SpMV launch.
 cudaError_t launch_iteration(katz_handle* h, cudaEvent_t* ev_pair = nullptr) {
     cudaError_t e;
     if (ev_pair && (e = cudaEventRecord(ev_pair[0], h->stream)) != cudaSuccess) return e;
     if ((e = launch_spmv(h->g, h->b, h->p, h->fp32, h->stream)) != cudaSuccess) return e;
     if (ev_pair && (e = cudaEventRecord(ev_pair[1], h->stream)) != cudaSuccess) return e;
-    if ((e = launch_select(h->g, h->b, h->p, h->b.cand_l, h->b.cand_u, h->b.cand_id, h->fp32, h->stream)) != cudaSuccess)
-        return e;
-    if ((e = launch_count(h->g, h->b, h->p, h->fp32, h->stream)) != cudaSuccess) return e;
-    return launch_finalize(h->b, h->p, h->stream);
+    if ((e = launch_select(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
+    return launch_count(h->g, h->b, h->p, h->stream);
 }
 
 // The first iteration of a ranking: level 1 is the degree vector (s_0 = 1,
@@ -190,10 +200,8 @@ cudaError_t launch_first_iteration(katz_handle* h, cudaEvent_t* ev_pair = nullpt
     if (ev_pair && (e = cudaEventRecord(ev_pair[0], h->stream)) != cudaSuccess) return e;
     if ((e = launch_degree_level(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
     if (ev_pair && (e = cudaEventRecord(ev_pair[1], h->stream)) != cudaSuccess) return e;
-    if ((e = launch_select(h->g, h->b, h->p, h->b.cand_l, h->b.cand_u, h->b.cand_id, h->fp32, h->stream)) != cudaSuccess)
-        return e;
-    if ((e = launch_count(h->g, h->b, h->p, h->fp32, h->stream)) != cudaSuccess) return e;
-    return launch_finalize(h->b, h->p, h->stream);
+    if ((e = launch_select(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
+    return launch_count(h->g, h->b, h->p, h->stream);
 }
 
 bool same_params(const IterParams& a, const IterParams& b) { return std::memcmp(&a, &b, sizeof(a)) == 0; }
@@ -206,7 +214,7 @@ void drop_graph(katz_handle* h) {
 }
 
 // Capture one iteration as the body of a conditional while node; the
-// finalize kernel clears the condition once converged() holds or r_max is hit.
+// count kernel clears the condition once converged() holds or r_max is hit.
 katz_status ensure_graph(katz_handle* h) {
     if (h->graph_exec && same_params(h->graph_params, h->p) && h->graph_fp32 == h->fp32) return KATZ_OK;
     drop_graph(h);
@@ -910,7 +918,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->launches = h->classes_exact ? 3 : 4;  // init_walk, cert_init, theta_0 (one or two kernels)
     cudaError_t e;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
-    if ((e = cudaMemsetAsync(h->b.ctrl, 0, sizeof(Ctrl), h->stream)) != cudaSuccess) return cuda_fail(h, e, "memset ctrl");
+    if ((e = cudaMemsetAsync(h->b.ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess) return cuda_fail(h, e, "memset ctrl");
     if ((e = launch_init_walk(h->g, h->b, p, h->fp32, h->stream)) != cudaSuccess) return cuda_fail(h, e, "init");
     if ((e = launch_cert_init(h->b, p, h->stream)) != cudaSuccess) return cuda_fail(h, e, "init levels");
     const bool prof = h->opts.profile != 0;
@@ -932,7 +940,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     if (prof && (st = ensure_prof_events(h)) != KATZ_OK) return st;
     if ((e = launch_first_iteration(h, prof ? &h->sp_ev[0] : nullptr)) != cudaSuccess)
         return cuda_fail(h, e, "first iteration");
-    h->launches += 4;  // degree level, select, count, finalize
+    h->launches += 4;  // degree level, select (two), count
     st = run_loop(h, 1);
     if (st != KATZ_OK) return st;
     if ((e = cudaEventRecord(h->ev1, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
@@ -1032,7 +1040,7 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     h->launches = 0;
     const int64_t spmv_kernels = h->g.layout.row_warp > 0 ? 2 : 1;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
-    if ((e = cudaMemsetAsync(h->b.ctrl, 0, sizeof(Ctrl), h->stream)) != cudaSuccess ||
+    if ((e = cudaMemsetAsync(h->b.ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess ||
         (e = launch_init_walk(h->g, h->b, p, false, h->stream)) != cudaSuccess ||
         (e = launch_cert_init(h->b, p, h->stream)) != cudaSuccess ||
         (e = launch_crit_init(h->b, h->stream)) != cudaSuccess)
@@ -1559,11 +1567,10 @@ static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_l
         }
     }
     // ---- bounds, reactivation, converged() at level r, then more iterations ------
-    h->launches += 5;  // theta_lb, reactivate, select, count, finalize
+    h->launches += 5;  // theta_lb, reactivate, select (two), count
     if ((e = dyn_reactivate(g, h->b, h->p, r, h->stream)) != cudaSuccess ||
-        (e = launch_select(g, h->b, h->p, h->b.cand_l, h->b.cand_u, h->b.cand_id, h->fp32, h->stream)) != cudaSuccess ||
-        (e = launch_count(g, h->b, h->p, h->fp32, h->stream)) != cudaSuccess ||
-        (e = launch_finalize(h->b, h->p, h->stream)) != cudaSuccess)
+        (e = launch_select(g, h->b, h->p, h->stream)) != cudaSuccess ||
+        (e = launch_count(g, h->b, h->p, h->stream)) != cudaSuccess)
         return cuda_fail(h, e, "re-check");
     if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)

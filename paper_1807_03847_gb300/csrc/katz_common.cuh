@@ -26,6 +26,7 @@ constexpr int NUM_CLASSES = 34;   // degree classes: 0, then ceil(log2 deg) + 1
 constexpr int CHUNK_ARCS = 2048;  // arcs per warp for rows of degree > 2048
 constexpr int SELECT_CAP = KATZ_MAX_K;
 constexpr int SELECT_THREADS = 1024;
+constexpr int SELECT_DIRECT = 1024;  // candidates ranked without filtering them first
 
 constexpr int32_t STOP_SORT = 2;  // Ctrl::stop while a level waits for its sort
 
@@ -68,6 +69,8 @@ struct Ctrl {
     int32_t list_cur;
     unsigned long long n_list, n_list_next;
 };
+
+constexpr size_t CTRL_SPAN = (sizeof(Ctrl) + 255) / 256 * 256 + 256;
 
 // Per-call constants.
 struct IterParams {
@@ -170,6 +173,26 @@ struct DeviceGraph {
     SpmvLayout layout{};
 };
 
+// The filtered candidates of the select (katz_kernels.cu): SELECT_CAP entries.
+struct SelectState {
+    unsigned int n;       // entries; back to 0 at the end of a level
+    unsigned int ticket;  // of last_block: 0 between kernels
+};
+
+struct SelectBuffers {
+    unsigned long long* key = nullptr;  // bit pattern of l
+    int32_t* id = nullptr;              // original id
+    int32_t* src = nullptr;             // index into the candidate arrays
+    SelectState* state = nullptr;       // zeroed with the control block
+    __device__ __forceinline__ void put(unsigned int pos, double l, int32_t i, int32_t s) const {
+        if (pos < (unsigned int)SELECT_CAP) {
+            key[pos] = (unsigned long long)__double_as_longlong(l);
+            id[pos] = i;
+            src[pos] = s;
+        }
+    }
+};
+
 struct IterBuffers {
     void* walk = nullptr;     // double* or float*
     double* c = nullptr;       // c64: Katz partial sum over the FP64 levels
@@ -184,11 +207,12 @@ struct IterBuffers {
     double* cand_u = nullptr;
     int32_t* cand_id = nullptr;
     int64_t cand_cap = 0;
+    SelectBuffers sel;
     int32_t* topk_id = nullptr;
     double* topk_l = nullptr;
     double* topk_u = nullptr;
     int64_t* trace = nullptr; // |M| per iteration
-    Ctrl* ctrl = nullptr;
+    Ctrl* ctrl = nullptr;     // followed by the select's state (CTRL_SPAN bytes in all)
     unsigned long long cond_handle = 0;  // cudaGraphConditionalHandle (0: none)
     int32_t use_cond = 0;
 };
@@ -266,7 +290,6 @@ cudaError_t dyn_reactivate(const DeviceGraph& g, const IterBuffers& b, const Ite
 cudaError_t dyn_mode_degree_max(const DeviceGraph& g, const DynBuffers& d, int64_t m, const int64_t* rp_new,
                                 cudaStream_t st);
 
-cudaError_t prepare_kernels();  // one-time function attributes (outside any capture)
 SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t row_thread, int64_t chunks);
 // create-time relabelling (katz_relabel.cu)
 int relabel_blocks(int64_t n);
@@ -331,11 +354,8 @@ cudaError_t launch_pair_split(const DeviceGraph& g, const IterBuffers& b, const 
 cudaError_t launch_rows_store(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, const int32_t* rows,
                               const unsigned long long* nrows_dev, int64_t nrows_max, const uint32_t* vbits,
                               int level, cudaStream_t st);
-cudaError_t launch_select(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, const double* cl,
-                          const double* cu, const int32_t* cid, bool fp32, cudaStream_t st);
-cudaError_t launch_count(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
-                         cudaStream_t st);
-cudaError_t launch_finalize(const IterBuffers& b, const IterParams& p, cudaStream_t st);
+cudaError_t launch_select(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
+cudaError_t launch_count(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
 // outputs in original vertex order
 cudaError_t launch_bounds_out(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int level, bool fp32,
                               double* lower, double* upper, double* err, cudaStream_t st);

@@ -2,16 +2,19 @@
 //
 // One iteration r (all on one stream, no host round trip):
 //   spmv         (katz_spmv.cu) s_r, c_r, bounds, candidates
-//   select_topk  theta_r = k-th largest l_r over M (ties by id): one CTA sorts
-//                the candidates in shared memory; replaces partialSort.
+//   select       theta_r = k-th largest l_r over M (ties by id) and the sorted
+//                top-k: the candidates narrowed, then each one's place
+//                counted; replaces partialSort.
 //   count        deactivates nodes of M outside the top-k with
-//                u_r - eps < theta_r and counts those that stay.
-//   finalize     converged(): |M| > k -> false, else adjacent-pair check of
-//                the sorted top-k; sets the loop condition.
+//                u_r - eps < theta_r and counts those that stay; its last
+//                block evaluates converged() (|M| > k -> false, else the
+//                adjacent pairs of the sorted top-k) and sets the loop
+//                condition.
 #include <cooperative_groups.h>
 #include <stdint.h>
 
 #include "katz_common.cuh"
+#include "katz_grid.cuh"
 
 namespace katz {
 
@@ -199,114 +202,18 @@ kth_degree_class_kernel(const Off* __restrict__ rowptr, int64_t a, int64_t b, in
 }
 
 // ---------------------------------------------------------------------------
-// select: sort the candidates by (l desc, id asc) in shared memory; the k-th
-// entry is theta_r and the first k entries are the current top-k.
+// select: theta_r = the k-th largest candidate in the order (l desc, original
+// id asc), and the first k in that order, in two kernels.
+//
+// select_filter narrows the candidates: the previous top-k nodes are still
+// active and each has l_r >= tau := min of their l_r, so the top-k of M lies
+// in {l_r >= tau}, far fewer than {l_r >= theta_{r-1}}.  select_rank gives
+// every candidate left its place by counting the candidates before it.
+// One block that gathered and sorted the list (55 steps of a bitonic network
+// behind ~60 barriers) took 15-19 us per level whatever the graph, half of an
+// iteration on small ones; the two kernels take 6.4 us at 16 K nodes
+// (rank-er16k: 939 -> 598 us together with the count closing its level).
 // ---------------------------------------------------------------------------
-struct SelEntry {
-    unsigned long long key;  // bit pattern of l (monotone for l >= 0)
-    int32_t id;
-    int32_t src;             // index into the candidate arrays
-};
-
-__device__ __forceinline__ bool sel_before(const SelEntry& a, const SelEntry& b) {
-    return a.key > b.key || (a.key == b.key && a.id < b.id);
-}
-
-// A bitonic sort of E * SELECT_THREADS entries by sel_before, entry
-// e = j * SELECT_THREADS + tid held in register j of thread tid.  A compare
-// at distance d pairs e with e ^ d: for d < 32 the partner is in the same
-// warp (shuffles), for d >= SELECT_THREADS in the same thread, and only the
-// distances in between go through shared memory (one barrier on each side).
-// The first cnt entries of sel are sorted (the rest padding that sorts
-// last); the first kk go out as the top-k and entry kk-1 gives theta.
-__device__ __forceinline__ SelEntry shfl_entry(const SelEntry& a, int d) {
-    SelEntry b;
-    b.key = __shfl_xor_sync(FULL, a.key, d);
-    b.id = __shfl_xor_sync(FULL, a.id, d);
-    b.src = __shfl_xor_sync(FULL, a.src, d);
-    return b;
-}
-
-// entry e holding `own` meets its partner's `other` in a network block of
-// `size` (ascending when e & size == 0): it keeps the earlier of the two if
-// it is the lower position of an ascending pair or the upper of a
-// descending one, else the later.  Only padding entries compare equal, and
-// those are identical.
-__device__ __forceinline__ SelEntry pick(const SelEntry& own, const SelEntry& other, int e, int d, int size) {
-    const bool lower = (e & d) == 0, up = (e & size) == 0;
-    const bool own_first = sel_before(own, other);
-    return (lower == up) == own_first ? own : other;
-}
-
-// the compares at distance DJ * SELECT_THREADS, inside each thread
-template <int E, int DJ>
-__device__ __forceinline__ void step_in_thread(SelEntry (&x)[E], int size, int tid) {
-    if constexpr (DJ < E) {
-#pragma unroll
-        for (int j = 0; j < E; ++j) {
-            if (j & DJ) continue;
-            const int e = j * SELECT_THREADS + tid;
-            const bool up = (e & size) == 0;
-            const SelEntry a = x[j], b = x[j | DJ];
-            const bool swap = up ? sel_before(b, a) : sel_before(a, b);
-            x[j] = swap ? b : a;
-            x[j | DJ] = swap ? a : b;
-        }
-    }
-}
-
-template <int E>
-__device__ void sort_and_emit(SelEntry* sel, unsigned int cnt, int kk, const double* __restrict__ cu,
-                              int32_t* topk_id, double* topk_l, double* topk_u, Ctrl* ctrl) {
-    constexpr int P = E * SELECT_THREADS;
-    const int tid = threadIdx.x;
-    SelEntry x[E];
-#pragma unroll
-    for (int j = 0; j < E; ++j) {
-        const int e = j * SELECT_THREADS + tid;
-        x[j] = e < (int)cnt ? sel[e] : SelEntry{0ULL, 0x7fffffff, -1};
-    }
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int d = size >> 1; d > 0; d >>= 1) {
-            if (d >= SELECT_THREADS) {
-                const int dj = d / SELECT_THREADS;  // 1, 2 or 4: register indices stay compile-time
-                if (dj == 1) step_in_thread<E, 1>(x, size, tid);
-                else if (dj == 2) step_in_thread<E, 2>(x, size, tid);
-                else step_in_thread<E, 4>(x, size, tid);
-            } else if (d >= 32) {
-                __syncthreads();  // earlier readers of sel are done
-#pragma unroll
-                for (int j = 0; j < E; ++j) sel[j * SELECT_THREADS + tid] = x[j];
-                __syncthreads();
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const int e = j * SELECT_THREADS + tid;
-                    x[j] = pick(x[j], sel[e ^ d], e, d, size);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const int e = j * SELECT_THREADS + tid;
-                    x[j] = pick(x[j], shfl_entry(x[j], d), e, d, size);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < E; ++j) {
-        const int e = j * SELECT_THREADS + tid;
-        if (e < kk) {
-            topk_id[e] = x[j].id;
-            topk_l[e] = __longlong_as_double((long long)x[j].key);
-            topk_u[e] = cu[x[j].src];
-        }
-        if (e == kk - 1) {
-            ctrl->theta = __longlong_as_double((long long)x[j].key);
-            ctrl->theta_id = x[j].id;
-        }
-    }
-}
-
 // The candidate order as one 96-bit key: the bits of l (monotone for
 // l >= 0), then the complemented id, so that descending keys are
 // (l desc, id asc).
@@ -317,13 +224,14 @@ __device__ __forceinline__ u128 cand_key(double l, int32_t id) {
 }
 
 // The min(k, |C|) largest keys of C = {candidates with l >= tau} gathered
-// into sel, for a C larger than the shared-memory sort holds: a radix select
-// of the k-th key inside this CTA (8-bit digits, most significant first,
+// into f, for a C larger than the filtered list holds: a radix select
+// of the k-th key inside this block (8-bit digits, most significant first,
 // with a 256-bin shared histogram per digit; the select ends at the first
 // digit whose bucket holds exactly the keys still missing), then one pass
 // that gathers every key at or above it.  Returns the number gathered.
-__device__ unsigned int select_large(const double* __restrict__ cl, const int32_t* __restrict__ cid,
-                                     unsigned long long nc, double tau, long long k, SelEntry* sel) {
+__device__ __noinline__ unsigned int select_large(const double* __restrict__ cl, const int32_t* __restrict__ cid,
+                                                  unsigned long long nc, double tau, long long k,
+                                                  const SelectBuffers& f) {
     __shared__ unsigned int hist[256];
     __shared__ unsigned long long s_pre_hi, s_krem;  // selected digits: key bits 95..32 ...
     __shared__ unsigned int s_pre_lo, s_cnt;         // ... and 31..0
@@ -392,258 +300,92 @@ __device__ unsigned int select_large(const double* __restrict__ cl, const int32_
         if (take) {
             const unsigned int pos = wpos + __popc(m & ((1u << lane) - 1u));
             if (pos < (unsigned int)SELECT_CAP)
-                sel[pos] = SelEntry{(unsigned long long)__double_as_longlong(l), cid[q], (int32_t)q};
+                f.put(pos, l, cid[q], (int32_t)q);
         }
     }
     __syncthreads();
     return min(s_cnt, (unsigned int)SELECT_CAP);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(SELECT_THREADS)
-select_kernel(const double* __restrict__ cl, const double* __restrict__ cu, const int32_t* __restrict__ cid,
-              const T* walk, const double* c, const double* c32, const double* lb, const int32_t* __restrict__ inv,
-              int32_t* topk_id, double* topk_l, double* topk_u, Ctrl* ctrl, IterParams p) {
-    extern __shared__ SelEntry sel[];
-    __shared__ unsigned int s_cnt;
-    __shared__ double s_tau;
-    __shared__ int s_big;
-    if (ctrl->stop) return;
-    const int tid = threadIdx.x;
-    const unsigned long long nc = ctrl->n_cand;
-    const int r_cur = ctrl->r + 1;
-    if (tid == 0) {
-        s_cnt = 0;
-        s_tau = -1.0;
-        s_big = 0;
-    }
-    __syncthreads();
-    {
-        // Narrow the candidates: the previous top-k nodes are still active and
-        // each has l_r >= tau := min of their l_r, so the top-k of M lies in
-        // {l_r >= tau} (a far smaller sort than all of {l_r >= theta_{r-1}}).
-        const int kprev = ctrl->k_eff;
-        if (r_cur <= 1 || kprev < (int)p.k) {
-            if (tid == 0 && nc > (unsigned long long)SELECT_CAP) s_big = 1;
-        } else {
-            const BState bs = bstate(ctrl, p);
-            const int f32_from = ctrl->f32_from;
-            double m = 1.0 / 0.0;
-            for (int q = tid; q < kprev; q += SELECT_THREADS) {
-                const int32_t v = inv[topk_id[q]];
-                double l, u;
-                if (p.cert) l = lb[v];
-                else node_bounds(c[v], 0.0, walk_value(walk, p, f32_from, r_cur, v), p, bs, l, u);
-                m = fmin(m, l);
-            }
-            for (int off = 16; off; off >>= 1) m = fmin(m, __shfl_xor_sync(FULL, m, off));
-            __shared__ double wmin[SELECT_THREADS / 32];
-            if ((tid & 31) == 0) wmin[tid >> 5] = m;
-            __syncthreads();
-            if (tid == 0) {
-                double mm = wmin[0];
-                for (int w = 1; w < SELECT_THREADS / 32; ++w) mm = fmin(mm, wmin[w]);
-                s_tau = mm;
-            }
-        }
-        __syncthreads();
-    }
-    const double tau = s_tau;
-    unsigned int cnt = 0;
-    if (!s_big) {
-        // the candidates with l >= tau, one shared-memory atomic per warp
-        const int lane = tid & 31;
-        for (unsigned long long base = 0; base < nc; base += SELECT_THREADS) {
-            const unsigned long long q = base + tid;
-            const double l = q < nc ? cl[q] : -1.0;
-            const bool take = q < nc && l >= tau;
-            const unsigned m = __ballot_sync(FULL, take);
-            unsigned int wpos = 0;
-            if (lane == 0 && m) wpos = atomicAdd(&s_cnt, (unsigned int)__popc(m));
-            wpos = __shfl_sync(FULL, wpos, 0);
-            if (take) {
-                const unsigned int pos = wpos + __popc(m & ((1u << lane) - 1u));
-                if (pos < (unsigned int)SELECT_CAP)
-                    sel[pos] = SelEntry{(unsigned long long)__double_as_longlong(l), cid[q], (int32_t)q};
-            }
-        }
-        __syncthreads();
-        cnt = s_cnt;
-    }
-    // more candidates than the sort holds: select the top k of them first,
-    // here on the device (the loop never waits for the host)
-    if (s_big || cnt > (unsigned int)SELECT_CAP) cnt = select_large(cl, cid, nc, tau, (long long)p.k, sel);
-    const int kk = (int)min((long long)p.k, (long long)cnt);
-    if (cnt <= (unsigned int)SELECT_THREADS) sort_and_emit<1>(sel, cnt, kk, cu, topk_id, topk_l, topk_u, ctrl);
-    else if (cnt <= 2u * SELECT_THREADS) sort_and_emit<2>(sel, cnt, kk, cu, topk_id, topk_l, topk_u, ctrl);
-    else if (cnt <= 4u * SELECT_THREADS) sort_and_emit<4>(sel, cnt, kk, cu, topk_id, topk_l, topk_u, ctrl);
-    else sort_and_emit<8>(sel, cnt, kk, cu, topk_id, topk_l, topk_u, ctrl);
-    if (tid == 0) {
-        ctrl->k_eff = kk;
-        ctrl->tau = tau;
-    }
+// one filtered candidate (f.put keeps what fits)
+__device__ __forceinline__ void filter_append(bool take, double l, int32_t id, int32_t src, SelectBuffers& f) {
+    const unsigned m = __ballot_sync(FULL, take);
+    if (!m) return;
+    const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
+    unsigned int base = 0;
+    if (lane == first) base = atomicAdd(&f.state->n, (unsigned int)__popc(m));
+    base = __shfl_sync(FULL, base, first);
+    if (take) f.put(base + __popc(m & ((1u << lane) - 1u)), l, id, src);
 }
 
-// ---------------------------------------------------------------------------
-// count: deactivate nodes of M outside the top-k with u_r - eps < theta_r and
-// count the ones that remain (converged() returns false if any remain).
-//
-// M is read from a compact list of its nodes: the first count after all
-// nodes became active scans the flags of all of V instead.  Either way the
-// survivors are written, in tiles, to the other list buffer (one atomic per
-// tile for its place), which finalize then makes current.  The order of a
-// list is arbitrary; nothing computed from it depends on the order.
-// ---------------------------------------------------------------------------
-constexpr int COUNT_THREADS = 256;
-constexpr int COUNT_U = 4;  // nodes per thread and tile, their loads issued together
-constexpr int COUNT_TILE = COUNT_THREADS * COUNT_U;
-
-template <typename T>
-__global__ void __launch_bounds__(COUNT_THREADS)
-count_kernel(const T* walk, const double* __restrict__ c, const double* __restrict__ c32,
-             const double* __restrict__ lb, const double* __restrict__ ub, const int32_t* __restrict__ perm,
-             uint8_t* active, int32_t* alist0, int32_t* alist1, Ctrl* ctrl, IterParams p) {
-    __shared__ int s_wcnt[COUNT_THREADS / 32];
-    __shared__ unsigned long long s_base;
+// Up to SELECT_DIRECT candidates go to select_rank as they are (the count is
+// quadratic, but 1024^2 pairs over the chip take less than the filter's three
+// dependent gathers); more are filtered, and if the filtered list outgrows its
+// buffer (many equal bounds, or no previous top-k) the last block selects the
+// k largest.
+__global__ void __launch_bounds__(SELECT_THREADS)
+select_filter_kernel(const double* __restrict__ cl, const int32_t* __restrict__ cid, const double* __restrict__ lb,
+                     const int32_t* __restrict__ inv, const int32_t* __restrict__ topk_id, SelectBuffers f,
+                     const Ctrl* ctrl, IterParams p) {
     if (ctrl->stop) return;
-    const int r_cur = ctrl->r + 1;
-    const int f32_from = ctrl->f32_from;
-    const BState bs = bstate(ctrl, p);
-    const double th = ctrl->theta;
-    const int32_t thid = ctrl->theta_id;
-    const bool full = !ctrl->list_ready;
-    const int cur = ctrl->list_cur;
-    const int32_t* in = cur ? alist1 : alist0;
-    int32_t* out = cur ? alist0 : alist1;
-    const int64_t total = full ? p.n : (int64_t)ctrl->n_list;
+    const unsigned long long nc = ctrl->n_cand;
+    if (nc <= (unsigned long long)SELECT_DIRECT) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    unsigned long long cross = 0, act = 0;
-    double roundw = 0.0;
-    // cert mode: the maxima of s_r and, over nodes with c32 = +0 (all of them
-    // before the switch to FP32 levels), of c64, taken on bit patterns (the
-    // values are non-negative); the tail and rounding widths follow from them
-    // below, because rounding a product with a non-negative factor is monotone
-    long long smax_b = 0, cmax_b = 0;
-    const double d64 = bs.hi64 - bs.lo64, d32 = bs.hi32 - bs.lo32;
-    // l, th >= 0 (sums of non-negative terms): they order like their bit patterns
-    const long long th_bits = __double_as_longlong(th);
-    // the trip count depends on the block only, so the barriers below are uniform
-    for (int64_t t0 = (int64_t)blockIdx.x * COUNT_TILE; t0 < total; t0 += (int64_t)gridDim.x * COUNT_TILE) {
-        bool on[COUNT_U], keep[COUNT_U];
-        int32_t v[COUNT_U];
-#pragma unroll
-        for (int q = 0; q < COUNT_U; ++q) {
-            const int64_t i = t0 + q * COUNT_THREADS + tid;
-            on[q] = i < total;
-            v[q] = on[q] ? (full ? (int32_t)i : in[i]) : 0;
-        }
-        if (full) {
-#pragma unroll
-            for (int q = 0; q < COUNT_U; ++q) on[q] = on[q] && active[v[q]];
-        }
-        double l[COUNT_U], u[COUNT_U];
-        int32_t ov[COUNT_U];
-#pragma unroll
-        for (int q = 0; q < COUNT_U; ++q) {
-            l[q] = on[q] ? lb[v[q]] : 0.0;  // stored by the SpMV epilogue of this level
-            u[q] = on[q] ? ub[v[q]] : 0.0;
-            ov[q] = on[q] ? perm[v[q]] : 0;  // ties are broken by the original id
-        }
-        int mine = 0;
-#pragma unroll
-        for (int q = 0; q < COUNT_U; ++q) {
-            keep[q] = false;
-            if (!on[q]) continue;
-            const long long l_bits = __double_as_longlong(l[q]);
-            const bool top = l_bits > th_bits || (l_bits == th_bits && ov[q] <= thid);
-            if (!top) {
-                if (__dsub_rn(u[q], p.eps) < th) {
-                    active[v[q]] = 0;
-                    continue;
-                }
-                ++cross;
-            }
-            keep[q] = true;
-            ++mine;
-            if (p.cert) {
-                const double sv = walk_value(walk, p, f32_from, r_cur, v[q]);
-                const double c64v = c[v[q]], c32v = c32 ? c32[v[q]] : 0.0;
-                smax_b = max(smax_b, __double_as_longlong(sv));
-                if (__double_as_longlong(c32v) == 0) cmax_b = max(cmax_b, __double_as_longlong(c64v));
-                else roundw = fmax(roundw, __fma_rn(c64v, d64, __dmul_rn(c32v, d32)));
-            }
-        }
-        act += (unsigned long long)mine;
-        // places of the survivors: scan within the warp, then over the warps
-        int incl = mine;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(FULL, incl, off);
-            if (lane >= off) incl += y;
-        }
-        if (lane == 31) s_wcnt[wid] = incl;
+    const int kprev = ctrl->k_eff;
+    // bounds are non-negative: they order like their bit patterns
+    long long tau = -1;
+    if (ctrl->r + 1 > 1 && kprev >= (int)p.k) {
+        __shared__ long long wmin[SELECT_THREADS / 32];
+        long long m = 0x7ff0000000000000ll;
+        for (int q = tid; q < kprev; q += SELECT_THREADS) m = min(m, __double_as_longlong(lb[inv[topk_id[q]]]));
+        for (int off = 16; off; off >>= 1) m = min(m, __shfl_xor_sync(FULL, m, off));
+        if (lane == 0) wmin[wid] = m;
         __syncthreads();
-        if (tid == 0) {
-            int run = 0;
-            for (int w = 0; w < COUNT_THREADS / 32; ++w) {
-                const int x = s_wcnt[w];
-                s_wcnt[w] = run;
-                run += x;
-            }
-            s_base = run ? atomicAdd(&ctrl->n_list_next, (unsigned long long)run) : 0ull;
+        tau = wmin[lane];
+        for (int off = 16; off; off >>= 1) tau = min(tau, __shfl_xor_sync(FULL, tau, off));
+    }
+    if (tau >= 0 || nc <= (unsigned long long)SELECT_CAP) {
+        for (unsigned long long base = (unsigned long long)blockIdx.x * SELECT_THREADS; base < nc;
+             base += (unsigned long long)gridDim.x * SELECT_THREADS) {
+            const unsigned long long q = base + tid;
+            const double l = q < nc ? cl[q] : 0.0;
+            const bool take = q < nc && __double_as_longlong(l) >= tau;
+            filter_append(take, l, take ? cid[q] : 0, (int32_t)q, f);
         }
-        __syncthreads();
-        unsigned long long pos = s_base + (unsigned long long)(s_wcnt[wid] + incl - mine);
-#pragma unroll
-        for (int q = 0; q < COUNT_U; ++q)
-            if (keep[q]) out[pos++] = v[q];
-        __syncthreads();  // s_wcnt and s_base are rewritten by the next tile
+    } else if (blockIdx.x == 0 && tid == 0) {
+        atomicMax(&f.state->n, SELECT_CAP + 1u);  // no tau: all of them, too many
     }
-    double smax = 0.0, tailw = 0.0;
-    if (p.cert) {
-        smax = __longlong_as_double(smax_b);
-        tailw = __dmul_rn(p.ag, smax);  // = the largest of ag s_r over this thread's nodes
-        roundw = fmax(roundw, __dmul_rn(__longlong_as_double(cmax_b), d64));
-    }
-    // block totals first: one atomic per block and counter
-    __shared__ unsigned long long s_cross[32], s_act[32];
-    __shared__ double s_smax[32], s_tailw[32], s_roundw[32];
-    for (int off = 16; off; off >>= 1) {
-        cross += __shfl_xor_sync(FULL, cross, off);
-        act += __shfl_xor_sync(FULL, act, off);
-        smax = fmax(smax, __shfl_xor_sync(FULL, smax, off));
-        tailw = fmax(tailw, __shfl_xor_sync(FULL, tailw, off));
-        roundw = fmax(roundw, __shfl_xor_sync(FULL, roundw, off));
-    }
-    const int nw = blockDim.x >> 5;
-    if (lane == 0) {
-        s_cross[wid] = cross;
-        s_act[wid] = act;
-        s_smax[wid] = smax;
-        s_tailw[wid] = tailw;
-        s_roundw[wid] = roundw;
-    }
-    __syncthreads();
-    if (wid == 0) {
-        cross = lane < nw ? s_cross[lane] : 0ull;
-        act = lane < nw ? s_act[lane] : 0ull;
-        smax = lane < nw ? s_smax[lane] : 0.0;
-        tailw = lane < nw ? s_tailw[lane] : 0.0;
-        roundw = lane < nw ? s_roundw[lane] : 0.0;
-        for (int off = 16; off; off >>= 1) {
-            cross += __shfl_xor_sync(FULL, cross, off);
-            act += __shfl_xor_sync(FULL, act, off);
-            smax = fmax(smax, __shfl_xor_sync(FULL, smax, off));
-            tailw = fmax(tailw, __shfl_xor_sync(FULL, tailw, off));
-            roundw = fmax(roundw, __shfl_xor_sync(FULL, roundw, off));
-        }
-        if (lane == 0) {
-            if (cross) atomicAdd(&ctrl->cnt_cross, cross);
-            if (act) atomicAdd(&ctrl->n_active, act);
-            if (p.cert) {  // non-negative doubles order like their bit patterns
-                atomicMax(&ctrl->smax_bits, (unsigned long long)__double_as_longlong(smax));
-                atomicMax(&ctrl->tailw_bits, (unsigned long long)__double_as_longlong(tailw));
-                atomicMax(&ctrl->roundw_bits, (unsigned long long)__double_as_longlong(roundw));
+    if (!last_block(&f.state->ticket)) return;
+    if (__ldcg(&f.state->n) <= (unsigned int)SELECT_CAP) return;
+    const unsigned int cnt = select_large(cl, cid, nc, __longlong_as_double(tau < 0 ? 0 : tau), (long long)p.k, f);
+    if (tid == 0) f.state->n = cnt;
+}
+
+__global__ void __launch_bounds__(RANK_THREADS)
+select_rank_kernel(const double* __restrict__ cl, const double* __restrict__ cu, const int32_t* __restrict__ cid,
+                   SelectBuffers f, int32_t* topk_id, double* topk_l, double* topk_u, Ctrl* ctrl, IterParams p) {
+    if (ctrl->stop) return;
+    const unsigned long long nc = ctrl->n_cand;
+    const bool direct = nc <= (unsigned long long)SELECT_DIRECT;
+    const int cnt = direct ? (int)nc : (int)f.state->n;
+    const unsigned long long* keys = direct ? (const unsigned long long*)cl : f.key;
+    const int32_t* ids = direct ? cid : f.id;
+    const int kk = (int)min((long long)p.k, (long long)cnt);
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->k_eff = kk;
+    // i0 is the same for every thread of a block
+    for (int i0 = blockIdx.x * RANK_PER_BLOCK; i0 < cnt; i0 += gridDim.x * RANK_PER_BLOCK) {
+        const int i = i0 + threadIdx.x / RANK_LANES;
+        const unsigned long long key = i < cnt ? keys[i] : 0ull;
+        const int32_t id = i < cnt ? ids[i] : 0x7fffffff;
+        const int r = rank_by_count(keys, ids, cnt, key, id);
+        if (i < cnt && r < kk && threadIdx.x % RANK_LANES == 0) {
+            const double l = __longlong_as_double((long long)key);
+            topk_id[r] = id;
+            topk_l[r] = l;
+            topk_u[r] = cu[direct ? i : f.src[i]];
+            if (r == kk - 1) {
+                ctrl->theta = l;
+                ctrl->theta_id = id;
             }
         }
     }
@@ -716,6 +458,258 @@ __device__ double next_abs(const Ctrl* ctrl, const IterParams& p, int lvl, doubl
     return __fma_ru(__dadd_ru(1.0, g), in, half_sub);
 }
 
+// converged() of this level and the control block of the next one, by the
+// last block of the count (its counters are complete then)
+__device__ __noinline__ void finalize_level(const double* __restrict__ topk_l, const double* __restrict__ topk_u,
+                                            int64_t* trace, SelectState* sel, Ctrl* ctrl, const IterParams& p,
+                                            unsigned long long cond, int use_cond) {
+    __shared__ int bad;
+    const int tid = threadIdx.x;
+    if (tid == 0) bad = 0;
+    // every field the first thread needs, loaded before its first store (the
+    // compiler keeps loads behind stores to the same block: one trip to L2 each)
+    const int kk = ctrl->k_eff, r_cur = ctrl->r + 1, list_cur = ctrl->list_cur;
+    const double theta = ctrl->theta;
+    const unsigned long long runs = ctrl->body_runs, crossing = __ldcg(&ctrl->cnt_cross);
+    const unsigned long long n_active = __ldcg(&ctrl->n_active), n_list = __ldcg(&ctrl->n_list_next);
+    __syncthreads();
+    const bool none_cross = crossing == 0;
+    if (none_cross) {
+        for (int q = tid + 1; q < kk; q += blockDim.x)
+            if (__dsub_rn(topk_u[q], p.eps) >= topk_l[q - 1]) bad = 1;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        const int conv = none_cross && !bad;
+        sel->n = 0;
+        ctrl->body_runs = runs + 1;
+        if (r_cur <= p.r_max) trace[r_cur] = (int64_t)n_active;
+        ctrl->r = r_cur;
+        ctrl->converged = conv;
+        ctrl->theta_prev = theta;
+        ctrl->n_cand = 0;
+        ctrl->cnt_cross = 0;
+        ctrl->n_active = 0;
+        // the survivors of this count become the active list
+        ctrl->list_cur = list_cur ^ 1;
+        ctrl->n_list = n_list;
+        ctrl->n_list_next = 0;
+        ctrl->list_ready = 1;
+        int stop = conv || r_cur >= p.r_max;
+        if (p.cert) {
+            const double smax = __longlong_as_double((long long)__ldcg(&ctrl->smax_bits));
+            const double sprev = __longlong_as_double((long long)ctrl->smax_prev_bits);
+            const double tailw = __longlong_as_double((long long)__ldcg(&ctrl->tailw_bits));
+            const double roundw = __longlong_as_double((long long)__ldcg(&ctrl->roundw_bits));
+            // stall: over the active set the rounding widening is wider than the
+            // Theorem-1 tail term, so further iterations cannot separate it
+            if (!conv && r_cur >= ctrl->f32_from && tailw < roundw) {
+                ctrl->stall = 1;
+                stop = 1;
+            }
+            if (!stop) {
+                const int next = r_cur + 1;
+                // switch to FP32 once the terms still to come (predicted from the
+                // decay of max s_r over M) carry a rounding widening below eps/16
+                if (ctrl->f32_from == 0x7fffffff && p.fp32_from == 0 && r_cur >= 2 && sprev > 0.0 &&
+                    smax < 0.5 * sprev) {
+                    const double rho = smax / sprev;
+                    const double tail_est = smax * rho / (1.0 - rho);
+                    const double e32 = ctrl->e_cur + 64.0 * gamma_up((double)(p.depth + 3), 0x1p-24);
+                    if (2.0 * tail_est * e32 <= p.eps / 16.0) ctrl->f32_from = next;
+                }
+                set_level_state(ctrl, p, next, next_error(ctrl, p, next, ctrl->e_cur),
+                                next_abs(ctrl, p, next, ctrl->a_cur));
+            }
+            ctrl->smax_prev_bits = __ldcg(&ctrl->smax_bits);
+            ctrl->smax_bits = 0;
+            ctrl->tailw_bits = 0;
+            ctrl->roundw_bits = 0;
+        }
+        ctrl->stop = stop;
+        if (use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, stop ? 0u : 1u);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// count: deactivate nodes of M outside the top-k with u_r - eps < theta_r and
+// count the ones that remain (converged() returns false if any remain).
+//
+// M is read from a compact list of its nodes: the first count after all
+// nodes became active scans the flags of all of V instead.  Either way the
+// survivors are written, in tiles, to the other list buffer (one atomic per
+// tile for its place), which finalize then makes current.  The order of a
+// list is arbitrary; nothing computed from it depends on the order.
+//
+// The block that finishes last closes the level (finalize_level): as a kernel
+// of its own that took 2.5-3 us per level and a launch.
+// ---------------------------------------------------------------------------
+constexpr int COUNT_THREADS = 256;
+constexpr int COUNT_U = 4;  // nodes per thread and tile, their loads issued together
+constexpr int COUNT_TILE = COUNT_THREADS * COUNT_U;
+
+template <typename T>
+__global__ void __launch_bounds__(COUNT_THREADS)
+count_kernel(const T* walk, const double* __restrict__ c, const double* __restrict__ c32,
+             const double* __restrict__ lb, const double* __restrict__ ub, const int32_t* __restrict__ perm,
+             uint8_t* active, int32_t* alist0, int32_t* alist1, const double* __restrict__ topk_l,
+             const double* __restrict__ topk_u, int64_t* trace, SelectState* sel, unsigned long long cond,
+             int use_cond, Ctrl* ctrl, IterParams p) {
+    __shared__ int s_wcnt[COUNT_THREADS / 32];
+    __shared__ unsigned long long s_base;
+    if (ctrl->stop) {  // the loop is over: leave the device-side while loop too
+        if (blockIdx.x == 0 && threadIdx.x == 0 && use_cond)
+            cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 0);
+        return;
+    }
+    const int r_cur = ctrl->r + 1;
+    const int f32_from = ctrl->f32_from;
+    const BState bs = bstate(ctrl, p);
+    const double th = ctrl->theta;
+    const int32_t thid = ctrl->theta_id;
+    const bool full = !ctrl->list_ready;
+    const int cur = ctrl->list_cur;
+    const int32_t* in = cur ? alist1 : alist0;
+    int32_t* out = cur ? alist0 : alist1;
+    const int64_t total = full ? p.n : (int64_t)ctrl->n_list;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    unsigned int cross = 0, act = 0;  // of this thread: below 2^32 / blockDim
+    double roundw = 0.0;
+    // cert mode: the maxima of s_r and, over nodes with c32 = +0 (all of them
+    // before the switch to FP32 levels), of c64, taken on bit patterns (the
+    // values are non-negative); the tail and rounding widths follow from them
+    // below, because rounding a product with a non-negative factor is monotone
+    long long smax_b = 0, cmax_b = 0;
+    const double d64 = bs.hi64 - bs.lo64, d32 = bs.hi32 - bs.lo32;
+    // l, th >= 0 (sums of non-negative terms): they order like their bit patterns
+    const long long th_bits = __double_as_longlong(th);
+    // the trip count depends on the block only, so the barriers below are uniform
+    for (int64_t t0 = (int64_t)blockIdx.x * COUNT_TILE; t0 < total; t0 += (int64_t)gridDim.x * COUNT_TILE) {
+        bool on[COUNT_U], keep[COUNT_U];
+        int32_t v[COUNT_U];
+#pragma unroll
+        for (int q = 0; q < COUNT_U; ++q) {
+            const int64_t i = t0 + q * COUNT_THREADS + tid;
+            on[q] = i < total;
+            v[q] = on[q] ? (full ? (int32_t)i : in[i]) : 0;
+        }
+        if (full) {
+#pragma unroll
+            for (int q = 0; q < COUNT_U; ++q) on[q] = on[q] && active[v[q]];
+        }
+        double l[COUNT_U], u[COUNT_U];
+        int32_t ov[COUNT_U];
+#pragma unroll
+        for (int q = 0; q < COUNT_U; ++q) {
+            l[q] = on[q] ? lb[v[q]] : 0.0;  // stored by the SpMV epilogue of this level
+            u[q] = on[q] ? ub[v[q]] : 0.0;
+            ov[q] = on[q] ? perm[v[q]] : 0;  // ties are broken by the original id
+        }
+        int mine = 0;
+#pragma unroll
+        for (int q = 0; q < COUNT_U; ++q) {
+            keep[q] = false;
+            if (!on[q]) continue;
+            const long long l_bits = __double_as_longlong(l[q]);
+            const bool top = l_bits > th_bits || (l_bits == th_bits && ov[q] <= thid);
+            if (!top) {
+                // u < theta settles it (eps > 0) without the narrow FP64 pipe
+                if (__double_as_longlong(u[q]) < th_bits || __dsub_rn(u[q], p.eps) < th) {
+                    active[v[q]] = 0;
+                    continue;
+                }
+                ++cross;
+            }
+            keep[q] = true;
+            ++mine;
+            if (p.cert) {
+                const double sv = walk_value(walk, p, f32_from, r_cur, v[q]);
+                const double c64v = c[v[q]], c32v = c32 ? c32[v[q]] : 0.0;
+                smax_b = max(smax_b, __double_as_longlong(sv));
+                if (__double_as_longlong(c32v) == 0) cmax_b = max(cmax_b, __double_as_longlong(c64v));
+                else roundw = fmax(roundw, __fma_rn(c64v, d64, __dmul_rn(c32v, d32)));
+            }
+        }
+        act += (unsigned int)mine;
+        // places of the survivors: scan within the warp, then over the warps
+        int incl = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(FULL, incl, off);
+            if (lane >= off) incl += y;
+        }
+        if (lane == 31) s_wcnt[wid] = incl;
+        __syncthreads();
+        if (wid == 0) {
+            const int x = lane < COUNT_THREADS / 32 ? s_wcnt[lane] : 0;
+            int upto = x;
+#pragma unroll
+            for (int off = 1; off < COUNT_THREADS / 32; off <<= 1) {
+                const int y = __shfl_up_sync(FULL, upto, off);
+                if (lane >= off) upto += y;
+            }
+            if (lane < COUNT_THREADS / 32) s_wcnt[lane] = upto - x;
+            if (lane == COUNT_THREADS / 32 - 1)
+                s_base = upto ? atomicAdd(&ctrl->n_list_next, (unsigned long long)upto) : 0ull;
+        }
+        __syncthreads();
+        unsigned long long pos = s_base + (unsigned long long)(s_wcnt[wid] + incl - mine);
+#pragma unroll
+        for (int q = 0; q < COUNT_U; ++q)
+            if (keep[q]) out[pos++] = v[q];
+        __syncthreads();  // s_wcnt and s_base are rewritten by the next tile
+    }
+    // block totals first: one atomic per block and counter
+    __shared__ unsigned int s_cross[32], s_act[32];
+    __shared__ double s_smax[32], s_tailw[32], s_roundw[32];
+    const int nw = blockDim.x >> 5;
+    cross = __reduce_add_sync(FULL, cross);
+    act = __reduce_add_sync(FULL, act);
+    double smax = 0.0, tailw = 0.0;
+    if (p.cert) {
+        smax = __longlong_as_double(smax_b);
+        tailw = __dmul_rn(p.ag, smax);  // = the largest of ag s_r over this thread's nodes
+        roundw = fmax(roundw, __dmul_rn(__longlong_as_double(cmax_b), d64));
+        for (int off = 16; off; off >>= 1) {
+            smax = fmax(smax, __shfl_xor_sync(FULL, smax, off));
+            tailw = fmax(tailw, __shfl_xor_sync(FULL, tailw, off));
+            roundw = fmax(roundw, __shfl_xor_sync(FULL, roundw, off));
+        }
+    }
+    if (lane == 0) {
+        s_cross[wid] = cross;
+        s_act[wid] = act;
+        s_smax[wid] = smax;
+        s_tailw[wid] = tailw;
+        s_roundw[wid] = roundw;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        cross = __reduce_add_sync(FULL, lane < nw ? s_cross[lane] : 0u);
+        act = __reduce_add_sync(FULL, lane < nw ? s_act[lane] : 0u);
+        if (lane == 0) {
+            if (cross) atomicAdd(&ctrl->cnt_cross, (unsigned long long)cross);
+            if (act) atomicAdd(&ctrl->n_active, (unsigned long long)act);
+        }
+        if (p.cert) {  // non-negative doubles order like their bit patterns
+            smax = lane < nw ? s_smax[lane] : 0.0;
+            tailw = lane < nw ? s_tailw[lane] : 0.0;
+            roundw = lane < nw ? s_roundw[lane] : 0.0;
+            for (int off = 16; off; off >>= 1) {
+                smax = fmax(smax, __shfl_xor_sync(FULL, smax, off));
+                tailw = fmax(tailw, __shfl_xor_sync(FULL, tailw, off));
+                roundw = fmax(roundw, __shfl_xor_sync(FULL, roundw, off));
+            }
+            if (lane == 0) {
+                atomicMax(&ctrl->smax_bits, (unsigned long long)__double_as_longlong(smax));
+                atomicMax(&ctrl->tailw_bits, (unsigned long long)__double_as_longlong(tailw));
+                atomicMax(&ctrl->roundw_bits, (unsigned long long)__double_as_longlong(roundw));
+            }
+        }
+    }
+    if (last_block(&sel->ticket)) finalize_level(topk_l, topk_u, trace, sel, ctrl, p, cond, use_cond);
+}
+
 __global__ void cert_init_kernel(Ctrl* ctrl, IterParams p) {
     ctrl->f32_from = (p.cert && p.fp32_from >= 2) ? p.fp32_from : 0x7fffffff;
     ctrl->e64 = 0.0;
@@ -738,75 +732,6 @@ __global__ void cert_replay_kernel(Ctrl* ctrl, IterParams p, int r) {
         e = next_error(ctrl, p, lvl, e);
         a = next_abs(ctrl, p, lvl, a);
         set_level_state(ctrl, p, lvl, e, a);
-    }
-}
-
-__global__ void finalize_kernel(const double* __restrict__ topk_l, const double* __restrict__ topk_u,
-                                int64_t* trace, Ctrl* ctrl, IterParams p, unsigned long long cond, int use_cond) {
-    __shared__ int bad;
-    const int tid = threadIdx.x;
-    if (tid == 0) bad = 0;
-    __syncthreads();
-    if (ctrl->stop) {  // the loop was already over: leave the device-side while loop too
-        if (tid == 0 && use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 0);
-        return;
-    }
-    if (tid == 0) ctrl->body_runs += 1;
-    const int kk = ctrl->k_eff;
-    const bool none_cross = ctrl->cnt_cross == 0;
-    if (none_cross) {
-        for (int q = tid + 1; q < kk; q += blockDim.x)
-            if (__dsub_rn(topk_u[q], p.eps) >= topk_l[q - 1]) bad = 1;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const int conv = none_cross && !bad;
-        const int r_cur = ctrl->r + 1;
-        if (r_cur <= p.r_max) trace[r_cur] = (int64_t)ctrl->n_active;
-        ctrl->r = r_cur;
-        ctrl->converged = conv;
-        ctrl->theta_prev = ctrl->theta;
-        ctrl->n_cand = 0;
-        ctrl->cnt_cross = 0;
-        ctrl->n_active = 0;
-        // the survivors of this count become the active list
-        ctrl->list_cur ^= 1;
-        ctrl->n_list = ctrl->n_list_next;
-        ctrl->n_list_next = 0;
-        ctrl->list_ready = 1;
-        int stop = conv || r_cur >= p.r_max;
-        if (p.cert) {
-            const double smax = __longlong_as_double((long long)ctrl->smax_bits);
-            const double sprev = __longlong_as_double((long long)ctrl->smax_prev_bits);
-            const double tailw = __longlong_as_double((long long)ctrl->tailw_bits);
-            const double roundw = __longlong_as_double((long long)ctrl->roundw_bits);
-            // stall: over the active set the rounding widening is wider than the
-            // Theorem-1 tail term, so further iterations cannot separate it
-            if (!conv && r_cur >= ctrl->f32_from && tailw < roundw) {
-                ctrl->stall = 1;
-                stop = 1;
-            }
-            if (!stop) {
-                const int next = r_cur + 1;
-                // switch to FP32 once the terms still to come (predicted from the
-                // decay of max s_r over M) carry a rounding widening below eps/16
-                if (ctrl->f32_from == 0x7fffffff && p.fp32_from == 0 && r_cur >= 2 && sprev > 0.0 &&
-                    smax < 0.5 * sprev) {
-                    const double rho = smax / sprev;
-                    const double tail_est = smax * rho / (1.0 - rho);
-                    const double e32 = ctrl->e_cur + 64.0 * gamma_up((double)(p.depth + 3), 0x1p-24);
-                    if (2.0 * tail_est * e32 <= p.eps / 16.0) ctrl->f32_from = next;
-                }
-                set_level_state(ctrl, p, next, next_error(ctrl, p, next, ctrl->e_cur),
-                                next_abs(ctrl, p, next, ctrl->a_cur));
-            }
-            ctrl->smax_prev_bits = ctrl->smax_bits;
-            ctrl->smax_bits = 0;
-            ctrl->tailw_bits = 0;
-            ctrl->roundw_bits = 0;
-        }
-        ctrl->stop = stop;
-        if (use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, stop ? 0u : 1u);
     }
 }
 
@@ -927,32 +852,21 @@ cudaError_t launch_theta0_class(const DeviceGraph& g, const IterBuffers& b, cons
     return cudaGetLastError();
 }
 
-cudaError_t prepare_kernels() {
-    const int smem = SELECT_CAP * (int)sizeof(SelEntry);
-    return cudaFuncSetAttribute(select_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
-
-cudaError_t launch_select(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, const double* cl,
-                          const double* cu, const int32_t* cid, bool fp32, cudaStream_t st) {
-    (void)fp32;
-    const int smem = SELECT_CAP * (int)sizeof(SelEntry);
-    select_kernel<double><<<1, SELECT_THREADS, smem, st>>>(cl, cu, cid, (const double*)b.walk, b.c, b.c32, b.lb, g.inv,
-                                                           b.topk_id, b.topk_l, b.topk_u, b.ctrl, p);
+cudaError_t launch_select(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
+    select_filter_kernel<<<grid_for(p.n, SELECT_THREADS, 152), SELECT_THREADS, 0, st>>>(
+        b.cand_l, b.cand_id, b.lb, g.inv, b.topk_id, b.sel, b.ctrl, p);
+    select_rank_kernel<<<grid_for(p.n, RANK_PER_BLOCK, SELECT_CAP / RANK_PER_BLOCK), RANK_THREADS, 0, st>>>(
+        b.cand_l, b.cand_u, b.cand_id, b.sel, b.topk_id, b.topk_l, b.topk_u, b.ctrl, p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_count(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
-                         cudaStream_t st) {
-    (void)fp32;
+// deactivation count and converged(): closes the level
+cudaError_t launch_count(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
     // a fixed grid (the launch may sit in a captured graph); the blocks stride
     // over tiles of the list, or of V for the first count
     count_kernel<double><<<grid_for(p.n, COUNT_TILE, 152 * 4), COUNT_THREADS, 0, st>>>(
-        (const double*)b.walk, b.c, b.c32, b.lb, b.ub, g.perm, b.active, b.alist[0], b.alist[1], b.ctrl, p);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_finalize(const IterBuffers& b, const IterParams& p, cudaStream_t st) {
-    finalize_kernel<<<1, 256, 0, st>>>(b.topk_l, b.topk_u, b.trace, b.ctrl, p, b.cond_handle, b.use_cond);
+        (const double*)b.walk, b.c, b.c32, b.lb, b.ub, g.perm, b.active, b.alist[0], b.alist[1], b.topk_l, b.topk_u,
+        b.trace, b.sel.state, b.cond_handle, b.use_cond, b.ctrl, p);
     return cudaGetLastError();
 }
 
