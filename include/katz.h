@@ -112,8 +112,11 @@ typedef struct {
                               so that the walk values one hub row gathers from them sit
                               together and a line fetched from DRAM serves several gathers;
                               -1 keeps them in original-id order; 0 (default): 1 when
-                              n >= 2^25 (walk vectors several times larger than L2), else -1.
-                              Results are the same bits either way. */
+                              n >= 2^25 (walk vectors several times larger than L2) and the
+                              handle keeps its history, else -1: without history such a
+                              handle stages its gathers (about 4 bytes per arc and 10 per
+                              arc into the low-degree rows, at most a quarter of the free
+                              memory).  Results are the same bits either way. */
     int32_t reserved;      /* set to 0 */
 } katz_opts;
 

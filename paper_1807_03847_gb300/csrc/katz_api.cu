@@ -146,7 +146,13 @@ katz_status ensure_iter_buffers(katz_handle* h) {
         return cuda_fail(h, e, "cudaMalloc " #ptr);               \
     }
     char* walk = nullptr;
-    KALLOC(walk, (size_t)slots * stride * esz);
+    if (h->g.stage.n_items > 0 && dmalloc(h, &walk, (size_t)slots * stride * esz) != cudaSuccess) {
+        // the staged gathers give their memory back before a ranking fails for it
+        cudaGetLastError();
+        stage_free(h);
+        drop_graph(h);
+    }
+    if (!walk) KALLOC(walk, (size_t)slots * stride * esz);
     b.walk = walk;
     KALLOC(b.c, n);
     KALLOC(b.lb, n);  // bounds of the active nodes at the last level (cert mode: monotone)
@@ -182,7 +188,12 @@ katz_status ensure_iter_buffers(katz_handle* h) {
     return KATZ_OK;
 }
 
-// One iteration of Algorithm 1 (four kernels, five with hub rows; no host synchronisation).
+// SpMV (with the hub rows' merge, and the staged gathers), select (two), count
+int64_t iteration_kernels(const katz_handle* h) {
+    return 4 + (h->g.layout.row_warp > 0 ? 1 : 0) + (h->g.stage.n_items > 0 ? 1 : 0);
+}
+
+// One iteration of Algorithm 1 (no host synchronisation).
 // ev_pair: optional events recorded around the SpMV launch.
 cudaError_t launch_iteration(katz_handle* h, cudaEvent_t* ev_pair = nullptr) {
     cudaError_t e;
@@ -300,7 +311,7 @@ katz_status run_loop(katz_handle* h, int done) {
                 cudaEvent_t* ev = nullptr;
                 if (prof && 2 * launched_iters + 1 < (int)h->sp_ev.size()) ev = &h->sp_ev[2 * launched_iters];
                 if ((e = launch_iteration(h, ev)) != cudaSuccess) return cuda_fail(h, e, "launch iteration");
-                h->launches += (h->g.layout.row_warp > 0 ? 5 : 4);
+                h->launches += iteration_kernels(h);
                 ++launched_iters;
             }
         }
@@ -571,6 +582,7 @@ void katz_destroy(katz_h h) {
     dfree(h, h->g.chunk_row);
     dfree(h, h->g.chunk_first);
     dfree(h, h->g.chunk_part);
+    stage_free(h);
     dfree(h, h->d_deghist);
     dfree(h, h->d_scratch);
     dfree(h, h->rank_ids);
@@ -753,7 +765,7 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
     // behind the column slices still in flight
     struct HostVals {
         unsigned long long bad, bad_col, max_chunks;
-        int64_t degmax, chunks;
+        int64_t degmax, chunks, head_arcs;
         uint64_t cs[NUM_CLASSES];
     };
     static_assert(sizeof(HostVals) <= H_SMALL, "pinned scratch");
@@ -761,7 +773,12 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
     KCHK2(cudaMemcpyAsync(&hv.bad, d_bad, sizeof(hv.bad), cudaMemcpyDeviceToHost, h->stream), "copy");
     KCHK2(cudaMemcpyAsync(&hv.degmax, d_degmax, sizeof(hv.degmax), cudaMemcpyDeviceToHost, h->stream), "copy");
     KCHK2(cudaMemcpyAsync(hv.cs, class_start, sizeof(hv.cs), cudaMemcpyDeviceToHost, h->stream), "copy classes");
+    hv.head_arcs = nnz;
+    if (n >= STAGE_MIN_N)
+        KCHK2(cudaMemcpyAsync(&hv.head_arcs, rp_new + STAGE_HOT, sizeof(int64_t), cudaMemcpyDeviceToHost, h->stream),
+              "copy");
     KCHK2(cudaStreamSynchronize(h->stream), "validate sync");
+    const int64_t head_arcs = hv.head_arcs;
     if (hv.bad) {
         drop_staging();
         katz_destroy(h);
@@ -793,8 +810,9 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
     // then the low-degree rows reordered inside their classes by anchor
     // (katz_opts.locality); the rows of degree > 16 keep their places, the
     // staging column array holds the old tail
-    const bool locality = (h->opts.locality > 0 || (h->opts.locality == 0 && n >= ((int64_t)1 << 25))) &&
-                          n - row_thread > 1;
+    const bool locality =
+        (h->opts.locality > 0 || (h->opts.locality == 0 && n >= ((int64_t)1 << 25) && !stage_wanted(h, head_arcs))) &&
+        n - row_thread > 1;
     if (locality) {
         const int64_t m = n - row_thread, cnt = 256 * radix_tiles(m);
         RadixBuffers rs;
@@ -861,6 +879,7 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
         return KATZ_EINVAL;
     }
 #undef KCHK2
+    KCHK(stage_build(h, head_arcs), "staged gathers");
     if ((st = alloc_rank_scratch(h)) != KATZ_OK) {
         katz_destroy(h);
         return st;
@@ -966,7 +985,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->trace.assign(tr.begin() + 1, tr.begin() + 1 + std::max(0, h->r));
     if (h->opts.use_graph && !h->opts.profile)
         // loop bodies that did work: all finalize runs but the first iteration's
-        h->launches += (h->g.layout.row_warp > 0 ? 5 : 4) * std::max<int64_t>(0, (int64_t)hc.body_runs - 1);
+        h->launches += iteration_kernels(h) * std::max<int64_t>(0, (int64_t)hc.body_runs - 1);
     double spmv_ms = 0.0;
     if (h->opts.profile) {  // levels 2..r: level 1 reads no walk values
         for (int q = 1; q < h->r && 2 * q + 1 < (int)h->sp_ev.size(); ++q) {
@@ -1038,7 +1057,7 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     h->criterion = criterion;
     h->ranked = false;
     h->launches = 0;
-    const int64_t spmv_kernels = h->g.layout.row_warp > 0 ? 2 : 1;
+    const int64_t spmv_kernels = iteration_kernels(h) - 3;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
     if ((e = cudaMemsetAsync(h->b.ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess ||
         (e = launch_init_walk(h->g, h->b, p, false, h->stream)) != cudaSuccess ||

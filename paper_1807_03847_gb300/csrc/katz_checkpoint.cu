@@ -329,6 +329,18 @@ katz_status katz_restore(katz_h* out, const void* buf, uint64_t bytes, const kat
             return KATZ_EINVAL;
         }
     }
+    int64_t head_arcs = hd.nnz;
+    if (hd.n >= STAGE_MIN_N) {  // one offset, of either width
+        int32_t narrow = 0;
+        e = g.off64 ? cudaMemcpy(&head_arcs, (int64_t*)g.rowptr + STAGE_HOT, sizeof(int64_t), cudaMemcpyDeviceToHost)
+                    : cudaMemcpy(&narrow, (int32_t*)g.rowptr + STAGE_HOT, sizeof(int32_t), cudaMemcpyDeviceToHost);
+        if (!g.off64) head_arcs = narrow;
+    }
+    if (e != cudaSuccess || (e = stage_build(h, head_arcs)) != cudaSuccess) {
+        st = cuda_fail(h, e, "staged gathers");
+        katz_destroy(h);
+        return st;
+    }
     h->p = hd.p;
     h->k_eff = hd.k_eff;
     h->f32_from = hd.f32_from;

@@ -151,6 +151,11 @@ __device__ __forceinline__ double walk_value(const double* walk, const IterParam
 // ---- launchers (katz_kernels.cu) -------------------------------------------
 
 // Internal row ranges of the SpMV row modes and their block ranges.
+// Staged gathers (katz_stage.cu): from this many vertices, with this many of
+// the vector's first entries (64 MB of FP64, half of L2) gathered directly
+constexpr int64_t STAGE_MIN_N = (int64_t)1 << 25;
+constexpr int64_t STAGE_HOT = (int64_t)1 << 23;
+
 struct SpmvLayout {
     int64_t n;
     int64_t row_warp;    // rows [0, row_warp): CHUNK mode (degree > 2048)
@@ -158,6 +163,23 @@ struct SpmvLayout {
     int64_t row_thread;  // rows [row_octet, row_thread): OCTET mode; [row_thread, n): THREAD
     int64_t chunks;      // CHUNK_ARCS-arc chunks of the CHUNK rows
     int64_t blk_warp, blk_octet, blk_thread, blocks_total;  // first block of each mode
+};
+
+// Staged gathers (katz_stage.cu): one window's places in bands [band0, band1)
+struct StageItem {
+    int32_t window;
+    int32_t band0, band1;
+};
+
+struct StageMap {
+    uint32_t* src = nullptr;    // [nnz] per arc: below hot an internal id, else hot + the arc's place in y
+    uint16_t* local = nullptr;  // [places] entry within the place's window
+    void* y = nullptr;          // [places] the staged values, FP64 or FP32 as the level's input
+    uint32_t* first = nullptr;  // [bands * windows + 1] first place of each (band, window) segment
+    StageItem* items = nullptr;
+    int32_t windows = 0;
+    int32_t n_items = 0;        // 0: plain gathers
+    uint32_t hot = 0;
 };
 
 struct DeviceGraph {
@@ -171,6 +193,7 @@ struct DeviceGraph {
     int64_t* chunk_first = nullptr;   // [row_warp + 1] first chunk of each CHUNK row
     double* chunk_part = nullptr;     // [3 chunks] chunk partial sums (three words per chunk)
     SpmvLayout layout{};
+    StageMap stage;                   // handles without history only: an update would move the arcs
 };
 
 // The filtered candidates of the select (katz_kernels.cu): SELECT_CAP entries.
@@ -341,6 +364,7 @@ cudaError_t launch_degree_store(const DeviceGraph& g, const IterBuffers& b, cons
 cudaError_t launch_degree_level(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
 cudaError_t launch_spmv(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
                         cudaStream_t st);
+cudaError_t launch_stage(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
 cudaError_t launch_spmv_store(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int level,
                               cudaStream_t st);
 // s_level recomputed for the listed rows (CHUNK rows excepted) and for the

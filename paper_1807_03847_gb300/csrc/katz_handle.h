@@ -166,6 +166,11 @@ inline void dfree_on(void* p, cudaStream_t st) {
     if (p) cudaFreeAsync(p, st);
 }
 
+// staged gathers of the handle's graph (katz_stage.cu); head_arcs: arcs of the
+// rows below STAGE_HOT
+bool stage_wanted(const katz_handle* h, int64_t head_arcs);
+cudaError_t stage_build(katz_handle* h, int64_t head_arcs);
+void stage_free(katz_handle* h);
 katz_status init_handle_runtime(katz_handle* h);
 katz_status ensure_iter_buffers(katz_handle* h);
 katz_status alloc_rank_scratch(katz_handle* h);

@@ -415,21 +415,40 @@ __device__ __forceinline__ double xacc_to_double(const XAcc& a) {
     return ldexp((double)T, be - 1075);  // subnormal result
 }
 
-// Exact sum of x[col[j]] for j in [a, b) with stride `step` from a + first:
+// Where an arc's value is read: the vector itself (entries S apart: S = 2 is
+// one state of the interleaved pairs of the two-state pass below), or, with
+// staged gathers (katz_stage.cu), the vector below `hot` and the arc's staged
+// place above (y points hot entries before the staged values).
+template <typename T, int S = 1>
+struct Direct {
+    const T* __restrict__ x;
+    __device__ __forceinline__ T operator()(int32_t c) const { return __ldg(x + (int64_t)S * c); }
+};
+
+template <typename T>
+struct Staged {
+    const T* __restrict__ x;
+    const T* __restrict__ y;
+    uint32_t hot;
+    __device__ __forceinline__ T operator()(int32_t c) const {
+        const uint32_t u = (uint32_t)c;
+        return __ldg((u < hot ? x : y) + u);
+    }
+};
+
+// Exact sum of x(col[j]) for j in [a, b) with stride `step` from a + first:
 // groups of G loads in flight (past the end: zero, which adds nothing).
 // G = 8 for rows whose lanes see many terms, G = 4 for short rows (fewer
 // padded slots).
-// S: entries of x are S apart (S = 2: one state of the interleaved pairs of
-// the two-state pass below).
-template <int G, int S = 1>
-__device__ __forceinline__ XAcc strided_xsum(const int32_t* __restrict__ col, const double* __restrict__ x,
-                                             int64_t a, int64_t b, int first, int step) {
+template <int G, typename X>
+__device__ __forceinline__ XAcc strided_xsum(const int32_t* __restrict__ col, const X& x, int64_t a, int64_t b,
+                                             int first, int step) {
     XAcc s = xacc_zero();
     const int32_t* __restrict__ cp = col + (a + first);
     for (int left = (int)(b - a) - first; left > 0; left -= G * step, cp += G * step) {
         double v[G];
 #pragma unroll
-        for (int q = 0; q < G; ++q) v[q] = left > q * step ? __ldg(x + (int64_t)S * cp[q * step]) : 0.0;
+        for (int q = 0; q < G; ++q) v[q] = left > q * step ? x(cp[q * step]) : 0.0;
         xacc_add_group(s, v);
     }
     return s;
@@ -465,15 +484,15 @@ __device__ __forceinline__ XAcc merge_chunks_warp(const double* __restrict__ par
 // Sum of x[col[j]] for j in [a, b) with stride `step` from a + first: eight
 // loads in flight, each group of eight added as a pairwise tree (depth 3),
 // groups chained in index order.
-template <typename Tin, typename Acc, int S = 1>
-__device__ __forceinline__ Acc strided_sum(const int32_t* __restrict__ col, const Tin* __restrict__ x, int64_t a,
-                                           int64_t b, int first, int step) {
+template <typename Acc, typename X>
+__device__ __forceinline__ Acc strided_sum(const int32_t* __restrict__ col, const X& x, int64_t a, int64_t b,
+                                           int first, int step) {
     Acc s = (Acc)0;
     const int32_t* __restrict__ cp = col + (a + first);
     for (int left = (int)(b - a) - first; left > 0; left -= 8 * step, cp += 8 * step) {
         Acc v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = left > q * step ? (Acc)__ldg(x + (int64_t)S * cp[q * step]) : (Acc)0;
+        for (int q = 0; q < 8; ++q) v[q] = left > q * step ? (Acc)x(cp[q * step]) : (Acc)0;
         const Acc t = addA<Acc>(addA<Acc>(addA<Acc>(v[0], v[1]), addA<Acc>(v[2], v[3])),
                                 addA<Acc>(addA<Acc>(v[4], v[5]), addA<Acc>(v[6], v[7])));
         s = addA<Acc>(s, t);
@@ -481,18 +500,17 @@ __device__ __forceinline__ Acc strided_sum(const int32_t* __restrict__ col, cons
     return s;
 }
 
-// One level: Tin = type of level r-1, Tout = type of level r.  FP64 levels
+// One level of type T (its input x has the same type).  FP64 levels
 // sum exactly (XAcc); FP32 levels add in FP32 (fixed pairwise order).
-template <typename Off, typename Tin, typename Tout>
+template <typename Off, typename T, typename X>
 __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                          const SpmvLayout& L, const Tin* __restrict__ x, const Epi& ep,
+                                          const SpmvLayout& L, const X& x, const Epi& ep,
                                           const int32_t* __restrict__ chunk_row,
                                           const int64_t* __restrict__ chunk_first, double* chunk_part,
                                           const IterParams& p) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t b = blockIdx.x;
-    if constexpr (sizeof(Tout) == 8) {
-        static_assert(sizeof(Tin) == 8, "FP64 levels follow FP64 levels");
+    if constexpr (sizeof(T) == 8) {
         if (b >= L.blk_thread) {  // THREAD rows
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
             if (u < L.n) finish_row<double>(u, xacc_to_double(strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], 0, 1)), ep, p);
@@ -525,19 +543,19 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
         typedef float Acc;
         if (b >= L.blk_thread) {  // THREAD rows
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
-            if (u < L.n) finish_row<Acc>(u, strided_sum<Tin, Acc>(col, x, rowptr[u], rowptr[u + 1], 0, 1), ep, p);
+            if (u < L.n) finish_row<Acc>(u, strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], 0, 1), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
             const int64_t u = L.row_octet + (b - L.blk_octet) * (BLOCK / 8) + (tid >> 3);
             const int sub = tid & 7;
             Acc s = (Acc)0;
-            if (u < L.row_thread) s = strided_sum<Tin, Acc>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
+            if (u < L.row_thread) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
 #pragma unroll
             for (int off = 4; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off, 8));
             if (sub == 0 && u < L.row_thread) finish_row<Acc>(u, s, ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
             const int64_t u = L.row_warp + (b - L.blk_warp) * WARPS + wid;
             Acc s = (Acc)0;
-            if (u < L.row_octet) s = strided_sum<Tin, Acc>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
+            if (u < L.row_octet) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
 #pragma unroll
             for (int off = 16; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off));
             if (lane == 0 && u < L.row_octet) finish_row<Acc>(u, s, ep, p);
@@ -548,7 +566,7 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
                 const int64_t u = chunk_row[ch];
                 const int64_t j0 = (int64_t)rowptr[u] + (ch - chunk_first[u]) * (int64_t)CHUNK_ARCS;
                 const int64_t j1 = min(j0 + (int64_t)CHUNK_ARCS, (int64_t)rowptr[u + 1]);
-                s = strided_sum<Tin, Acc>(col, x, j0, j1, lane, 32);
+                s = strided_sum<Acc>(col, x, j0, j1, lane, 32);
             }
 #pragma unroll
             for (int off = 16; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off));
@@ -593,10 +611,12 @@ __global__ void degree_level_kernel(const Off* __restrict__ rowptr, int64_t n, d
 }
 
 // Six 256-thread blocks per SM (40 registers): the gathers need the warps in
-// flight more than the lanes need registers.
-template <typename Off>
+// flight more than the lanes need registers.  Stage: col holds the arcs'
+// staged sources (StageMap::src), stage_y the staged values.
+template <typename Off, bool Stage>
 __global__ void __launch_bounds__(BLOCK, 6)
-spmv_rows_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col, SpmvLayout L, double* walk,
+spmv_rows_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col, SpmvLayout L,
+                 const void* __restrict__ stage_y, uint32_t hot, double* walk,
                  double* c64, double* c32, double* lb, double* ub, uint8_t* active, const int32_t* __restrict__ perm,
                  const int32_t* __restrict__ chunk_row, const int64_t* __restrict__ chunk_first, double* chunk_part,
                  double* cand_l, double* cand_u, int32_t* cand_id, int64_t cand_cap, float* s32, Ctrl* ctrl,
@@ -610,12 +630,25 @@ spmv_rows_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
     Epi ep = make_epi(ys, c64, c32, lb, ub, active, perm, cand_l, cand_u, cand_id, cand_cap, ctrl, p,
                       writes_s32(ctrl, p, r_cur, store_level) ? s32 : nullptr);
     ep.store_only = store_level > 0;
-    if (r_cur < f32_from)  // level 1, when it comes here, gathers s_0 = 1 (f32_from >= 2)
-        spmv_rows<Off, double, double>(rowptr, col, L, xs, ep, chunk_row, chunk_first, chunk_part, p);
-    else if (r_cur == f32_from)
-        spmv_rows<Off, float, float>(rowptr, col, L, s32, ep, chunk_row, chunk_first, chunk_part, p);
-    else
-        spmv_rows<Off, float, float>(rowptr, col, L, (const float*)xs, ep, chunk_row, chunk_first, chunk_part, p);
+    if constexpr (Stage) {
+        if (r_cur < f32_from)
+            spmv_rows<Off, double>(rowptr, col, L, Staged<double>{xs, (const double*)stage_y - hot, hot}, ep, chunk_row,
+                                   chunk_first, chunk_part, p);
+        else if (r_cur == f32_from)
+            spmv_rows<Off, float>(rowptr, col, L, Staged<float>{s32, (const float*)stage_y - hot, hot}, ep, chunk_row,
+                                  chunk_first, chunk_part, p);
+        else
+            spmv_rows<Off, float>(rowptr, col, L, Staged<float>{(const float*)xs, (const float*)stage_y - hot, hot}, ep,
+                                  chunk_row, chunk_first, chunk_part, p);
+    } else {
+        if (r_cur < f32_from)  // level 1, when it comes here, gathers s_0 = 1 (f32_from >= 2)
+            spmv_rows<Off, double>(rowptr, col, L, Direct<double>{xs}, ep, chunk_row, chunk_first, chunk_part, p);
+        else if (r_cur == f32_from)
+            spmv_rows<Off, float>(rowptr, col, L, Direct<float>{s32}, ep, chunk_row, chunk_first, chunk_part, p);
+        else
+            spmv_rows<Off, float>(rowptr, col, L, Direct<float>{(const float*)xs}, ep, chunk_row, chunk_first,
+                                  chunk_part, p);
+    }
 }
 
 // CHUNK rows of an FP32 level: the chunk sums of a row, in groups of 64, each
@@ -691,20 +724,28 @@ int max_sum_depth(const SpmvLayout& L, int64_t max_chunks_per_row) {
                         L.row_warp > 0 ? std::max<int64_t>(max_chunks_per_row, 1) : 0);
 }
 
+template <typename Off, bool Stage>
+static void spmv_rows_launch(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int store_level,
+                             cudaStream_t st) {
+    spmv_rows_kernel<Off, Stage><<<(unsigned)g.layout.blocks_total, BLOCK, 0, st>>>(
+        (const Off*)g.rowptr, Stage ? (const int32_t*)g.stage.src : g.col, g.layout, g.stage.y, g.stage.hot,
+        (double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, g.perm, g.chunk_row, g.chunk_first, g.chunk_part, b.cand_l,
+        b.cand_u, b.cand_id, b.cand_cap, b.s32, b.ctrl, p, store_level);
+}
+
 static cudaError_t spmv_launch(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int store_level,
                                cudaStream_t st) {
     const SpmvLayout& L = g.layout;
+    const bool stage = g.stage.n_items > 0 && !store_level;
+    if (stage) {
+        const cudaError_t e = launch_stage(g, b, p, st);
+        if (e != cudaSuccess) return e;
+    }
     if (L.blocks_total > 0) {
-        if (g.off64)
-            spmv_rows_kernel<int64_t><<<(unsigned)L.blocks_total, BLOCK, 0, st>>>(
-                (const int64_t*)g.rowptr, g.col, L, (double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, g.perm,
-                g.chunk_row, g.chunk_first, g.chunk_part, b.cand_l, b.cand_u, b.cand_id, b.cand_cap, b.s32, b.ctrl, p,
-                store_level);
-        else
-            spmv_rows_kernel<int32_t><<<(unsigned)L.blocks_total, BLOCK, 0, st>>>(
-                (const int32_t*)g.rowptr, g.col, L, (double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, g.perm,
-                g.chunk_row, g.chunk_first, g.chunk_part, b.cand_l, b.cand_u, b.cand_id, b.cand_cap, b.s32, b.ctrl, p,
-                store_level);
+        if (g.off64 && stage) spmv_rows_launch<int64_t, true>(g, b, p, store_level, st);
+        else if (g.off64) spmv_rows_launch<int64_t, false>(g, b, p, store_level, st);
+        else if (stage) spmv_rows_launch<int32_t, true>(g, b, p, store_level, st);
+        else spmv_rows_launch<int32_t, false>(g, b, p, store_level, st);
     }
     if (L.row_warp > 0)
         spmv_chunk_fixup<<<(unsigned)((L.row_warp * 32 + 127) / 128), 128, 0, st>>>(
@@ -795,7 +836,7 @@ __global__ void rows_store_kernel(const Off* __restrict__ rowptr, const int32_t*
     const int64_t nrows = (int64_t)*nrows_ptr;
     const int f32_from = ctrl->f32_from;
     if (level >= f32_from) {  // FP32 level: the FP32 order of spmv_rows
-        const float* __restrict__ x = level == f32_from ? s32 : (const float*)walk_slot(walk, p, level - 1);
+        const Direct<float> x{level == f32_from ? s32 : (const float*)walk_slot(walk, p, level - 1)};
         float* y = (float*)walk_slot(walk, p, level);
         for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; w < nrows; w += warps) {
             const int64_t u = rows[w];
@@ -803,13 +844,13 @@ __global__ void rows_store_kernel(const Off* __restrict__ rowptr, const int32_t*
             const int64_t a = rowptr[u], e = rowptr[u + 1];
             float s = 0.0f;
             if (u >= L.row_thread) {
-                if (lane == 0) s = strided_sum<float, float>(col, x, a, e, 0, 1);
+                if (lane == 0) s = strided_sum<float>(col, x, a, e, 0, 1);
             } else if (u >= L.row_octet) {
-                if (lane < 8) s = strided_sum<float, float>(col, x, a, e, lane, 8);
+                if (lane < 8) s = strided_sum<float>(col, x, a, e, lane, 8);
 #pragma unroll
                 for (int off = 4; off; off >>= 1) s = addA<float>(s, __shfl_down_sync(FULL, s, off, 8));
             } else {
-                s = strided_sum<float, float>(col, x, a, e, lane, 32);
+                s = strided_sum<float>(col, x, a, e, lane, 32);
 #pragma unroll
                 for (int off = 16; off; off >>= 1) s = addA<float>(s, __shfl_down_sync(FULL, s, off));
             }
@@ -817,7 +858,7 @@ __global__ void rows_store_kernel(const Off* __restrict__ rowptr, const int32_t*
         }
         return;
     }
-    const double* __restrict__ x = walk_slot(walk, p, level - 1);
+    const Direct<double> x{walk_slot(walk, p, level - 1)};
     double* y = walk_slot(walk, p, level);
     float* t = writes_s32(ctrl, p, level, level) ? s32 : nullptr;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; w < nrows; w += warps) {
@@ -856,15 +897,15 @@ __global__ void hub_chunks_store_kernel(const Off* __restrict__ rowptr, const in
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
     const int f32_from = ctrl->f32_from;
-    const double* __restrict__ x = walk_slot(walk, p, level - 1);
-    const float* __restrict__ xf = level == f32_from ? s32 : (const float*)x;
+    const Direct<double> x{walk_slot(walk, p, level - 1)};
+    const Direct<float> xf{level == f32_from ? s32 : (const float*)x.x};
     for (int64_t ch = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; ch < L.chunks; ch += warps) {
         const int64_t u = chunk_row[ch];
         if (!visited(vbits, u)) continue;
         const int64_t j0 = (int64_t)rowptr[u] + (ch - chunk_first[u]) * (int64_t)CHUNK_ARCS;
         const int64_t j1 = min(j0 + (int64_t)CHUNK_ARCS, (int64_t)rowptr[u + 1]);
         if (level >= f32_from) {  // FP32 level: the chunk sum of spmv_rows, exact in FP64
-            float s = strided_sum<float, float>(col, xf, j0, j1, lane, 32);
+            float s = strided_sum<float>(col, xf, j0, j1, lane, 32);
 #pragma unroll
             for (int off = 16; off; off >>= 1) s = addA<float>(s, __shfl_down_sync(FULL, s, off));
             if (lane == 0) chunk_part[3 * ch] = (double)s;
@@ -1159,30 +1200,30 @@ __global__ void pair_fix_rows_kernel(const Off* __restrict__ rowptr, const int32
         const int64_t u = rows[w];
         const int64_t a = rowptr[u], e = rowptr[u + 1];
         if (level >= f32_from) {
-            const float* __restrict__ x = level == f32_from ? (const float*)t_in
-                                                            : (const float*)(P + (size_t)(level - 1) * pstride);
+            const Direct<float, 2> x{level == f32_from ? (const float*)t_in
+                                                       : (const float*)(P + (size_t)(level - 1) * pstride)};
             float s = 0.0f;
             if (u >= L.row_thread) {
-                if (lane == 0) s = strided_sum<float, float, 2>(col, x, a, e, 0, 1);
+                if (lane == 0) s = strided_sum<float>(col, x, a, e, 0, 1);
             } else if (u >= L.row_octet) {
-                if (lane < 8) s = strided_sum<float, float, 2>(col, x, a, e, lane, 8);
+                if (lane < 8) s = strided_sum<float>(col, x, a, e, lane, 8);
                 s = fsum_group<8>(s);
             } else {
-                s = strided_sum<float, float, 2>(col, x, a, e, lane, 32);
+                s = strided_sum<float>(col, x, a, e, lane, 32);
                 s = fsum_group<32>(s);
             }
             if (lane == 0) ((float*)(P + (size_t)level * pstride))[2 * u] = __fmul_rn(alpha_f, s);
             continue;
         }
-        const double* __restrict__ x = P + (size_t)(level - 1) * pstride;
+        const Direct<double, 2> x{P + (size_t)(level - 1) * pstride};
         XAcc s = xacc_zero();
         if (u >= L.row_thread) {
-            if (lane == 0) s = strided_xsum<4, 2>(col, x, a, e, 0, 1);
+            if (lane == 0) s = strided_xsum<4>(col, x, a, e, 0, 1);
         } else if (u >= L.row_octet) {
-            if (lane < 8) s = strided_xsum<4, 2>(col, x, a, e, lane, 8);
+            if (lane < 8) s = strided_xsum<4>(col, x, a, e, lane, 8);
             s = xacc_group_sum<8>(s);
         } else {
-            s = strided_xsum<8, 2>(col, x, a, e, lane, 32);
+            s = strided_xsum<8>(col, x, a, e, lane, 32);
             s = xacc_group_sum<32>(s);
         }
         if (lane == 0) {
@@ -1208,12 +1249,13 @@ __global__ void pair_fix_hub_chunks_kernel(const Off* __restrict__ rowptr, const
         const int64_t j0 = (int64_t)rowptr[u] + (ch - chunk_first[u]) * (int64_t)CHUNK_ARCS;
         const int64_t j1 = min(j0 + (int64_t)CHUNK_ARCS, (int64_t)rowptr[u + 1]);
         if (level >= f32_from) {
-            const float* __restrict__ x = level == f32_from ? (const float*)t_in
-                                                            : (const float*)(P + (size_t)(level - 1) * pstride);
-            const float s = fsum_group<32>(strided_sum<float, float, 2>(col, x, j0, j1, lane, 32));
+            const Direct<float, 2> x{level == f32_from ? (const float*)t_in
+                                                       : (const float*)(P + (size_t)(level - 1) * pstride)};
+            const float s = fsum_group<32>(strided_sum<float>(col, x, j0, j1, lane, 32));
             if (lane == 0) part[3 * ch] = (double)s;
         } else {
-            const XAcc t = xacc_group_sum<32>(strided_xsum<8, 2>(col, P + (size_t)(level - 1) * pstride, j0, j1, lane, 32));
+            const XAcc t = xacc_group_sum<32>(
+                strided_xsum<8>(col, Direct<double, 2>{P + (size_t)(level - 1) * pstride}, j0, j1, lane, 32));
             if (lane == 0) store_part(part, ch, t);
         }
     }

@@ -1,0 +1,283 @@
+// Staged gathers for walk vectors far larger than L2.
+//
+// A gather of s_{r-1} that misses L2 moves a whole 128-byte line from DRAM for
+// 8 bytes: on a Chung-Lu graph of 2^27 vertices a level read 111 GB against 14
+// GB of algorithmic bytes, at the measured copy bandwidth.  So the arcs into
+// the cold part of the vector (internal ids from `hot` on: the low-degree end
+// of the degree-class order) get their values in two steps that only stream:
+//
+//   1. stage_gather: the cold part is cut into windows of STAGE_WIN entries.
+//      A block loads one window into shared memory and writes, for every arc
+//      into it, the value gathered there to the arc's place in y.  The rows
+//      form STAGE_BANDS runs of equal numbers of arcs; y holds one band after
+//      the other, and in a band the places of one window's arcs are
+//      consecutive, in the order of the arcs' rows (a segment).
+//   2. the SpMV reads y at the arc's place instead of the vector.  Rows that
+//      run at the same time take neighbouring places of every window, so each
+//      line of y is fetched once and shared while it is in L2, and the places
+//      in use at one time lie in one band.  With y in one band
+//      (7.6 GB at 2^27 vertices, one page of every window in use at a time) the
+//      SpMV took 16.3 ms; address translation bound it, not DRAM (24 GB read).
+//      32 bands: 9.7 ms; 16 bands: 13.6 for the level in place of 11.6.
+//
+// Per cold arc that is 2 + 8 bytes in step 1 and 8 in step 2 (4-byte values: 2
+// + 4 and 4) in place of 128.  The values and the order of every row sum are
+// those of the plain gather, so the results are the same bits.
+//
+// Measured on that graph, FP64: a level 17.1 -> 11.4 ms (2.3 of it step 1), the
+// ranking 193 -> 131 ms; n = 6e7: 63.2 -> 54.9 ms, FP32-certified 57.3 -> 53.1;
+// n = 4e7: 38.2 -> 36.1; G(3.6e7, 4 n): 48.8 -> 27.9.  Building it takes no more of
+// a create than the anchor order (katz_relabel.cu), which it replaces: 61 against
+// 77 ms at 2^27.  Below 2^25 vertices the gain (2.68 -> 2.54 ms a level at 2^25 - 39)
+// does not pay for a create three times as long.
+//
+// 2^23 hot entries, 8192 per window: with 2^22 the level took 11.6 ms, 2^21 12.5,
+// 2^24 12.3 (the hot part then contends for L2); 64 or 128 bands changed nothing;
+// windows of 16384 (one block per SM) 16.1 ms with 16 bands.
+#include <stdint.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "katz_common.cuh"
+#include "katz_handle.h"
+
+namespace katz {
+
+namespace {
+
+constexpr int STAGE_BITS = 13;
+constexpr int STAGE_WIN = 1 << STAGE_BITS;   // entries per window: 64 KB of FP64, three blocks per SM
+constexpr int STAGE_THREADS = 512;
+constexpr int STAGE_WARPS = STAGE_THREADS / 32;
+constexpr int STAGE_BANDS = 2 * STAGE_WARPS; // runs of rows with equal numbers of arcs
+constexpr int STAGE_CHUNK = 1 << 16;         // arcs per block: a window is loaded once per chunk
+constexpr int STAGE_ALIGN = 32;              // places of a segment start at a multiple of this
+constexpr int STAGE_MAX_WINDOWS = 1 << 15;   // 128 KB of counters in shared memory
+constexpr int STAGE_HIST_BLOCKS = 10;        // per band
+constexpr int STAGE_ASSIGN = 2048;           // arcs per block of the assignment; a band is a multiple of it
+
+// arcs of every band into every window (gridDim.y: the band)
+__global__ void __launch_bounds__(1024)
+stage_hist_kernel(const int32_t* __restrict__ col, int64_t nnz, int64_t band_arcs, uint32_t hot, int windows,
+                  unsigned int* counts) {
+    extern __shared__ unsigned int h[];
+    for (int q = threadIdx.x; q < windows; q += blockDim.x) h[q] = 0;
+    __syncthreads();
+    const int64_t end = min(nnz, (int64_t)(blockIdx.y + 1) * band_arcs);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t j0 = blockIdx.y * band_arcs + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j0 < end;
+         j0 += 4 * stride) {
+        uint32_t c[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] = j0 + q * stride < end ? (uint32_t)col[j0 + q * stride] : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (c[q] >= hot) atomicAdd(&h[(c[q] - hot) >> STAGE_BITS], 1u);
+    }
+    __syncthreads();
+    unsigned int* out = counts + (size_t)blockIdx.y * windows;
+    for (int q = threadIdx.x; q < windows; q += blockDim.x)
+        if (h[q]) atomicAdd(&out[q], h[q]);
+}
+
+// the place of every cold arc: blocks run in arc order, so the places of a
+// segment follow the order of the rows up to the blocks in flight
+__global__ void __launch_bounds__(256)
+stage_assign_kernel(const int32_t* __restrict__ col, int64_t nnz, int64_t band_arcs, uint32_t hot, int windows,
+                    unsigned int* cursor, uint32_t* __restrict__ src, uint16_t* __restrict__ local) {
+    const int64_t j0 = (int64_t)blockIdx.x * STAGE_ASSIGN + threadIdx.x;
+    unsigned int* cur = cursor + (size_t)((int64_t)blockIdx.x * STAGE_ASSIGN / band_arcs) * windows;
+    constexpr int U = STAGE_ASSIGN / 256;
+    uint32_t c[U], p[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) c[q] = j0 + q * 256 < nnz ? (uint32_t)col[j0 + q * 256] : 0u;
+#pragma unroll
+    for (int q = 0; q < U; ++q) p[q] = c[q] >= hot ? atomicAdd(&cur[(c[q] - hot) >> STAGE_BITS], 1u) : 0u;
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+        if (j0 + q * 256 >= nnz) continue;
+        if (c[q] >= hot) local[p[q]] = (uint16_t)((c[q] - hot) & (STAGE_WIN - 1));
+        src[j0 + q * 256] = c[q] >= hot ? hot + p[q] : c[q];
+    }
+}
+
+// y[p] = x[entry of place p] for the places of one window in some bands, a
+// warp per band
+template <typename T>
+__device__ __forceinline__ void stage_window(const T* __restrict__ x, int64_t n, const StageMap& m,
+                                             const StageItem& it, T* win) {
+    const int64_t base = (int64_t)m.hot + ((int64_t)it.window << STAGE_BITS);
+    const int len = (int)min((int64_t)STAGE_WIN, n - base);
+    constexpr int V = 16 / (int)sizeof(T);
+    const uint4* __restrict__ src = (const uint4*)(x + base);  // 16-byte aligned: base and the slots are
+#pragma unroll 4
+    for (int q = threadIdx.x; q < len / V; q += STAGE_THREADS) ((uint4*)win)[q] = src[q];
+    for (int q = len / V * V + threadIdx.x; q < len; q += STAGE_THREADS) win[q] = x[base + q];
+    __syncthreads();
+    // two places per lane (a place past a segment's last one holds entry 0 and is read by no arc)
+    struct alignas(2 * sizeof(T)) Two { T a, b; };
+    const int lane = threadIdx.x & 31;
+    for (int band = it.band0 + (threadIdx.x >> 5); band < it.band1; band += STAGE_WARPS) {
+        const uint32_t first = m.first[(size_t)band * m.windows + it.window];
+        const int pairs = (int)(m.first[(size_t)band * m.windows + it.window + 1] - first) / 2;  // padded
+        const ushort2* __restrict__ l2 = (const ushort2*)(m.local + first);
+        Two* __restrict__ y2 = (Two*)((T*)m.y + first);
+#pragma unroll 4
+        for (int q = lane; q < pairs; q += 32) {
+            const ushort2 e = __ldcs(l2 + q);
+            y2[q] = Two{win[e.x], win[e.y]};
+        }
+    }
+}
+
+// level types as in spmv_rows_kernel: the FP64 slot, the roundings s32, or the
+// FP32 slot of level r-1
+__global__ void __launch_bounds__(STAGE_THREADS, 3)
+stage_gather_kernel(StageMap m, const double* walk, const float* __restrict__ s32, const Ctrl* ctrl, IterParams p) {
+    extern __shared__ uint4 win[];
+    if (ctrl->stop) return;
+    const int r_cur = ctrl->r + 1, f32_from = ctrl->f32_from;
+    const double* xs = walk_slot(walk, p, r_cur - 1);
+    const StageItem it = m.items[blockIdx.x];
+    if (r_cur < f32_from)
+        stage_window<double>(xs, p.n, m, it, (double*)win);
+    else
+        stage_window<float>(r_cur == f32_from ? s32 : (const float*)xs, p.n, m, it, (float*)win);
+}
+
+}  // namespace
+
+cudaError_t launch_stage(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
+    stage_gather_kernel<<<(unsigned)g.stage.n_items, STAGE_THREADS, STAGE_WIN * sizeof(double), st>>>(
+        g.stage, (const double*)b.walk, b.s32, b.ctrl, p);
+    return cudaGetLastError();
+}
+
+void stage_free(katz_handle* h) {
+    StageMap& m = h->g.stage;
+    dfree(h, m.src);
+    dfree(h, m.local);
+    dfree(h, m.y);
+    dfree(h, m.items);
+    dfree(h, m.first);
+    m = StageMap();
+}
+
+// Worth it where many arcs are cold.  In a symmetric graph as many arcs lead
+// into the rows from STAGE_HOT on as leave them; for a directed one that is an
+// estimate.  The places must fit 32 bits and the windows' counters one block.
+bool stage_wanted(const katz_handle* h, int64_t head_arcs) {
+    const int64_t n = h->g.n, nnz = h->g.nnz, cold = nnz - head_arcs;
+    if (n < STAGE_MIN_N || h->opts.keep_history || cold < nnz / 8) return false;
+    const int64_t windows = (n - STAGE_HOT + STAGE_WIN - 1) / STAGE_WIN;
+    return windows <= STAGE_MAX_WINDOWS &&
+           STAGE_HOT + cold + windows * STAGE_BANDS * STAGE_ALIGN <= (int64_t)0xffffffff;
+}
+
+// The staged gathers of the graph a handle holds (its final internal order).
+// Without the memory for them the handle goes on with plain gathers.  Waits
+// for the handle's stream.
+cudaError_t stage_build(katz_handle* h, int64_t head_arcs) {
+    DeviceGraph& g = h->g;
+    if (!stage_wanted(h, head_arcs)) return cudaSuccess;
+    const uint32_t hot = (uint32_t)STAGE_HOT;
+    const int64_t span = g.n - STAGE_HOT;
+    const int64_t windows = (span + STAGE_WIN - 1) / STAGE_WIN;
+    cudaError_t e;
+    const size_t cells = (size_t)windows * STAGE_BANDS;
+    const int64_t band_arcs = ((g.nnz + STAGE_BANDS - 1) / STAGE_BANDS + STAGE_ASSIGN - 1) / STAGE_ASSIGN * STAGE_ASSIGN;
+    unsigned int* counts = nullptr;
+    if ((e = dmalloc(h, &counts, cells)) != cudaSuccess) return e;
+    std::vector<unsigned int> cnt(cells), first(cells + 1);
+    e = cudaMemsetAsync(counts, 0, cells * sizeof(unsigned int), h->stream);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(stage_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 STAGE_MAX_WINDOWS * (int)sizeof(unsigned int));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(stage_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 STAGE_WIN * (int)sizeof(double));
+    if (e == cudaSuccess) {
+        stage_hist_kernel<<<dim3(STAGE_HIST_BLOCKS, STAGE_BANDS), 1024, (size_t)windows * sizeof(unsigned int),
+                            h->stream>>>(g.col, g.nnz, band_arcs, hot, (int)windows, counts);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(cnt.data(), counts, cells * sizeof(unsigned int), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) {
+        dfree(h, counts);
+        return e;
+    }
+    int64_t places = 0;
+    for (size_t q = 0; q < cells; ++q) {
+        first[q] = (unsigned int)places;
+        places += ((int64_t)cnt[q] + STAGE_ALIGN - 1) / STAGE_ALIGN * STAGE_ALIGN;
+    }
+    first[cells] = (unsigned int)places;
+    if (places == 0 || places + STAGE_HOT > 0xffffffffll) {
+        dfree(h, counts);
+        return cudaSuccess;
+    }
+    std::vector<StageItem> items;
+    for (int64_t w = 0; w < windows; ++w) {
+        int64_t arcs = 0;
+        int band0 = 0;
+        for (int band = 0; band < STAGE_BANDS; ++band) {
+            arcs += cnt[(size_t)band * windows + w];
+            if (arcs >= STAGE_CHUNK || band + 1 == STAGE_BANDS) {
+                if (arcs > 0) items.push_back(StageItem{(int32_t)w, band0, band + 1});
+                arcs = 0;
+                band0 = band + 1;
+            }
+        }
+    }
+    // at most a quarter of the memory left, the library's own free blocks
+    // included: a ranking's buffers and the caller's work come first
+    size_t free_b = 0, total_b = 0;
+    unsigned long long reserved = 0, used = 0;
+    const cudaMemPool_t pool = library_pool(h->dev);
+    if ((e = cudaMemGetInfo(&free_b, &total_b)) == cudaSuccess &&
+        (e = cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved)) == cudaSuccess)
+        e = cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used);
+    const double need = 4.0 * (double)g.nnz + 10.0 * (double)places + 4.0 * (double)cells;
+    if (e != cudaSuccess || need > 0.25 * ((double)free_b + (double)(reserved - used))) {
+        dfree(h, counts);
+        return e;
+    }
+    StageMap& m = g.stage;
+    if ((e = dmalloc(h, &m.src, (size_t)g.nnz)) == cudaSuccess &&
+        (e = dmalloc(h, &m.local, (size_t)places)) == cudaSuccess &&
+        (e = dmalloc(h, (double**)&m.y, (size_t)places)) == cudaSuccess &&
+        (e = dmalloc(h, &m.first, cells + 1)) == cudaSuccess)
+        e = dmalloc(h, &m.items, items.size());
+    if (e != cudaSuccess) {  // no memory: plain gathers
+        cudaGetLastError();
+        dfree(h, counts);
+        stage_free(h);
+        return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    }
+    e = cudaMemcpyAsync(m.first, first.data(), (cells + 1) * sizeof(unsigned int), cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(counts, m.first, cells * sizeof(unsigned int), cudaMemcpyDeviceToDevice, h->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m.items, items.data(), items.size() * sizeof(StageItem), cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m.local, 0, (size_t)places * sizeof(uint16_t), h->stream);
+    if (e == cudaSuccess) {
+        stage_assign_kernel<<<(unsigned)((g.nnz + STAGE_ASSIGN - 1) / STAGE_ASSIGN), 256, 0, h->stream>>>(
+            g.col, g.nnz, band_arcs, hot, (int)windows, counts, m.src, m.local);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // the host arrays above are in use until here
+    dfree(h, counts);
+    if (e != cudaSuccess) {
+        stage_free(h);
+        return e;
+    }
+    m.n_items = (int32_t)items.size();
+    m.windows = (int32_t)windows;
+    m.hot = hot;
+    return cudaSuccess;
+}
+
+}  // namespace katz
