@@ -10,10 +10,17 @@
 // degree, so the lanes that share a row (or the rows that share a warp) carry
 // equal work, and no lane waits on a merge search or a block barrier:
 //   THREAD  deg <= 16         one thread per row
-//   OCTET   16 < deg <= 128   eight lanes per row
-//   WARP    128 < deg <= 2048 one warp per row
+//   OCTET   16 < deg <= 128   eight lanes per row (FP64 levels: four)
+//   WARP    128 < deg <= 2048 one warp per row (FP64 levels: half a warp)
 //   CHUNK   deg > 2048        one warp per 2048-arc chunk; spmv_chunk_fixup adds
 //                             a row's chunk sums as a pairwise tree and finishes it
+// The exact sums of FP64 levels do not depend on the split, and merging the
+// lanes' accumulators, rounding and the epilogue cost as much as 30 arcs: with
+// half the lanes a warp pays for them once per two (WARP) or eight (OCTET)
+// rows.  R-MAT22, per level: WARP rows 162 -> 138 us, OCTET 110 -> 99; two lanes
+// per OCTET row or eight per WARP row gain nothing more.  FP32 levels keep their
+// lanes: the split sets the order of their sums, and longer chains of FP32
+// additions would widen the error bound.
 // The walk vector is gathered with read-only loads (one L2 request per arc:
 // this access, not HBM bandwidth, bounds the kernel on power-law graphs).
 //
@@ -54,6 +61,10 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int BLOCK = 256;
 constexpr int WARPS = BLOCK / 32;
+constexpr int OCTET_LANES = 4;   // lanes per OCTET row of an FP64 level (FP32: 8)
+constexpr int WARP_LANES = 16;   // lanes per WARP row of an FP64 level (FP32: 32)
+constexpr int OCTET_ROWS = BLOCK / OCTET_LANES;  // rows per block; FP32 levels take two passes
+constexpr int WARP_ROWS = BLOCK / WARP_LANES;
 
 struct Epi {
     void* y;          // level r slot (double or float)
@@ -356,7 +367,7 @@ __device__ __forceinline__ void xacc_merge(XAcc& a, XAcc b) {
     add128(a, b.w0, b.w1, b.w2, b.w3);
 }
 
-// Sum over groups of `width` lanes (8 or 32): every lane aligns to the
+// Sum over groups of `width` lanes (4 to 32): every lane aligns to the
 // group's largest exponent, then the aligned integers meet in a shuffle tree.
 template <int width>
 __device__ __forceinline__ XAcc xacc_group_sum(XAcc a) {
@@ -515,18 +526,19 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
             if (u < L.n) finish_row<double>(u, xacc_to_double(strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], 0, 1)), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
-            const int64_t u = L.row_octet + (b - L.blk_octet) * (BLOCK / 8) + (tid >> 3);
-            const int sub = tid & 7;
+            const int64_t u = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + tid / OCTET_LANES;
+            const int sub = tid % OCTET_LANES;
             XAcc s = xacc_zero();
-            if (u < L.row_thread) s = strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
-            s = xacc_group_sum<8>(s);
+            if (u < L.row_thread) s = strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], sub, OCTET_LANES);
+            s = xacc_group_sum<OCTET_LANES>(s);
             if (sub == 0 && u < L.row_thread) finish_row<double>(u, xacc_to_double(s), ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARPS + wid;
+            const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
+            const int sub = tid % WARP_LANES;
             XAcc s = xacc_zero();
-            if (u < L.row_octet) s = strided_xsum<8>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
-            s = xacc_group_sum<32>(s);
-            if (lane == 0 && u < L.row_octet) finish_row<double>(u, xacc_to_double(s), ep, p);
+            if (u < L.row_octet) s = strided_xsum<8>(col, x, rowptr[u], rowptr[u + 1], sub, WARP_LANES);
+            s = xacc_group_sum<WARP_LANES>(s);
+            if (sub == 0 && u < L.row_octet) finish_row<double>(u, xacc_to_double(s), ep, p);
         } else {  // CHUNK rows: one warp per chunk of CHUNK_ARCS arcs
             const int64_t ch = b * WARPS + wid;
             XAcc s = xacc_zero();
@@ -545,20 +557,24 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
             if (u < L.n) finish_row<Acc>(u, strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], 0, 1), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
-            const int64_t u = L.row_octet + (b - L.blk_octet) * (BLOCK / 8) + (tid >> 3);
             const int sub = tid & 7;
-            Acc s = (Acc)0;
-            if (u < L.row_thread) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
+            const int64_t u0 = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + (tid >> 3);
+            for (int64_t u = u0; u < u0 + OCTET_ROWS; u += BLOCK / 8) {
+                Acc s = (Acc)0;
+                if (u < L.row_thread) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
 #pragma unroll
-            for (int off = 4; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off, 8));
-            if (sub == 0 && u < L.row_thread) finish_row<Acc>(u, s, ep, p);
+                for (int off = 4; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off, 8));
+                if (sub == 0 && u < L.row_thread) finish_row<Acc>(u, s, ep, p);
+            }
         } else if (b >= L.blk_warp) {  // WARP rows
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARPS + wid;
-            Acc s = (Acc)0;
-            if (u < L.row_octet) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
+            const int64_t u0 = L.row_warp + (b - L.blk_warp) * WARP_ROWS + wid;
+            for (int64_t u = u0; u < u0 + WARP_ROWS; u += WARPS) {
+                Acc s = (Acc)0;
+                if (u < L.row_octet) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
 #pragma unroll
-            for (int off = 16; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off));
-            if (lane == 0 && u < L.row_octet) finish_row<Acc>(u, s, ep, p);
+                for (int off = 16; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off));
+                if (lane == 0 && u < L.row_octet) finish_row<Acc>(u, s, ep, p);
+            }
         } else {  // CHUNK rows: one warp per chunk of CHUNK_ARCS arcs
             const int64_t ch = b * WARPS + wid;
             Acc s = (Acc)0;
@@ -1062,22 +1078,23 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
                 store_pair64(y, t_out, u, sa, sb, alpha);
             }
         } else if (b >= L.blk_octet) {
-            const int64_t u = L.row_octet + (b - L.blk_octet) * (BLOCK / 8) + (tid >> 3);
-            const int sub = tid & 7;
+            const int64_t u = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + tid / OCTET_LANES;
+            const int sub = tid % OCTET_LANES;
             sa = xacc_zero();
             sb = xacc_zero();
-            if (u < L.row_thread) strided_xsum2<4>(col, x, rowptr[u], rowptr[u + 1], sub, 8, sa, sb);
-            sa = xacc_group_sum<8>(sa);
-            sb = xacc_group_sum<8>(sb);
+            if (u < L.row_thread) strided_xsum2<4>(col, x, rowptr[u], rowptr[u + 1], sub, OCTET_LANES, sa, sb);
+            sa = xacc_group_sum<OCTET_LANES>(sa);
+            sb = xacc_group_sum<OCTET_LANES>(sb);
             if (sub == 0 && u < L.row_thread) store_pair64(y, t_out, u, sa, sb, alpha);
         } else if (b >= L.blk_warp) {
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARPS + wid;
+            const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
+            const int sub = tid % WARP_LANES;
             sa = xacc_zero();
             sb = xacc_zero();
-            if (u < L.row_octet) strided_xsum2<8>(col, x, rowptr[u], rowptr[u + 1], lane, 32, sa, sb);
-            sa = xacc_group_sum<32>(sa);
-            sb = xacc_group_sum<32>(sb);
-            if (lane == 0 && u < L.row_octet) store_pair64(y, t_out, u, sa, sb, alpha);
+            if (u < L.row_octet) strided_xsum2<8>(col, x, rowptr[u], rowptr[u + 1], sub, WARP_LANES, sa, sb);
+            sa = xacc_group_sum<WARP_LANES>(sa);
+            sb = xacc_group_sum<WARP_LANES>(sb);
+            if (sub == 0 && u < L.row_octet) store_pair64(y, t_out, u, sa, sb, alpha);
         } else {
             const int64_t ch = b * WARPS + wid;
             sa = xacc_zero();
@@ -1106,18 +1123,26 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
                 y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
             }
         } else if (b >= L.blk_octet) {
-            const int64_t u = L.row_octet + (b - L.blk_octet) * (BLOCK / 8) + (tid >> 3);
             const int sub = tid & 7;
-            if (u < L.row_thread) strided_sum2(col, x, rowptr[u], rowptr[u + 1], sub, 8, sa, sb);
-            sa = fsum_group<8>(sa);
-            sb = fsum_group<8>(sb);
-            if (sub == 0 && u < L.row_thread) y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
+            const int64_t u0 = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + (tid >> 3);
+            for (int64_t u = u0; u < u0 + OCTET_ROWS; u += BLOCK / 8) {
+                sa = 0.0f;
+                sb = 0.0f;
+                if (u < L.row_thread) strided_sum2(col, x, rowptr[u], rowptr[u + 1], sub, 8, sa, sb);
+                sa = fsum_group<8>(sa);
+                sb = fsum_group<8>(sb);
+                if (sub == 0 && u < L.row_thread) y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
+            }
         } else if (b >= L.blk_warp) {
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARPS + wid;
-            if (u < L.row_octet) strided_sum2(col, x, rowptr[u], rowptr[u + 1], lane, 32, sa, sb);
-            sa = fsum_group<32>(sa);
-            sb = fsum_group<32>(sb);
-            if (lane == 0 && u < L.row_octet) y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
+            const int64_t u0 = L.row_warp + (b - L.blk_warp) * WARP_ROWS + wid;
+            for (int64_t u = u0; u < u0 + WARP_ROWS; u += WARPS) {
+                sa = 0.0f;
+                sb = 0.0f;
+                if (u < L.row_octet) strided_sum2(col, x, rowptr[u], rowptr[u + 1], lane, 32, sa, sb);
+                sa = fsum_group<32>(sa);
+                sb = fsum_group<32>(sb);
+                if (lane == 0 && u < L.row_octet) y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
+            }
         } else {
             const int64_t ch = b * WARPS + wid;
             if (ch < L.chunks) {
@@ -1394,8 +1419,8 @@ SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t r
     L.row_thread = row_thread;
     L.chunks = chunks;
     const int64_t bc = (chunks + WARPS - 1) / WARPS;
-    const int64_t bw = (row_octet - row_warp + WARPS - 1) / WARPS;
-    const int64_t bo = (row_thread - row_octet + BLOCK / 8 - 1) / (BLOCK / 8);
+    const int64_t bw = (row_octet - row_warp + WARP_ROWS - 1) / WARP_ROWS;
+    const int64_t bo = (row_thread - row_octet + OCTET_ROWS - 1) / OCTET_ROWS;
     const int64_t bt = (n - row_thread + BLOCK - 1) / BLOCK;
     L.blk_warp = bc;
     L.blk_octet = bc + bw;

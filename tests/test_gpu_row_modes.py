@@ -1,0 +1,72 @@
+"""Row sums at the edges of the row modes (degrees 16/17, 128/129, 2048/2049)
+and of the blocks that share rows, FP64 and FP32 levels, one state and two.
+
+FP64: s_2 = alpha (A s_1), s_1 = alpha deg, against exact integer sums;
+tolerance 1e-15 (three roundings of 2^-53 each side).  FP32 level 2: the
+longest chain of FP32 additions here is below 24, plus the rounding of the
+inputs, of alpha and of the product: 27 x 2^-24 < 2e-6.
+"""
+import numpy as np
+import pytest
+import torch
+
+import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(counts, seed):
+    """Rows of the given {degree: count}, their neighbours random leaves."""
+    rng = np.random.default_rng(seed)
+    deg = np.repeat(list(counts), list(counts.values()))
+    rng.shuffle(deg)
+    m, leaves = len(deg), 6000
+    u = np.repeat(np.arange(m), deg)
+    v = np.concatenate([m + rng.choice(leaves, d, replace=False) for d in deg])
+    return gg.from_edges(m + leaves, u, v)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("counts", [
+    {1: 3, 15: 5, 16: 300, 17: 64, 18: 1}, {17: 65, 32: 7, 33: 70, 127: 3, 128: 129, 129: 15},
+    {129: 17, 130: 1, 255: 16, 256: 33}, {2047: 2, 2048: 17, 2049: 3, 4096: 2, 4097: 1}, {5999: 1}])
+def test_row_sums_at_the_mode_edges(counts, precision):
+    import paper_1807_03847_gb300 as K
+
+    g = _graph(counts, 3)
+    h = K.Katz(torch.from_numpy(g.rowptr).cuda(), torch.from_numpy(g.col).cuda(),
+               K.katz_default_opts(r_max=2, precision=precision, fp32_from=2 if precision else 0))
+    h.rank(0.0, 1, 1e-300, check=False)
+    deg = np.diff(g.rowptr)
+    two = np.zeros(g.n, np.int64)
+    np.add.at(two, np.repeat(np.arange(g.n), deg), deg[g.col])
+    a = 1.0 / (deg.max() + 1)
+    np.testing.assert_allclose(h.walk(2), a * a * two, rtol=2e-6 if precision else 1e-15)
+    h.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_two_states_at_the_mode_edges(precision):
+    import paper_1807_03847_gb300 as K
+
+    g = _graph({16: 70, 17: 66, 128: 33, 129: 18, 2048: 5, 2049: 3}, 4)
+    D = g.deg_max() + 8
+    opts = dict(keep_history=1, deg_bound=D, precision=precision)
+    first = gg.update_batch(g, 40, 1)
+    batches = [first, gg.update_batch(gg.apply_batch(g, *first), 40, 2)]
+    walks = []
+    for pair in (0, 2):
+        h = K.Katz(g.rowptr, g.col, K.katz_default_opts(**opts))
+        h.rank(0.0, 20, 1e-9)
+        s = K.Server(workers=1, pair_batches=pair)
+        s.attach(h, 20)
+        answers = [s.wait(t) for t in [s.submit(h, *b) for b in batches]]
+        s.close()
+        assert all(a[0] == 0 for a in answers)
+        r = answers[-1][2].info.r
+        walks.append([h.walk(i) for i in range(1, r + 1)] + [np.concatenate([a[1] for a in answers])])
+        h.close()
+    assert len(walks[0]) == len(walks[1])
+    for x, y in zip(*walks):
+        assert np.array_equal(x, y)  # the pass over two states has the bits of one by one
+
