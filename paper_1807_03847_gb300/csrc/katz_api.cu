@@ -603,7 +603,7 @@ void katz_destroy(katz_h h) {
                           (void*)d.err, (void*)d.delta, (void*)d.ins_cnt, (void*)d.cursor, (void*)d.touched,
                           (void*)d.ins_start, (void*)d.ins_rows, (void*)d.n_ins_rows, (void*)d.bucket,
                           (void*)d.vbits, (void*)d.frontier, (void*)d.fsize, (void*)h->rrowptr, (void*)h->rcol,
-                          (void*)d.hub_keep})
+                          (void*)d.hub_keep, (void*)d.hub_bits})
             dfree(h, ptr);
         dfree(h, h->col_spare);
         dfree(h, h->rp_new);
@@ -1332,16 +1332,20 @@ katz_status update_prepare(katz_handle* h, const int32_t* src, const int32_t* ds
     const bool hubs = g.layout.row_warp > 0;
     if (hubs && g.layout.chunks > d.hub_keep_cap) {
         dfree_on(h->dyn.hub_keep, sa);
+        dfree_on(h->dyn.hub_bits, sa);
         h->dyn.hub_keep = nullptr;
+        h->dyn.hub_bits = nullptr;
         h->dyn.hub_keep_cap = 0;
         const int64_t cap = g.layout.chunks + g.layout.chunks / 8 + 64;
-        if ((e = dmalloc_on(h, &h->dyn.hub_keep, (size_t)cap, sa)) != cudaSuccess) {
+        if ((e = dmalloc_on(h, &h->dyn.hub_keep, (size_t)cap, sa)) != cudaSuccess ||
+            (e = dmalloc_on(h, &h->dyn.hub_bits, (size_t)cap * (CHUNK_ARCS / 32), sa)) != cudaSuccess) {
             dyn_clear(g, d, m, sa);
             cudaStreamSynchronize(sa);
             return cuda_done(e, "cudaMalloc hub chunks");
         }
         h->dyn.hub_keep_cap = cap;
         d.hub_keep = h->dyn.hub_keep;
+        d.hub_bits = h->dyn.hub_bits;
         d.hub_keep_cap = cap;
     }
     if ((e = dyn_rebuild(g, d, m, h->rp_new, h->col_spare, promote ? (void*)h->rp64_next : h->rowptr_spare, promote,
@@ -1481,8 +1485,11 @@ static katz_status repair_levels(katz_handle* h, int64_t& full_levels, int64_t& 
     all_rows = false;
     if (pd.applied) {
         // directed: the reverse BFS walks in-arcs, from the transposed CSR of
-        // the updated graph
-        if (!d.undirected) {
+        // the updated graph, built when the first expansion needs it (a batch
+        // whose levels go full at once expands nothing)
+        bool transposed = d.undirected;
+        auto transpose = [&]() -> katz_status {
+            transposed = true;
             if (!h->rrowptr && (e = dmalloc(h, &h->rrowptr, (size_t)n + 1)) != cudaSuccess)
                 return cuda_fail(h, e, "cudaMalloc transposed offsets");
             if (!h->t_cnt && ((e = dmalloc(h, &h->t_cnt, (size_t)n + 1)) != cudaSuccess ||
@@ -1503,7 +1510,8 @@ static katz_status repair_levels(katz_handle* h, int64_t& full_levels, int64_t& 
             if ((e = dyn_transpose(g, d, h->t_cnt, h->t_sums, h->stream)) != cudaSuccess)
                 return cuda_fail(h, e, "transpose");
             h->launches += 3 + (g.nnz > 0 ? 1 + (g.n > g.layout.row_warp ? 1 : 0) + (g.layout.chunks > 0 ? 1 : 0) : 0);
-        }
+            return KATZ_OK;
+        };
         // ---- repair s_1..s_r: affected rows only, or whole levels once the
         //      affected set is large (Sec. 4) ------------------------------------------
         if ((e = dyn_seed(g, d, m, h->stream)) != cudaSuccess) return cuda_fail(h, e, "seed frontier");
@@ -1546,6 +1554,10 @@ static katz_status repair_levels(katz_handle* h, int64_t& full_levels, int64_t& 
                     continue;
                 }
                 vol_lo = fs[1];
+                if (!transposed) {
+                    const katz_status st = transpose();
+                    if (st != KATZ_OK) return st;
+                }
                 if ((e = dyn_expand(g, d, lo, hi, i, h->stream)) != cudaSuccess) return cuda_fail(h, e, "expand");
                 h->launches += hi > lo ? 1 + (d.undirected && g.layout.chunks > 0 ? 1 : 0) : 0;
                 if ((e = cudaMemcpyAsync(fs, d.fsize, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,

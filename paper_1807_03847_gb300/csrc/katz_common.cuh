@@ -264,6 +264,7 @@ struct DynBuffers {
     unsigned long long* fsize = nullptr;  // [2] frontier size, sum of the frontier's degrees
     int32_t* hub_epoch = nullptr;    // [row_warp] level at which a CHUNK row joined the frontier
     int64_t* hub_keep = nullptr;     // [hub_keep_cap >= chunks] kept arcs, then place, of each hub chunk
+    unsigned* hub_bits = nullptr;    // [hub_keep_cap * CHUNK_ARCS / 32] which arcs of each hub chunk stay
     int64_t hub_keep_cap = 0;
     int64_t* rrowptr = nullptr;      // [n+1] directed: transposed CSR (in-arcs) of the current graph
     int32_t* rcol = nullptr;         // [rcap]

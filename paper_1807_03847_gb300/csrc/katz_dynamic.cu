@@ -41,18 +41,24 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     return z ^ (z >> 31);
 }
 
-// position of `target` in row u (first match), -1 if absent; one warp
+// whether `target` is in row u; one warp, eight loads in flight per lane (a
+// batch's longest rows set its time: 66 us per batch of R-MAT20 with one load
+// at a time, 13 us so)
 template <typename Off>
-__device__ __forceinline__ int64_t find_in_row(const Off* rowptr, const int32_t* col, int64_t u, int32_t target) {
-    const int lane = threadIdx.x & 31;
-    const int64_t a = rowptr[u], b = rowptr[u + 1];
-    for (int64_t base = a; base < b; base += 32) {
-        const int64_t j = base + lane;
-        const bool hit = j < b && col[j] == target;
-        const unsigned m = __ballot_sync(FULL, hit);
-        if (m) return base + (__ffs(m) - 1);
+__device__ __forceinline__ bool find_in_row(const Off* rowptr, const int32_t* col, int64_t u, int32_t target) {
+    constexpr int U = 8;
+    const int32_t* __restrict__ cp = col + (int64_t)rowptr[u] + (threadIdx.x & 31);
+    for (int left = (int)((int64_t)rowptr[u + 1] - (int64_t)rowptr[u]) - (int)(threadIdx.x & 31);
+         __any_sync(FULL, left > 0); left -= U * 32, cp += U * 32) {
+        int32_t x[U];
+        bool hit = false;
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = left > q * 32 ? cp[q * 32] : -1;
+#pragma unroll
+        for (int q = 0; q < U; ++q) hit |= x[q] == target;
+        if (__any_sync(FULL, hit)) return true;
     }
-    return -1;
+    return false;
 }
 
 constexpr unsigned long long DEL_BIT = 1ull << 63;
@@ -64,17 +70,31 @@ __device__ __forceinline__ unsigned long long pair_key(int32_t u, int32_t v, boo
     return (((unsigned long long)(uint32_t)a << 32) | (uint32_t)b) + 1ull;
 }
 
-// the stored entry of `key` (with its delete bit), 0 if absent
-__device__ __forceinline__ unsigned long long table_find(const unsigned long long* __restrict__ table, int64_t mask,
-                                                         unsigned long long key) {
-    int64_t h = (int64_t)(mix64(key) & (unsigned long long)mask);
-    for (int64_t probe = 0; probe <= mask; ++probe) {
-        const unsigned long long t = table[h];
-        if (t == 0ull) return 0ull;
-        if ((t & ~DEL_BIT) == key) return t;
-        h = (h + 1) & mask;
+constexpr int KEEP_U = 4;  // arcs per lane looked up at once
+
+// which of the row's arcs x[q] (entries < 0: none) stay, as one ballot per q:
+// an arc goes if the batch deletes it.  The first probes of all KEEP_U keys are
+// in flight together (a chain of one load per arc left the warps waiting).
+__device__ __forceinline__ void keep_ballots(const int32_t (&x)[KEEP_U], int32_t u,
+                                             const unsigned long long* __restrict__ table, int64_t mask, bool und,
+                                             unsigned (&kb)[KEEP_U]) {
+    unsigned long long key[KEEP_U], t[KEEP_U];
+    int64_t h[KEEP_U];
+#pragma unroll
+    for (int q = 0; q < KEEP_U; ++q) {
+        key[q] = pair_key(u, x[q], und);
+        h[q] = (int64_t)(mix64(key[q]) & (unsigned long long)mask);
+        t[q] = x[q] >= 0 ? table[h[q]] : 0ull;
     }
-    return 0ull;
+#pragma unroll
+    for (int q = 0; q < KEEP_U; ++q) {
+        for (int64_t probe = 0; probe < mask && t[q] != 0ull && (t[q] & ~DEL_BIT) != key[q]; ++probe) {
+            h[q] = (h[q] + 1) & mask;
+            t[q] = table[h[q]];
+        }
+        const bool gone = (t[q] & ~DEL_BIT) == key[q] && (t[q] & DEL_BIT);
+        kb[q] = __ballot_sync(FULL, x[q] >= 0 && !gone);
+    }
 }
 
 // out[j - a] = col[j] for j in [a, b): one warp, eight loads in flight per
@@ -129,10 +149,10 @@ __global__ void validate_batch_kernel(const Off* __restrict__ rowptr, const int3
         }
         const int64_t da = (int64_t)rowptr[ua + 1] - (int64_t)rowptr[ua];
         const int64_t db = (int64_t)rowptr[ub + 1] - (int64_t)rowptr[ub];
-        const int64_t pos =
+        const bool present =
             (!und || da <= db) ? find_in_row(rowptr, col, ua, ub) : find_in_row(rowptr, col, ub, ua);
         if (lane == 0) {
-            if (ins[e] ? pos >= 0 : pos < 0) atomicOr(err, DYN_E_INVAL);
+            if (present == (ins[e] != 0)) atomicOr(err, DYN_E_INVAL);
             const int d = ins[e] ? 1 : -1;
             atomicAdd(&delta[ua], d);
             touched[ua] = 1;
@@ -279,32 +299,53 @@ __device__ __forceinline__ void rebuild_touched_row(const Off* __restrict__ rowp
         warp_copy(col, a, b, col_new + o);
         o += b - a;
     }
-    for (int64_t base = a; !no_deletes && base < b; base += 32) {
-        const int64_t j = base + lane;
-        const int32_t x = j < b ? col[j] : -1;
-        const bool keep = x >= 0 && !(table_find(table, mask, pair_key((int32_t)v, x, und)) & DEL_BIT);
-        const unsigned kb = __ballot_sync(FULL, keep);
-        if (keep) col_new[o + __popc(kb & ((1u << lane) - 1u))] = x;
-        o += __popc(kb);
+    for (int64_t base = a; !no_deletes && base < b; base += 32 * KEEP_U) {
+        int32_t x[KEEP_U];
+        unsigned kb[KEEP_U];
+#pragma unroll
+        for (int q = 0; q < KEEP_U; ++q) x[q] = base + q * 32 + lane < b ? col[base + q * 32 + lane] : -1;
+        keep_ballots(x, (int32_t)v, table, mask, und, kb);
+#pragma unroll
+        for (int q = 0; q < KEEP_U; ++q) {
+            if ((kb[q] >> lane) & 1u) col_new[o + __popc(kb[q] & ((1u << lane) - 1u))] = x[q];
+            o += __popc(kb[q]);
+        }
     }
     const int c = ins_cnt[v];
     const int32_t* bkt = bucket + ins_start[v];
     for (int q = lane; q < c; q += 32) col_new[o + q] = bkt[q];
 }
 
-// rows from row_lo on (no CHUNK rows): one warp per 32 consecutive rows; a
-// run without touched rows is one contiguous copy
+// rows from row_warp on (no CHUNK rows): one warp per group of consecutive
+// rows, 2 WARP rows, 16 OCTET rows or 32 THREAD rows, so that a group holds at
+// most 4096 arcs (a batch may lengthen rows past their mode).  With 32 rows of
+// any mode a few warps copied 64 K arcs each: 170 us per batch of R-MAT20,
+// 47 us so.  A run without touched rows is one contiguous copy.
+constexpr int GROUP_WARP = 2, GROUP_OCTET = 16, GROUP_THREAD = 32;
+
+__host__ __device__ __forceinline__ int64_t groups_of(int64_t rows, int per) { return (rows + per - 1) / per; }
+
 template <typename Off>
 __global__ void rebuild_groups_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
                                       const int64_t* __restrict__ rowptr_new, const uint8_t* __restrict__ touched,
-                                      const int32_t* __restrict__ ins_cnt, const int64_t* __restrict__ ins_start,
-                                      const int32_t* __restrict__ bucket, const unsigned long long* __restrict__ table,
-                                      int64_t mask, bool und, int64_t row_lo, int64_t n, int32_t* col_new) {
+                                      SpmvLayout L, int32_t* col_new) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
-    const int64_t groups = (n - row_lo + 31) / 32;
+    const int64_t gw = groups_of(L.row_octet - L.row_warp, GROUP_WARP);
+    const int64_t go = gw + groups_of(L.row_thread - L.row_octet, GROUP_OCTET);
+    const int64_t groups = go + groups_of(L.n - L.row_thread, GROUP_THREAD);
     for (int64_t gi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; gi < groups; gi += warps) {
-        const int64_t u0 = row_lo + gi * 32, u1 = min(u0 + 32, n);
+        int64_t u0, u1;
+        if (gi < gw) {
+            u0 = L.row_warp + gi * GROUP_WARP;
+            u1 = min(u0 + GROUP_WARP, L.row_octet);
+        } else if (gi < go) {
+            u0 = L.row_octet + (gi - gw) * GROUP_OCTET;
+            u1 = min(u0 + GROUP_OCTET, L.row_thread);
+        } else {
+            u0 = L.row_thread + (gi - go) * GROUP_THREAD;
+            u1 = min(u0 + GROUP_THREAD, L.n);
+        }
         const bool t = u0 + lane < u1 && touched[u0 + lane];
         const unsigned tb = __ballot_sync(FULL, t);
         // the runs of untouched rows between touched ones, each one copy
@@ -370,8 +411,8 @@ __global__ void rebuild_chunks_kernel(const Off* __restrict__ rowptr, const int3
     }
 }
 
-// Touched CHUNK rows, compacted chunk by chunk: (A) one warp per chunk counts
-// the arcs it keeps, (B) one warp per row turns the counts into the chunks'
+// Touched CHUNK rows, compacted chunk by chunk: (A) one warp per chunk looks
+// its arcs up among the deleted ones and counts those it keeps, (B) one warp per row turns the counts into the chunks'
 // places in the new row and appends the inserted arcs after them, (C) one
 // warp per chunk writes its kept arcs, in order, at its place.
 template <typename Off>
@@ -383,12 +424,15 @@ __device__ __forceinline__ void hub_chunk_range(const Off* __restrict__ rowptr, 
     j1 = min(j0 + (int64_t)CHUNK_ARCS, (int64_t)rowptr[u + 1]);
 }
 
+constexpr int KEEP_WORDS = CHUNK_ARCS / 32;  // ballots per chunk
+
+// the ballots stay in bits for (C), which looks nothing up again
 template <typename Off>
 __global__ void hub_keep_count_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
                                       const uint8_t* __restrict__ touched, const int32_t* __restrict__ chunk_row,
                                       const int64_t* __restrict__ chunk_first, int64_t chunks,
                                       const unsigned long long* __restrict__ table, int64_t mask, bool und,
-                                      int64_t* keep) {
+                                      int64_t* keep, unsigned* __restrict__ bits) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
     for (int64_t ch = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; ch < chunks; ch += warps) {
@@ -396,11 +440,17 @@ __global__ void hub_keep_count_kernel(const Off* __restrict__ rowptr, const int3
         hub_chunk_range(rowptr, chunk_row, chunk_first, ch, u, j0, j1);
         if (!touched[u]) continue;
         int64_t cnt = 0;
-        for (int64_t base = j0; base < j1; base += 32) {
-            const int64_t j = base + lane;
-            const int32_t x = j < j1 ? col[j] : -1;
-            const bool k = x >= 0 && !(table_find(table, mask, pair_key((int32_t)u, x, und)) & DEL_BIT);
-            cnt += __popc(__ballot_sync(FULL, k));
+        for (int64_t base = j0; base < j1; base += 32 * KEEP_U) {
+            int32_t x[KEEP_U];
+            unsigned kb[KEEP_U];
+#pragma unroll
+            for (int q = 0; q < KEEP_U; ++q) x[q] = base + q * 32 + lane < j1 ? col[base + q * 32 + lane] : -1;
+            keep_ballots(x, (int32_t)u, table, mask, und, kb);
+#pragma unroll
+            for (int q = 0; q < KEEP_U; ++q) {
+                cnt += __popc(kb[q]);
+                if (lane == q) bits[ch * KEEP_WORDS + (base - j0) / 32 + q] = kb[q];
+            }
         }
         if (lane == 0) keep[ch] = cnt;
     }
@@ -438,8 +488,8 @@ template <typename Off>
 __global__ void hub_keep_write_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
                                       const uint8_t* __restrict__ touched, const int32_t* __restrict__ chunk_row,
                                       const int64_t* __restrict__ chunk_first, int64_t chunks,
-                                      const unsigned long long* __restrict__ table, int64_t mask, bool und,
-                                      const int64_t* __restrict__ place, int32_t* col_new) {
+                                      const unsigned* __restrict__ bits, const int64_t* __restrict__ place,
+                                      int32_t* col_new) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
     for (int64_t ch = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; ch < chunks; ch += warps) {
@@ -447,13 +497,21 @@ __global__ void hub_keep_write_kernel(const Off* __restrict__ rowptr, const int3
         hub_chunk_range(rowptr, chunk_row, chunk_first, ch, u, j0, j1);
         if (!touched[u]) continue;
         int64_t o = place[ch];
-        for (int64_t base = j0; base < j1; base += 32) {
-            const int64_t j = base + lane;
-            const int32_t x = j < j1 ? col[j] : -1;
-            const bool k = x >= 0 && !(table_find(table, mask, pair_key((int32_t)u, x, und)) & DEL_BIT);
-            const unsigned kb = __ballot_sync(FULL, k);
-            if (k) col_new[o + __popc(kb & ((1u << lane) - 1u))] = x;
-            o += __popc(kb);
+        constexpr int U = 8;
+        for (int64_t base = j0; base < j1; base += 32 * U) {
+            int32_t x[U];
+            unsigned kb[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                const int64_t j = base + q * 32;
+                x[q] = j + lane < j1 ? col[j + lane] : -1;
+                kb[q] = j < j1 ? bits[ch * KEEP_WORDS + (j - j0) / 32] : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                if ((kb[q] >> lane) & 1u) col_new[o + __popc(kb[q] & ((1u << lane) - 1u))] = x[q];
+                o += __popc(kb[q]);
+            }
         }
     }
 }
@@ -787,11 +845,12 @@ static void rebuild_launch(const DeviceGraph& g, const DynBuffers& d, int64_t m,
                            int32_t* col_new, cudaStream_t st) {
     const Off* rp = (const Off*)g.rowptr;
     const SpmvLayout& L = g.layout;
-    const int64_t groups = (g.n - L.row_warp + 31) / 32;
+    const int64_t groups = groups_of(L.row_octet - L.row_warp, GROUP_WARP) +
+                           groups_of(L.row_thread - L.row_octet, GROUP_OCTET) +
+                           groups_of(L.n - L.row_thread, GROUP_THREAD);
     if (groups > 0) {
-        rebuild_groups_kernel<Off><<<grid_for(groups * 32, 256), 256, 0, st>>>(
-            rp, g.col, rowptr_new, d.touched, d.ins_cnt, d.ins_start, d.bucket, d.table, d.table_mask, d.undirected,
-            L.row_warp, g.n, col_new);
+        rebuild_groups_kernel<Off><<<grid_for(groups * 32, 256), 256, 0, st>>>(rp, g.col, rowptr_new, d.touched, L,
+                                                                               col_new);
         rebuild_touched_kernel<Off><<<grid_for(m * 32, 256), 256, 0, st>>>(
             rp, g.col, rowptr_new, g.inv, d.src, d.dst, m, d.undirected, L.row_warp, d.touched, d.ins_cnt, d.delta,
             d.ins_start, d.bucket, d.table, d.table_mask, col_new);
@@ -802,12 +861,11 @@ static void rebuild_launch(const DeviceGraph& g, const DynBuffers& d, int64_t m,
     if (L.row_warp > 0) {
         hub_keep_count_kernel<Off><<<grid_for(L.chunks * 32, 256), 256, 0, st>>>(
             rp, g.col, d.touched, g.chunk_row, g.chunk_first, L.chunks, d.table, d.table_mask, d.undirected,
-            d.hub_keep);
+            d.hub_keep, d.hub_bits);
         hub_keep_scan_kernel<Off><<<grid_for(L.row_warp * 32, 256), 256, 0, st>>>(
             d.touched, g.chunk_first, rowptr_new, d.ins_cnt, d.ins_start, d.bucket, L.row_warp, d.hub_keep, col_new);
         hub_keep_write_kernel<Off><<<grid_for(L.chunks * 32, 256), 256, 0, st>>>(
-            rp, g.col, d.touched, g.chunk_row, g.chunk_first, L.chunks, d.table, d.table_mask, d.undirected,
-            d.hub_keep, col_new);
+            rp, g.col, d.touched, g.chunk_row, g.chunk_first, L.chunks, d.hub_bits, d.hub_keep, col_new);
     }
 }
 

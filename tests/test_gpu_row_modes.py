@@ -70,3 +70,44 @@ def test_two_states_at_the_mode_edges(precision):
     for x, y in zip(*walks):
         assert np.array_equal(x, y)  # the pass over two states has the bits of one by one
 
+
+
+@pytest.mark.parametrize("seed,kinds", [(1, "delete"), (2, "both"), (3, "both"), (4, "insert")])
+def test_rebuilt_rows_at_the_mode_edges(seed, kinds):
+    """A batch that empties whole stretches of hub rows and touches first and
+    last rows of every mode: the walk vectors are those of a new handle on the
+    updated graph, bit for bit (exact row sums)."""
+    import paper_1807_03847_gb300 as K
+
+    g = _graph({1: 5, 16: 33, 17: 34, 128: 17, 129: 3, 2048: 2, 2049: 2, 4600: 2}, seed)
+    rng = np.random.default_rng(seed)
+    rows = np.repeat(np.arange(g.n), np.diff(g.rowptr))
+    keep = rows < g.col
+    u, v = rows[keep], g.col[keep]
+    hub = int(np.argmax(np.diff(g.rowptr)))
+    chosen = np.zeros(len(u), bool)
+    if kinds != "insert":
+        chosen |= rng.random(len(u)) < 0.05
+        chosen |= (u == hub) & (v > np.median(g.col))  # most of a chunk
+    src, dst = list(u[chosen]), list(v[chosen])
+    ins = [0] * len(src)
+    if kinds != "delete":
+        present = set(zip(u.tolist(), v.tolist()))
+        for a, b in rng.integers(0, g.n, (400, 2)).tolist():
+            a, b = min(a, b), max(a, b)
+            if a != b and (a, b) not in present:
+                present.add((a, b))
+                src.append(a), dst.append(b), ins.append(1)
+    src, dst, ins = np.array(src, np.int32), np.array(dst, np.int32), np.array(ins, np.uint8)
+    D = g.deg_max() + 64
+    opts = dict(keep_history=1, deg_bound=D)
+    h = K.Katz(g.rowptr, g.col, K.katz_default_opts(**opts))
+    h.rank(0.0, 10, 1e-9)
+    info = h.update(src, dst, ins)
+    new = gg.apply_batch(g, src, dst, ins)
+    fresh = K.Katz(new.rowptr, new.col, K.katz_default_opts(r_max=info.r, **opts))
+    fresh.rank(0.0, 10, 1e-300, check=False)
+    for i in range(1, info.r + 1):
+        assert np.array_equal(h.walk(i), fresh.walk(i))
+    h.close()
+    fresh.close()
