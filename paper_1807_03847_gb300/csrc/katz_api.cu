@@ -87,11 +87,15 @@ katz_status init_handle_runtime(katz_handle* h) {
     }
     if ((e = cudaEventCreate(&h->ev0)) != cudaSuccess || (e = cudaEventCreate(&h->ev1)) != cudaSuccess)
         return cuda_fail(h, e, "cudaEventCreate");
-    // one pinned block: the control block, then a small scratch for device-to-host reads
+    // one pinned block: the control block, a small scratch for device-to-host
+    // reads, and the trace (up to H_TRACE levels; a longer one is read pageable)
+    const size_t trace = h->opts.r_max + 2 <= H_TRACE ? (size_t)h->opts.r_max + 2 : 0;
     void* blk = nullptr;
-    if ((e = cudaMallocHost(&blk, CTRL_BYTES + H_SMALL)) != cudaSuccess) return cuda_fail(h, e, "cudaMallocHost");
+    if ((e = cudaMallocHost(&blk, CTRL_BYTES + H_SMALL + trace * sizeof(int64_t))) != cudaSuccess)
+        return cuda_fail(h, e, "cudaMallocHost");
     h->h_ctrl = (Ctrl*)blk;
     h->h_small = (unsigned char*)blk + CTRL_BYTES;
+    h->h_trace = trace ? (int64_t*)(h->h_small + H_SMALL) : nullptr;
     return KATZ_OK;
 }
 
@@ -271,6 +275,34 @@ katz_status ensure_graph(katz_handle* h) {
     return KATZ_OK;
 }
 
+// The control block and the trace as of the work queued so far, and ev1 after
+// that work: one wait.
+katz_status read_state(katz_handle* h) {
+    cudaError_t e;
+    if ((e = cudaEventRecord(h->ev1, h->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
+        return cuda_fail(h, e, "copy ctrl");
+    if (h->h_trace && (e = cudaMemcpyAsync(h->h_trace, h->b.trace, ((size_t)h->opts.r_max + 2) * sizeof(int64_t),
+                                           cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
+        return cuda_fail(h, e, "copy trace");
+    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "iteration");
+    return KATZ_OK;
+}
+
+// |M| of levels 1..r, from the state read last
+katz_status take_trace(katz_handle* h) {
+    const size_t len = (size_t)std::max(0, h->r);
+    if (h->h_trace) {
+        h->trace.assign(h->h_trace + 1, h->h_trace + 1 + len);
+        return KATZ_OK;
+    }
+    h->trace.assign(len, 0);
+    cudaError_t e = cudaMemcpyAsync(h->trace.data(), h->b.trace + 1, len * sizeof(int64_t), cudaMemcpyDeviceToHost,
+                                    h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    return e == cudaSuccess ? KATZ_OK : cuda_fail(h, e, "copy trace");
+}
+
 // Run iterations until the device sets ctrl.stop (converged or r_max).
 // Graph mode: one graph launch runs the whole loop on the device; the host
 // only steps in when the candidate set outgrows the one-CTA select.
@@ -315,9 +347,8 @@ katz_status run_loop(katz_handle* h, int done) {
                 ++launched_iters;
             }
         }
-        if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
-            return cuda_fail(h, e, "copy ctrl");
-        if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "iteration");
+        const katz_status st = read_state(h);
+        if (st != KATZ_OK) return st;
         if (h->h_ctrl->stop) return KATZ_OK;
     }
 }
@@ -403,8 +434,8 @@ katz_status dyn_reserve(katz_handle* h, int64_t m, int64_t nnz_cap, cudaStream_t
         DALLOC(d.fsize, 2);
         DALLOC(d.hub_epoch, std::max<int64_t>(g.layout.row_warp, 1));
         DALLOC(d.n_ins_rows, 1);
-        DALLOC(d.err, 1);
-        DALLOC(d.mode_dmax, 3);
+        DALLOC(d.err, 2);
+        DALLOC(d.mode_dmax, 4);
         DALLOC(h->rp_new, n + 1);
         DALLOC(h->deg_tmp, n + 1);
         DALLOC(h->scan_sums, scan_blocks(n + 1));
@@ -418,12 +449,15 @@ katz_status dyn_reserve(katz_handle* h, int64_t m, int64_t nnz_cap, cudaStream_t
             h->rowptr_spare = rp;
         }
         DALLOC(h->chunk_first_spare, g.layout.row_warp + 1);
-        DALLOC(h->chunk_row_spare, std::max<int64_t>(h->chunk_row_cap, 1));
-        h->chunk_row_spare_cap = std::max<int64_t>(h->chunk_row_cap, 1);
+        const int64_t chunk_cap = h->chunk_row_cap + h->chunk_row_cap / 8 + 16;  // batches may add chunks
+        DALLOC(h->chunk_row_spare, chunk_cap);
+        h->chunk_row_spare_cap = chunk_cap;
         if ((e = cudaMemsetAsync(d.delta, 0, (size_t)n * sizeof(int32_t), st)) != cudaSuccess ||
             (e = cudaMemsetAsync(d.ins_cnt, 0, (size_t)n * sizeof(int32_t), st)) != cudaSuccess ||
             (e = cudaMemsetAsync(d.cursor, 0, (size_t)n * sizeof(int32_t), st)) != cudaSuccess ||
-            (e = cudaMemsetAsync(d.touched, 0, (size_t)((n + 3) / 4 * 4), st)) != cudaSuccess)
+            (e = cudaMemsetAsync(d.touched, 0, (size_t)((n + 3) / 4 * 4), st)) != cudaSuccess ||
+            (e = cudaMemsetAsync(h->chunk_first_spare, 0, ((size_t)g.layout.row_warp + 1) * sizeof(int64_t), st)) !=
+                cudaSuccess)
             return cuda_fail(h, e, "memset dynamic scratch");
         h->col_cap = g.nnz;
     }
@@ -962,10 +996,6 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->launches += 4;  // degree level, select (two), count
     st = run_loop(h, 1);
     if (st != KATZ_OK) return st;
-    if ((e = cudaEventRecord(h->ev1, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
-    if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
-        return cuda_fail(h, e, "copy ctrl");
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "sync");
     float ms = 0.f;
     cudaEventElapsedTime(&ms, h->ev0, h->ev1);
     const Ctrl& hc = *h->h_ctrl;
@@ -977,12 +1007,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->eps = eps;
     h->ranked = true;
     h->last_ms = ms;
-    std::vector<int64_t> tr((size_t)h->opts.r_max + 2, 0);
-    if ((e = cudaMemcpyAsync(tr.data(), h->b.trace, tr.size() * sizeof(int64_t), cudaMemcpyDeviceToHost,
-                             h->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
-        return cuda_fail(h, e, "copy trace");
-    h->trace.assign(tr.begin() + 1, tr.begin() + 1 + std::max(0, h->r));
+    if ((st = take_trace(h)) != KATZ_OK) return st;
     if (h->opts.use_graph && !h->opts.profile)
         // loop bodies that did work: all finalize runs but the first iteration's
         h->launches += iteration_kernels(h) * std::max<int64_t>(0, (int64_t)hc.body_runs - 1);
@@ -1265,10 +1290,10 @@ katz_status update_prepare(katz_handle* h, const int32_t* src, const int32_t* ds
         (e = cudaMemcpyAsync(d.ins, is_insert, (size_t)m, cudaMemcpyDefault, sa)) != cudaSuccess)
         return cuda_done(e, "copy batch");
     // ---- validate (nothing changes unless the whole batch is valid) --------------
-    int32_t* herr = (int32_t*)(h->h_small + H_SMALL - 64);  // pinned words of this phase
-    if ((e = cudaMemsetAsync(d.err, 0, sizeof(int32_t), sa)) != cudaSuccess ||
+    int32_t* herr = (int32_t*)(h->h_small + H_SMALL - 64);  // pinned words of this phase: errors, insertions
+    if ((e = cudaMemsetAsync(d.err, 0, 2 * sizeof(int32_t), sa)) != cudaSuccess ||
         (e = dyn_validate(g, d, m, h->D, sa)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(herr, d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, sa)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(herr, d.err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, sa)) != cudaSuccess ||
         (e = cudaStreamSynchronize(sa)) != cudaSuccess)
         return cuda_done(e, "validate batch");
     pd.launches += 2;
@@ -1295,12 +1320,9 @@ katz_status update_prepare(katz_handle* h, const int32_t* src, const int32_t* ds
                                       sa)) != cudaSuccess))
         return cuda_done(e, "degree maxima");
     pd.launches += cert ? 1 : 0;
-    int64_t* hnnz = (int64_t*)(h->h_small + H_SMALL - 56);
-    if ((e = cudaMemcpyAsync(hnnz, h->rp_new + n, sizeof(int64_t), cudaMemcpyDeviceToHost, sa)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(sa)) != cudaSuccess)
-        return cuda_done(e, "rebuild size");
-    const unsigned long long dmax[3] = {cert ? hdmax[0] : 0ull, cert ? hdmax[1] : 0ull, cert ? hdmax[2] : 0ull};
-    const int64_t nnz_new = *hnnz;
+    // a valid batch changes the arcs by its insertions less its deletions: no
+    // need to wait for the new offsets
+    const int64_t nnz_new = g.nnz + (d.undirected ? 2 : 1) * (2 * (int64_t)herr[1] - m);
     // the updated graph outgrows 32-bit offsets: its offsets go to a new
     // int64 array, and a second one becomes the spare of later batches; the
     // swap installs both and releases the two int32 arrays
@@ -1354,44 +1376,39 @@ katz_status update_prepare(katz_handle* h, const int32_t* src, const int32_t* ds
     pd.launches += (g.n > g.layout.row_warp ? 2 : 0) + (g.layout.chunks > 0 ? 1 : 0) + (hubs ? 3 : 0) + 1;
     if ((e = dyn_clear(g, d, m, sa)) != cudaSuccess) return cuda_done(e, "clear batch");
     pd.launches += 1;
-    // chunk table of the CHUNK rows from their new degrees, into the spares
+    // chunk table of the CHUNK rows from their new degrees, into the spares (as
+    // at create: every CHUNK row adds at most one chunk to nnz / CHUNK_ARCS)
     const int64_t rw = g.layout.row_warp;
-    std::vector<int64_t> hrp((size_t)rw + 1);
-    if ((e = cudaMemcpyAsync(hrp.data(), h->rp_new, hrp.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, sa)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(sa)) != cudaSuccess)
-        return cuda_done(e, "copy rowptr head");
-    std::vector<int64_t> first((size_t)rw + 1, 0);
-    int64_t max_chunks = 0;
-    for (int64_t u = 0; u < rw; ++u) {
-        const int64_t c = (hrp[u + 1] - hrp[u] + CHUNK_ARCS - 1) / CHUNK_ARCS;
-        first[u + 1] = first[u] + c;
-        max_chunks = std::max(max_chunks, c);
-    }
-    const int64_t chunks = first[rw];
-    if (cert) {
-        const SpmvLayout& L = g.layout;
-        pd.depth = sum_depth_of((int64_t)dmax[0], (int64_t)dmax[1], (int64_t)dmax[2], L.row_thread > L.row_octet,
-                                L.row_octet > L.row_warp, rw > 0 ? std::max<int64_t>(max_chunks, 1) : 0);
-    }
-    if (chunks > h->chunk_row_spare_cap) {
+    const int64_t chunks_cap = rw > 0 ? nnz_new / CHUNK_ARCS + rw + 1 : 0;
+    if (chunks_cap > h->chunk_row_spare_cap) {
         dfree_on(h->chunk_row_spare, sa);
         h->chunk_row_spare = nullptr;
         h->chunk_row_spare_cap = 0;
-        const int64_t cap = chunks + chunks / 8 + 16;
+        const int64_t cap = chunks_cap + chunks_cap / 8 + 16;
         if ((e = dmalloc_on(h, &h->chunk_row_spare, (size_t)cap, sa)) != cudaSuccess)
             return cuda_done(e, "cudaMalloc chunks");
         h->chunk_row_spare_cap = cap;
     }
-    std::vector<int32_t> crow((size_t)std::max<int64_t>(chunks, 1));
-    for (int64_t u = 0; u < rw; ++u)
-        for (int64_t q = first[u]; q < first[u + 1]; ++q) crow[q] = (int32_t)u;
-    if ((e = cudaMemcpyAsync(h->chunk_first_spare, first.data(), first.size() * sizeof(int64_t),
-                             cudaMemcpyHostToDevice, sa)) != cudaSuccess ||
-        (chunks > 0 && (e = cudaMemcpyAsync(h->chunk_row_spare, crow.data(), (size_t)chunks * sizeof(int32_t),
-                                            cudaMemcpyHostToDevice, sa)) != cudaSuccess) ||
-        (e = cudaStreamSynchronize(sa)) != cudaSuccess)
-        return cuda_done(e, "copy chunks");
+    int64_t* hchunks = (int64_t*)(h->h_small + H_SMALL - 96);  // the chunks, the most of one row
+    hchunks[0] = hchunks[1] = 0;
+    if (rw > 0) {
+        if ((e = cudaMemsetAsync(d.mode_dmax + 3, 0, sizeof(unsigned long long), sa)) != cudaSuccess ||
+            (e = build_chunk_table(h->rp_new, rw, h->deg_tmp, h->scan_sums, h->chunk_first_spare, h->chunk_row_spare,
+                                   d.mode_dmax + 3, sa)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(hchunks, h->chunk_first_spare + rw, sizeof(int64_t), cudaMemcpyDeviceToHost, sa)) !=
+                cudaSuccess ||
+            (e = cudaMemcpyAsync(hchunks + 1, d.mode_dmax + 3, sizeof(int64_t), cudaMemcpyDeviceToHost, sa)) !=
+                cudaSuccess)
+            return cuda_done(e, "chunk table");
+        pd.launches += 5;  // counts, scan (three), fill
+    }
+    if ((rw > 0 || cert) && (e = cudaStreamSynchronize(sa)) != cudaSuccess) return cuda_done(e, "chunk table");
+    const int64_t chunks = hchunks[0];
+    if (cert) {
+        const SpmvLayout& L = g.layout;
+        pd.depth = sum_depth_of((int64_t)hdmax[0], (int64_t)hdmax[1], (int64_t)hdmax[2], L.row_thread > L.row_octet,
+                                L.row_octet > L.row_warp, rw > 0 ? std::max<int64_t>(hchunks[1], 1) : 0);
+    }
     pd.nnz = nnz_new;
     pd.chunks = chunks;
     pd.applied = true;
@@ -1603,18 +1620,12 @@ static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_l
         (e = launch_select(g, h->b, h->p, h->stream)) != cudaSuccess ||
         (e = launch_count(g, h->b, h->p, h->stream)) != cudaSuccess)
         return cuda_fail(h, e, "re-check");
-    if ((e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
-        return cuda_fail(h, e, "re-check sync");
-    katz_status st = KATZ_OK;
+    katz_status st = read_state(h);
+    if (st != KATZ_OK) return st;
     if (!h->h_ctrl->stop) {
         st = run_loop(h, 0);
         if (st != KATZ_OK) return st;
     }
-    if ((e = cudaEventRecord(h->ev1, h->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(h->h_ctrl, h->b.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
-        return cuda_fail(h, e, "sync");
     float ms = 0.f;
     cudaEventElapsedTime(&ms, h->ev0, h->ev1);
     const Ctrl& hc = *h->h_ctrl;
@@ -1624,12 +1635,7 @@ static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_l
     h->last_ms = ms;
     h->f32_from = hc.f32_from;
     const bool stalled = !hc.converged && hc.stall;
-    std::vector<int64_t> tr((size_t)h->opts.r_max + 2, 0);
-    if ((e = cudaMemcpyAsync(tr.data(), h->b.trace, tr.size() * sizeof(int64_t), cudaMemcpyDeviceToHost,
-                             h->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
-        return cuda_fail(h, e, "copy trace");
-    h->trace.assign(tr.begin() + 1, tr.begin() + 1 + std::max(0, h->r));
+    if ((st = take_trace(h)) != KATZ_OK) return st;
     if (stalled && h->opts.precision == KATZ_FP32_CERT_AUTO) {
         // the FP32 widening stalls the certificate on the updated graph: its
         // levels are recomputed in FP64 (the handle continues in FP64)

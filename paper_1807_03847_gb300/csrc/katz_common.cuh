@@ -250,7 +250,7 @@ struct DynBuffers {
     bool undirected = true;          // edges are unordered pairs (both arcs) or ordered ones
     unsigned long long* table = nullptr;  // open-addressing set of the batch's internal-id pairs (bit 63: delete)
     int64_t table_mask = 0;
-    int32_t* err = nullptr;
+    int32_t* err = nullptr;          // [2] error bits, number of insertions
     int32_t* delta = nullptr;        // [n] degree change
     int32_t* ins_cnt = nullptr;      // [n] inserted arcs per row
     int32_t* cursor = nullptr;       // [n]
@@ -269,7 +269,8 @@ struct DynBuffers {
     int64_t* rrowptr = nullptr;      // [n+1] directed: transposed CSR (in-arcs) of the current graph
     int32_t* rcol = nullptr;         // [rcap]
     int64_t rcap = 0;
-    unsigned long long* mode_dmax = nullptr;  // [3] FP32-certified: largest new degree per row mode in a batch
+    unsigned long long* mode_dmax = nullptr;  // [4] FP32-certified: largest new degree per row mode in a batch;
+                                              //   the most chunks of one CHUNK row
 };
 
 // ---- stopping criteria other than top-k (katz_criteria.cu) -------------------

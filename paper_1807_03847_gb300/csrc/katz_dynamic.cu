@@ -164,14 +164,18 @@ __global__ void validate_batch_kernel(const Off* __restrict__ rowptr, const int3
     }
 }
 
-// the rows the batch changes stay within D arcs (out-degrees when directed)
+// the rows the batch changes stay within D arcs (out-degrees when directed);
+// err[1] counts the insertions
 template <typename Off>
 __global__ void degree_check_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ inv,
-                                    const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m,
-                                    int64_t n, bool und, const int32_t* __restrict__ delta, int64_t D, int32_t* err) {
+                                    const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                    const uint8_t* __restrict__ ins, int64_t m, int64_t n, bool und,
+                                    const int32_t* __restrict__ delta, int64_t D, int32_t* err) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int mine = 0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
         const int32_t a = src[e], b = dst[e];
+        mine += ins[e] != 0;
         if (a < 0 || b < 0 || a >= n || b >= n) continue;
         const int32_t ends[2] = {inv[a], inv[b]};
         for (int q = 0; q < (und ? 2 : 1); ++q) {
@@ -179,6 +183,8 @@ __global__ void degree_check_kernel(const Off* __restrict__ rowptr, const int32_
             if ((int64_t)rowptr[u + 1] - (int64_t)rowptr[u] + delta[u] > D) atomicOr(err, DYN_E_ALPHA);
         }
     }
+    mine = __reduce_add_sync(FULL, mine);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(err + 1, mine);
 }
 
 // undo the per-node scratch of a batch (delta, insertion counters, marks)
@@ -801,10 +807,10 @@ cudaError_t dyn_validate(const DeviceGraph& g, const DynBuffers& d, int64_t m, i
                                                                d.delta, d.touched, d.err);
     if (g.off64)
         degree_check_kernel<int64_t><<<grid_for(m, 256), 256, 0, st>>>((const int64_t*)g.rowptr, g.inv, d.src, d.dst,
-                                                                      m, g.n, d.undirected, d.delta, D, d.err);
+                                                                      d.ins, m, g.n, d.undirected, d.delta, D, d.err);
     else
         degree_check_kernel<int32_t><<<grid_for(m, 256), 256, 0, st>>>((const int32_t*)g.rowptr, g.inv, d.src, d.dst,
-                                                                      m, g.n, d.undirected, d.delta, D, d.err);
+                                                                      d.ins, m, g.n, d.undirected, d.delta, D, d.err);
     return cudaGetLastError();
 }
 

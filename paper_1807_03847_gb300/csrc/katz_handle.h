@@ -35,6 +35,7 @@ struct katz_handle {
     double* d_scratch = nullptr;
     katz::Ctrl* h_ctrl = nullptr;  // pinned (one block with h_small)
     unsigned char* h_small = nullptr;  // pinned scratch of H_SMALL bytes for small device-to-host reads
+    int64_t* h_trace = nullptr;        // pinned, r_max + 2 entries (nullptr: r_max above H_TRACE)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // profiling: one event pair per SpMV launch
     std::vector<cudaEvent_t> sp_ev;
@@ -135,6 +136,7 @@ class L2FetchScope {
 
 constexpr size_t CTRL_BYTES = (sizeof(Ctrl) + 255) / 256 * 256;
 constexpr size_t H_SMALL = 4096;
+constexpr int H_TRACE = 1 << 16;
 
 cudaMemPool_t library_pool(int dev);
 
