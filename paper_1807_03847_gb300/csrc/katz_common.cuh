@@ -163,6 +163,7 @@ struct SpmvLayout {
     int64_t row_thread;  // rows [row_octet, row_thread): OCTET mode; [row_thread, n): THREAD
     int64_t chunks;      // CHUNK_ARCS-arc chunks of the CHUNK rows
     int64_t blk_warp, blk_octet, blk_thread, blocks_total;  // first block of each mode
+    int32_t octet_passes;  // OCTET rows per block, in units of one pass
 };
 
 // Staged gathers (katz_stage.cu): one window's places in bands [band0, band1)

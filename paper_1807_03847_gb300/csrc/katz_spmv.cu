@@ -18,7 +18,11 @@
 // lanes' accumulators, rounding and the epilogue cost as much as 30 arcs: with
 // half the lanes a warp pays for them once per two (WARP) or eight (OCTET)
 // rows.  R-MAT22, per level: WARP rows 162 -> 138 us, OCTET 110 -> 99; two lanes
-// per OCTET row or eight per WARP row gain nothing more.  FP32 levels keep their
+// per OCTET row or eight per WARP row gain nothing more.  A warp then takes up
+// to 32 OCTET rows in passes of eight (FP32: four) and finishes them together,
+// one row per lane: the epilogue runs once on full lanes and its accesses are
+// whole lines.  OCTET rows of R-MAT22 99 -> 92 us, of G(2^20, 8 n) 54 -> 45, of
+// Chung-Lu 2^25 857 -> 756.  FP32 levels keep their
 // lanes: the split sets the order of their sums, and longer chains of FP32
 // additions would widen the error bound.
 // The walk vector is gathered with read-only loads (one L2 request per arc:
@@ -63,8 +67,9 @@ constexpr int BLOCK = 256;
 constexpr int WARPS = BLOCK / 32;
 constexpr int OCTET_LANES = 4;   // lanes per OCTET row of an FP64 level (FP32: 8)
 constexpr int WARP_LANES = 16;   // lanes per WARP row of an FP64 level (FP32: 32)
-constexpr int OCTET_ROWS = BLOCK / OCTET_LANES;  // rows per block; FP32 levels take two passes
-constexpr int WARP_ROWS = BLOCK / WARP_LANES;
+constexpr int OCTET_ROWS = BLOCK / OCTET_LANES;  // rows per block and pass (FP32: two passes of 32)
+constexpr int WARP_ROWS = BLOCK / WARP_LANES;    // rows per block (FP32: in two passes)
+constexpr int64_t FULL_CHIP = 152 * 6 * 2;       // blocks: two waves of six per multiprocessor
 
 struct Epi {
     void* y;          // level r slot (double or float)
@@ -524,14 +529,29 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
     if constexpr (sizeof(T) == 8) {
         if (b >= L.blk_thread) {  // THREAD rows
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
-            if (u < L.n) finish_row<double>(u, xacc_to_double(strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], 0, 1)), ep, p);
+            if (u < L.n)
+                finish_row<double>(u, xacc_to_double(strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], 0, 1)), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
-            const int64_t u = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + tid / OCTET_LANES;
-            const int sub = tid % OCTET_LANES;
+            const int rows = L.octet_passes * (32 / OCTET_LANES);  // of this warp
+            const int64_t u0 = L.row_octet + (b - L.blk_octet) * (OCTET_ROWS * (int64_t)L.octet_passes) + wid * rows;
+            const int64_t u = u0 + lane;  // the row this lane finishes
+            const bool mine = lane < rows && u < L.row_thread;
+            const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
             XAcc s = xacc_zero();
-            if (u < L.row_thread) s = strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], sub, OCTET_LANES);
-            s = xacc_group_sum<OCTET_LANES>(s);
-            if (sub == 0 && u < L.row_thread) finish_row<double>(u, xacc_to_double(s), ep, p);
+            for (int first = 0; first < rows; first += 32 / OCTET_LANES) {
+                const int r = first + lane / OCTET_LANES;  // rows past the last one are empty
+                XAcc t = strided_xsum<4>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r),
+                                         lane % OCTET_LANES, OCTET_LANES);
+                t = xacc_group_sum<OCTET_LANES>(t);
+                const int from = (lane - first) * OCTET_LANES & 31;
+                t.w0 = __shfl_sync(FULL, t.w0, from);
+                t.w1 = __shfl_sync(FULL, t.w1, from);
+                t.w2 = __shfl_sync(FULL, t.w2, from);
+                t.w3 = __shfl_sync(FULL, t.w3, from);
+                t.E = __shfl_sync(FULL, t.E, from);
+                if (lane >= first && lane < first + 32 / OCTET_LANES) s = t;
+            }
+            if (mine) finish_row<double>(u, xacc_to_double(s), ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
             const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
             const int sub = tid % WARP_LANES;
@@ -557,15 +577,21 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
             const int64_t u = L.row_thread + (b - L.blk_thread) * BLOCK + tid;
             if (u < L.n) finish_row<Acc>(u, strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], 0, 1), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
-            const int sub = tid & 7;
-            const int64_t u0 = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + (tid >> 3);
-            for (int64_t u = u0; u < u0 + OCTET_ROWS; u += BLOCK / 8) {
-                Acc s = (Acc)0;
-                if (u < L.row_thread) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], sub, 8);
+            const int rows = L.octet_passes * (32 / OCTET_LANES);
+            const int64_t u0 = L.row_octet + (b - L.blk_octet) * (OCTET_ROWS * (int64_t)L.octet_passes) + wid * rows;
+            const int64_t u = u0 + lane;
+            const bool mine = lane < rows && u < L.row_thread;
+            const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
+            Acc s = (Acc)0;
+            for (int first = 0; first < rows; first += 4) {
+                const int r = first + (lane >> 3);
+                Acc t = strided_sum<Acc>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r), lane & 7, 8);
 #pragma unroll
-                for (int off = 4; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off, 8));
-                if (sub == 0 && u < L.row_thread) finish_row<Acc>(u, s, ep, p);
+                for (int off = 4; off; off >>= 1) t = addA<Acc>(t, __shfl_down_sync(FULL, t, off, 8));
+                t = __shfl_sync(FULL, t, (lane - first) * 8 & 31);
+                if (lane >= first && lane < first + 4) s = t;
             }
+            if (mine) finish_row<Acc>(u, s, ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
             const int64_t u0 = L.row_warp + (b - L.blk_warp) * WARP_ROWS + wid;
             for (int64_t u = u0; u < u0 + WARP_ROWS; u += WARPS) {
@@ -1078,14 +1104,16 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
                 store_pair64(y, t_out, u, sa, sb, alpha);
             }
         } else if (b >= L.blk_octet) {
-            const int64_t u = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + tid / OCTET_LANES;
             const int sub = tid % OCTET_LANES;
-            sa = xacc_zero();
-            sb = xacc_zero();
-            if (u < L.row_thread) strided_xsum2<4>(col, x, rowptr[u], rowptr[u + 1], sub, OCTET_LANES, sa, sb);
-            sa = xacc_group_sum<OCTET_LANES>(sa);
-            sb = xacc_group_sum<OCTET_LANES>(sb);
-            if (sub == 0 && u < L.row_thread) store_pair64(y, t_out, u, sa, sb, alpha);
+            const int64_t rows = OCTET_ROWS * (int64_t)L.octet_passes, u0 = L.row_octet + (b - L.blk_octet) * rows;
+            for (int64_t u = u0 + tid / OCTET_LANES; u < u0 + rows; u += OCTET_ROWS) {
+                sa = xacc_zero();
+                sb = xacc_zero();
+                if (u < L.row_thread) strided_xsum2<4>(col, x, rowptr[u], rowptr[u + 1], sub, OCTET_LANES, sa, sb);
+                sa = xacc_group_sum<OCTET_LANES>(sa);
+                sb = xacc_group_sum<OCTET_LANES>(sb);
+                if (sub == 0 && u < L.row_thread) store_pair64(y, t_out, u, sa, sb, alpha);
+            }
         } else if (b >= L.blk_warp) {
             const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
             const int sub = tid % WARP_LANES;
@@ -1124,8 +1152,8 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
             }
         } else if (b >= L.blk_octet) {
             const int sub = tid & 7;
-            const int64_t u0 = L.row_octet + (b - L.blk_octet) * OCTET_ROWS + (tid >> 3);
-            for (int64_t u = u0; u < u0 + OCTET_ROWS; u += BLOCK / 8) {
+            const int64_t rows = OCTET_ROWS * (int64_t)L.octet_passes, u0 = L.row_octet + (b - L.blk_octet) * rows;
+            for (int64_t u = u0 + (tid >> 3); u < u0 + rows; u += BLOCK / 8) {
                 sa = 0.0f;
                 sb = 0.0f;
                 if (u < L.row_thread) strided_sum2(col, x, rowptr[u], rowptr[u + 1], sub, 8, sa, sb);
@@ -1420,7 +1448,11 @@ SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t r
     L.chunks = chunks;
     const int64_t bc = (chunks + WARPS - 1) / WARPS;
     const int64_t bw = (row_octet - row_warp + WARP_ROWS - 1) / WARP_ROWS;
-    const int64_t bo = (row_thread - row_octet + OCTET_ROWS - 1) / OCTET_ROWS;
+    // OCTET rows: a warp takes up to 32 of them and finishes them together, as
+    // long as the blocks fill the chip a few times over
+    const int64_t octets = row_thread - row_octet;
+    L.octet_passes = octets >= 4 * OCTET_ROWS * FULL_CHIP ? 4 : (octets >= 2 * OCTET_ROWS * FULL_CHIP ? 2 : 1);
+    const int64_t bo = (octets + OCTET_ROWS * L.octet_passes - 1) / (OCTET_ROWS * L.octet_passes);
     const int64_t bt = (n - row_thread + BLOCK - 1) / BLOCK;
     L.blk_warp = bc;
     L.blk_octet = bc + bw;
