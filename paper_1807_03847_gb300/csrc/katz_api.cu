@@ -894,6 +894,8 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
           "copy");
     KCHK2(cudaStreamSynchronize(h->stream), "relabel sync");
     g.layout = make_layout(n, row_warp, row_octet, row_thread, hv.chunks);
+    // two walk slots and no batches: the rows of degree 0 stay as level 1 leaves them
+    if (!h->opts.keep_history) g.layout.row_empty = std::max<int64_t>((int64_t)hv.cs[0], row_thread);
     h->sum_depth = max_sum_depth(g.layout, (int64_t)hv.max_chunks);
     dfree(h, d_bad);
     dfree(h, d_degmax);

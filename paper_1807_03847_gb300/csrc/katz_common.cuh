@@ -161,6 +161,7 @@ struct SpmvLayout {
     int64_t row_warp;    // rows [0, row_warp): CHUNK mode (degree > 2048)
     int64_t row_octet;   // rows [row_warp, row_octet): WARP mode
     int64_t row_thread;  // rows [row_octet, row_thread): OCTET mode; [row_thread, n): THREAD
+    int64_t row_empty;   // rows [row_empty, n) are known to have no arcs, now and later (n: none)
     int64_t chunks;      // CHUNK_ARCS-arc chunks of the CHUNK rows
     int64_t blk_warp, blk_octet, blk_thread, blocks_total;  // first block of each mode
     int32_t octet_passes;  // OCTET rows per block, in units of one pass

@@ -28,9 +28,10 @@ def test_tied_candidates(n, k, r_max):
 
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("k", [10, 1500, CAP])
-@pytest.mark.parametrize("graph", ["rmat", "er", "directed"])
+@pytest.mark.parametrize("graph", ["rmat", "er", "directed", "mostly-empty"])
 def test_spread_candidates(graph, k, precision):
     g = {"rmat": lambda: gg.rmat(15, 16, seed=3), "er": lambda: gg.erdos_renyi(40000, 320000, seed=4),
+         "mostly-empty": lambda: gg.from_edges(30000, np.arange(900), (np.arange(900) * 7 + 1) % 1000),
          "directed": lambda: gg.orient(gg.rmat(15, 16, seed=5), 6)}[graph]()
     for r_max in (1, 2, 3, 7):
         _check(g, k, r_max, precision, undirected=0 if graph == "directed" else 1)
@@ -41,8 +42,10 @@ def _check(g, k, r_max, precision=0, undirected=1):
 
     h = K.Katz(torch.from_numpy(g.rowptr).cuda(), torch.from_numpy(g.col).cuda(),
                K.katz_default_opts(r_max=r_max, precision=precision, undirected=undirected))
-    h.rank(0.0, k, 1e-9, check=False)
+    info = h.rank(0.0, k, 1e-9, check=False)
     lo, _, _ = h.bounds()
     kk = min(k, g.n)
     assert np.array_equal(h.ranking(kk), np.lexsort((np.arange(g.n), -lo))[:kk])
+    empty = np.diff(g.rowptr) == 0  # rows the later levels leave alone
+    assert not h.walk(info.r)[empty].any() and not lo[empty].any()
     h.close()
