@@ -23,13 +23,13 @@ __device__ __forceinline__ bool last_block(unsigned int* ticket) {
 }
 
 constexpr int RANK_THREADS = 256;
-constexpr int RANK_LANES = 16;  // lanes that count for one candidate
+constexpr int RANK_LANES = 32;  // lanes that count for one candidate
 constexpr int RANK_PER_BLOCK = RANK_THREADS / RANK_LANES;
 constexpr int RANK_TILE = 2048;  // keys staged in shared memory at a time
 
 // Place of candidate (key, id) among the cnt candidates in the order (key
 // desc, id asc): the number of candidates before it, counted by RANK_LANES
-// lanes (an aligned group of a warp) and returned to all of them.  Sorting the
+// lanes (a warp) and returned to all of them.  Sorting the
 // list in one block left the other multiprocessors idle behind ~100 barriers;
 // counting compares cnt^2 pairs, but over the whole chip: a top-1000 list takes
 // 7.4 us where the sort took 46.
@@ -56,7 +56,8 @@ __device__ __forceinline__ int rank_by_count(const unsigned long long* __restric
 #pragma unroll 8
         for (int j = tid & (RANK_LANES - 1); j < m; j += RANK_LANES) {
             const unsigned long long k = s_key[j];
-            before += k > key || (k == key && s_id[j] < id);
+            const int32_t i = s_id[j];  // read in any case: no branch
+            before += (k > key) | ((k == key) & (i < id));
         }
     }
 #pragma unroll

@@ -13,6 +13,8 @@
 #include <cooperative_groups.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "katz_common.cuh"
 #include "katz_grid.cuh"
 
@@ -355,6 +357,7 @@ select_filter_kernel(const double* __restrict__ cl, const int32_t* __restrict__ 
     } else if (blockIdx.x == 0 && tid == 0) {
         atomicMax(&f.state->n, SELECT_CAP + 1u);  // no tau: all of them, too many
     }
+    if (nc <= (unsigned long long)SELECT_CAP) return;  // all of them fit
     if (!last_block(&f.state->ticket)) return;
     if (__ldcg(&f.state->n) <= (unsigned int)SELECT_CAP) return;
     const unsigned int cnt = select_large(cl, cid, nc, __longlong_as_double(tau < 0 ? 0 : tau), (long long)p.k, f);
@@ -855,7 +858,10 @@ cudaError_t launch_theta0_class(const DeviceGraph& g, const IterBuffers& b, cons
 cudaError_t launch_select(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
     select_filter_kernel<<<grid_for(p.n, SELECT_THREADS, 152), SELECT_THREADS, 0, st>>>(
         b.cand_l, b.cand_id, b.lb, g.inv, b.topk_id, b.sel, b.ctrl, p);
-    select_rank_kernel<<<grid_for(p.n, RANK_PER_BLOCK, SELECT_CAP / RANK_PER_BLOCK), RANK_THREADS, 0, st>>>(
+    // a block per RANK_PER_BLOCK candidates of a usual list (blocks without any
+    // cost a launch all the same); longer lists are strided over
+    const int64_t usual = std::min<int64_t>(p.n, std::max<int64_t>(SELECT_DIRECT, 2 * p.k));
+    select_rank_kernel<<<grid_for(usual, RANK_PER_BLOCK, SELECT_CAP / RANK_PER_BLOCK), RANK_THREADS, 0, st>>>(
         b.cand_l, b.cand_u, b.cand_id, b.sel, b.topk_id, b.topk_l, b.topk_u, b.ctrl, p);
     return cudaGetLastError();
 }
