@@ -164,7 +164,7 @@ struct SpmvLayout {
     int64_t row_empty;   // rows [row_empty, n) are known to have no arcs, now and later (n: none)
     int64_t chunks;      // CHUNK_ARCS-arc chunks of the CHUNK rows
     int64_t blk_warp, blk_octet, blk_thread, blocks_total;  // first block of each mode
-    int32_t octet_passes;  // OCTET rows per block, in units of one pass
+    int32_t octet_passes, warp_passes;  // OCTET and WARP rows per block, in units of one pass
 };
 
 // Staged gathers (katz_stage.cu): one window's places in bands [band0, band1)
@@ -317,7 +317,9 @@ cudaError_t dyn_reactivate(const DeviceGraph& g, const IterBuffers& b, const Ite
 cudaError_t dyn_mode_degree_max(const DeviceGraph& g, const DynBuffers& d, int64_t m, const int64_t* rp_new,
                                 cudaStream_t st);
 
-SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t row_thread, int64_t chunks);
+// *_passes: at most so many passes of WARP / OCTET rows per warp (1, 2 or 4)
+SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t row_thread, int64_t chunks,
+                       int warp_passes = 4, int octet_passes = 4);
 // create-time relabelling (katz_relabel.cu)
 int relabel_blocks(int64_t n);
 int64_t scan_blocks(int64_t n);

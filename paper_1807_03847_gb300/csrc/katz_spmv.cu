@@ -22,7 +22,9 @@
 // to 32 OCTET rows in passes of eight (FP32: four) and finishes them together,
 // one row per lane: the epilogue runs once on full lanes and its accesses are
 // whole lines.  OCTET rows of R-MAT22 99 -> 92 us, of G(2^20, 8 n) 54 -> 45, of
-// Chung-Lu 2^25 857 -> 756.  FP32 levels keep their
+// Chung-Lu 2^25 857 -> 756.  Eight WARP rows at a time (FP64 in passes of two, FP32 of
+// one): R-MAT22 138 -> 135 us, the R-MAT24 FP32-certified ranking 12.6 -> 12.4 ms.
+// FP32 levels keep their
 // lanes: the split sets the order of their sums, and longer chains of FP32
 // additions would widen the error bound.
 // The walk vector is gathered with read-only loads (one L2 request per arc:
@@ -67,8 +69,8 @@ constexpr int BLOCK = 256;
 constexpr int WARPS = BLOCK / 32;
 constexpr int OCTET_LANES = 4;   // lanes per OCTET row of an FP64 level (FP32: 8)
 constexpr int WARP_LANES = 16;   // lanes per WARP row of an FP64 level (FP32: 32)
-constexpr int OCTET_ROWS = BLOCK / OCTET_LANES;  // rows per block and pass (FP32: two passes of 32)
-constexpr int WARP_ROWS = BLOCK / WARP_LANES;    // rows per block (FP32: in two passes)
+constexpr int OCTET_ROWS = BLOCK / OCTET_LANES;  // rows per block and pass
+constexpr int WARP_ROWS = BLOCK / WARP_LANES;
 constexpr int64_t FULL_CHIP = 152 * 6 * 2;       // blocks: two waves of six per multiprocessor
 
 struct Epi {
@@ -437,12 +439,14 @@ __device__ __forceinline__ double xacc_to_double(const XAcc& a) {
 // place above (y points hot entries before the staged values).
 template <typename T, int S = 1>
 struct Direct {
+    static constexpr bool FAR = false;
     const T* __restrict__ x;
     __device__ __forceinline__ T operator()(int32_t c) const { return __ldg(x + (int64_t)S * c); }
 };
 
 template <typename T>
 struct Staged {
+    static constexpr bool FAR = true;  // values far apart: more loads in flight for WARP rows
     const T* __restrict__ x;
     const T* __restrict__ y;
     uint32_t hot;
@@ -516,6 +520,56 @@ __device__ __forceinline__ Acc strided_sum(const int32_t* __restrict__ col, cons
     return s;
 }
 
+// Rows [u0, u0 + rows) below row_end by one warp (rows <= 32), `Lanes` lanes
+// per row: 32 / Lanes rows are summed at a time, every sum handed to a lane of
+// its own, and all of them finished together.
+template <int G, int Lanes, typename Off, typename X>
+__device__ __forceinline__ void finish_batch(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                             const X& x, int64_t u0, int rows, int64_t row_end, const Epi& ep,
+                                             const IterParams& p) {
+    constexpr int AT_ONCE = 32 / Lanes;
+    const int lane = threadIdx.x & 31;
+    const int64_t u = u0 + lane;  // the row this lane finishes
+    const bool mine = lane < rows && u < row_end;
+    const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
+    XAcc s = xacc_zero();
+    for (int first = 0; first < rows; first += AT_ONCE) {
+        const int r = first + lane / Lanes;  // rows past the last one are empty
+        XAcc t = strided_xsum<G>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r), lane % Lanes, Lanes);
+        t = xacc_group_sum<Lanes>(t);
+        const int from = (lane - first) * Lanes & 31;
+        t.w0 = __shfl_sync(FULL, t.w0, from);
+        t.w1 = __shfl_sync(FULL, t.w1, from);
+        t.w2 = __shfl_sync(FULL, t.w2, from);
+        t.w3 = __shfl_sync(FULL, t.w3, from);
+        t.E = __shfl_sync(FULL, t.E, from);
+        if (lane >= first && lane < first + AT_ONCE) s = t;
+    }
+    if (mine) finish_row<double>(u, xacc_to_double(s), ep, p);
+}
+
+// the same for an FP32 level (sums in the fixed order of Lanes lanes)
+template <int Lanes, typename Off, typename X>
+__device__ __forceinline__ void finish_batch_f32(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                                 const X& x, int64_t u0, int rows, int64_t row_end, const Epi& ep,
+                                                 const IterParams& p) {
+    constexpr int AT_ONCE = 32 / Lanes;
+    const int lane = threadIdx.x & 31;
+    const int64_t u = u0 + lane;
+    const bool mine = lane < rows && u < row_end;
+    const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
+    float s = 0.0f;
+    for (int first = 0; first < rows; first += AT_ONCE) {
+        const int r = first + lane / Lanes;
+        float t = strided_sum<float>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r), lane % Lanes, Lanes);
+#pragma unroll
+        for (int off = Lanes / 2; off; off >>= 1) t = addA<float>(t, __shfl_down_sync(FULL, t, off, Lanes));
+        t = __shfl_sync(FULL, t, (lane - first) * Lanes & 31);
+        if (lane >= first && lane < first + AT_ONCE) s = t;
+    }
+    if (mine) finish_row<float>(u, s, ep, p);
+}
+
 // One level of type T (its input x has the same type).  FP64 levels
 // sum exactly (XAcc); FP32 levels add in FP32 (fixed pairwise order).
 template <typename Off, typename T, typename X>
@@ -533,32 +587,23 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
                 finish_row<double>(u, xacc_to_double(strided_xsum<4>(col, x, rowptr[u], rowptr[u + 1], 0, 1)), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
             const int rows = L.octet_passes * (32 / OCTET_LANES);  // of this warp
-            const int64_t u0 = L.row_octet + (b - L.blk_octet) * (OCTET_ROWS * (int64_t)L.octet_passes) + wid * rows;
-            const int64_t u = u0 + lane;  // the row this lane finishes
-            const bool mine = lane < rows && u < L.row_thread;
-            const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
-            XAcc s = xacc_zero();
-            for (int first = 0; first < rows; first += 32 / OCTET_LANES) {
-                const int r = first + lane / OCTET_LANES;  // rows past the last one are empty
-                XAcc t = strided_xsum<4>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r),
-                                         lane % OCTET_LANES, OCTET_LANES);
-                t = xacc_group_sum<OCTET_LANES>(t);
-                const int from = (lane - first) * OCTET_LANES & 31;
-                t.w0 = __shfl_sync(FULL, t.w0, from);
-                t.w1 = __shfl_sync(FULL, t.w1, from);
-                t.w2 = __shfl_sync(FULL, t.w2, from);
-                t.w3 = __shfl_sync(FULL, t.w3, from);
-                t.E = __shfl_sync(FULL, t.E, from);
-                if (lane >= first && lane < first + 32 / OCTET_LANES) s = t;
-            }
-            if (mine) finish_row<double>(u, xacc_to_double(s), ep, p);
+            finish_batch<4, OCTET_LANES>(rowptr, col, x, L.row_octet + ((b - L.blk_octet) * WARPS + wid) * rows, rows,
+                                         L.row_thread, ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
-            const int sub = tid % WARP_LANES;
-            XAcc s = xacc_zero();
-            if (u < L.row_octet) s = strided_xsum<8>(col, x, rowptr[u], rowptr[u + 1], sub, WARP_LANES);
-            s = xacc_group_sum<WARP_LANES>(s);
-            if (sub == 0 && u < L.row_octet) finish_row<double>(u, xacc_to_double(s), ep, p);
+            if constexpr (X::FAR) {
+                const int64_t rows = WARP_ROWS * (int64_t)L.warp_passes, u0 = L.row_warp + (b - L.blk_warp) * rows;
+                for (int64_t u = u0 + tid / WARP_LANES; u < u0 + rows; u += WARP_ROWS) {
+                    XAcc s = xacc_zero();
+                    if (u < L.row_octet)
+                        s = strided_xsum<8>(col, x, rowptr[u], rowptr[u + 1], tid % WARP_LANES, WARP_LANES);
+                    s = xacc_group_sum<WARP_LANES>(s);
+                    if (tid % WARP_LANES == 0 && u < L.row_octet) finish_row<double>(u, xacc_to_double(s), ep, p);
+                }
+            } else {
+                const int rows = L.warp_passes * (32 / WARP_LANES);
+                finish_batch<4, WARP_LANES>(rowptr, col, x, L.row_warp + ((b - L.blk_warp) * WARPS + wid) * rows, rows,
+                                            L.row_octet, ep, p);
+            }
         } else {  // CHUNK rows: one warp per chunk of CHUNK_ARCS arcs
             const int64_t ch = b * WARPS + wid;
             XAcc s = xacc_zero();
@@ -578,29 +623,12 @@ __device__ __forceinline__ void spmv_rows(const Off* __restrict__ rowptr, const 
             if (u < rows_end) finish_row<Acc>(u, strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], 0, 1), ep, p);
         } else if (b >= L.blk_octet) {  // OCTET rows
             const int rows = L.octet_passes * (32 / OCTET_LANES);
-            const int64_t u0 = L.row_octet + (b - L.blk_octet) * (OCTET_ROWS * (int64_t)L.octet_passes) + wid * rows;
-            const int64_t u = u0 + lane;
-            const bool mine = lane < rows && u < L.row_thread;
-            const Off ra = mine ? rowptr[u] : (Off)0, rb = mine ? rowptr[u + 1] : (Off)0;
-            Acc s = (Acc)0;
-            for (int first = 0; first < rows; first += 4) {
-                const int r = first + (lane >> 3);
-                Acc t = strided_sum<Acc>(col, x, __shfl_sync(FULL, ra, r), __shfl_sync(FULL, rb, r), lane & 7, 8);
-#pragma unroll
-                for (int off = 4; off; off >>= 1) t = addA<Acc>(t, __shfl_down_sync(FULL, t, off, 8));
-                t = __shfl_sync(FULL, t, (lane - first) * 8 & 31);
-                if (lane >= first && lane < first + 4) s = t;
-            }
-            if (mine) finish_row<Acc>(u, s, ep, p);
+            finish_batch_f32<8>(rowptr, col, x, L.row_octet + ((b - L.blk_octet) * WARPS + wid) * rows, rows,
+                                L.row_thread, ep, p);
         } else if (b >= L.blk_warp) {  // WARP rows
-            const int64_t u0 = L.row_warp + (b - L.blk_warp) * WARP_ROWS + wid;
-            for (int64_t u = u0; u < u0 + WARP_ROWS; u += WARPS) {
-                Acc s = (Acc)0;
-                if (u < L.row_octet) s = strided_sum<Acc>(col, x, rowptr[u], rowptr[u + 1], lane, 32);
-#pragma unroll
-                for (int off = 16; off; off >>= 1) s = addA<Acc>(s, __shfl_down_sync(FULL, s, off));
-                if (lane == 0 && u < L.row_octet) finish_row<Acc>(u, s, ep, p);
-            }
+            const int rows = L.warp_passes * (32 / WARP_LANES);
+            finish_batch_f32<32>(rowptr, col, x, L.row_warp + ((b - L.blk_warp) * WARPS + wid) * rows, rows,
+                                 L.row_octet, ep, p);
         } else {  // CHUNK rows: one warp per chunk of CHUNK_ARCS arcs
             const int64_t ch = b * WARPS + wid;
             Acc s = (Acc)0;
@@ -1123,14 +1151,16 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
                 if (sub == 0 && u < L.row_thread) store_pair64(y, t_out, u, sa, sb, alpha);
             }
         } else if (b >= L.blk_warp) {
-            const int64_t u = L.row_warp + (b - L.blk_warp) * WARP_ROWS + tid / WARP_LANES;
             const int sub = tid % WARP_LANES;
-            sa = xacc_zero();
-            sb = xacc_zero();
-            if (u < L.row_octet) strided_xsum2<8>(col, x, rowptr[u], rowptr[u + 1], sub, WARP_LANES, sa, sb);
-            sa = xacc_group_sum<WARP_LANES>(sa);
-            sb = xacc_group_sum<WARP_LANES>(sb);
-            if (sub == 0 && u < L.row_octet) store_pair64(y, t_out, u, sa, sb, alpha);
+            const int64_t rows = WARP_ROWS * (int64_t)L.warp_passes, u0 = L.row_warp + (b - L.blk_warp) * rows;
+            for (int64_t u = u0 + tid / WARP_LANES; u < u0 + rows; u += WARP_ROWS) {
+                sa = xacc_zero();
+                sb = xacc_zero();
+                if (u < L.row_octet) strided_xsum2<8>(col, x, rowptr[u], rowptr[u + 1], sub, WARP_LANES, sa, sb);
+                sa = xacc_group_sum<WARP_LANES>(sa);
+                sb = xacc_group_sum<WARP_LANES>(sb);
+                if (sub == 0 && u < L.row_octet) store_pair64(y, t_out, u, sa, sb, alpha);
+            }
         } else {
             const int64_t ch = b * WARPS + wid;
             sa = xacc_zero();
@@ -1170,8 +1200,8 @@ spmv_pair_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col
                 if (sub == 0 && u < L.row_thread) y[u] = make_float2(__fmul_rn(alpha_f, sa), __fmul_rn(alpha_f, sb));
             }
         } else if (b >= L.blk_warp) {
-            const int64_t u0 = L.row_warp + (b - L.blk_warp) * WARP_ROWS + wid;
-            for (int64_t u = u0; u < u0 + WARP_ROWS; u += WARPS) {
+            const int64_t rows = WARP_ROWS * (int64_t)L.warp_passes, u0 = L.row_warp + (b - L.blk_warp) * rows;
+            for (int64_t u = u0 + wid; u < u0 + rows; u += WARPS) {
                 sa = 0.0f;
                 sb = 0.0f;
                 if (u < L.row_octet) strided_sum2(col, x, rowptr[u], rowptr[u + 1], lane, 32, sa, sb);
@@ -1447,7 +1477,8 @@ cudaError_t launch_pair_split(const DeviceGraph& g, const IterBuffers& b, const 
 }
 
 // Block ranges of the four row modes from the internal row boundaries.
-SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t row_thread, int64_t chunks) {
+SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t row_thread, int64_t chunks,
+                       int warp_passes, int octet_passes) {
     SpmvLayout L{};
     L.n = n;
     L.row_warp = row_warp;
@@ -1456,12 +1487,18 @@ SpmvLayout make_layout(int64_t n, int64_t row_warp, int64_t row_octet, int64_t r
     L.row_empty = n;
     L.chunks = chunks;
     const int64_t bc = (chunks + WARPS - 1) / WARPS;
-    const int64_t bw = (row_octet - row_warp + WARP_ROWS - 1) / WARP_ROWS;
-    // OCTET rows: a warp takes up to 32 of them and finishes them together, as
-    // long as the blocks fill the chip a few times over
-    const int64_t octets = row_thread - row_octet;
-    L.octet_passes = octets >= 4 * OCTET_ROWS * FULL_CHIP ? 4 : (octets >= 2 * OCTET_ROWS * FULL_CHIP ? 2 : 1);
-    const int64_t bo = (octets + OCTET_ROWS * L.octet_passes - 1) / (OCTET_ROWS * L.octet_passes);
+    // a warp takes up to 32 OCTET rows, or eight WARP rows, and finishes them
+    // together, as long as the blocks fill the chip a few times over
+    auto passes = [](int64_t rows, int per_block, int most) -> int32_t {
+        int32_t p = most;
+        while (p > 1 && rows < p * per_block * FULL_CHIP) p /= 2;
+        return p;
+    };
+    L.octet_passes = passes(row_thread - row_octet, OCTET_ROWS, octet_passes);
+    L.warp_passes = passes(row_octet - row_warp, WARP_ROWS, warp_passes);
+    const int64_t per_bw = WARP_ROWS * (int64_t)L.warp_passes, per_bo = OCTET_ROWS * (int64_t)L.octet_passes;
+    const int64_t bw = (row_octet - row_warp + per_bw - 1) / per_bw;
+    const int64_t bo = (row_thread - row_octet + per_bo - 1) / per_bo;
     const int64_t bt = (n - row_thread + BLOCK - 1) / BLOCK;
     L.blk_warp = bc;
     L.blk_octet = bc + bw;
