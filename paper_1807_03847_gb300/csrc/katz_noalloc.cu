@@ -14,7 +14,7 @@
 // Its work is the selection and checking half of an iteration of the
 // library's main loop, run over all n nodes:
 //   groups   the nodes fall into 8192 groups by a hash of their id; the k-th
-//            largest of the groups' largest lower bounds, cut to its upper 32
+//            largest of the groups' largest lower bounds, cut to its upper 22
 //            bits, is reached by at least k nodes, and by few more (about 1660
 //            for k = 1500, wherever the large bounds lie);
 //   compact  the nodes that reach it, the candidates;
@@ -27,7 +27,7 @@
 // Each of the three passes over the nodes reads one array of 8 n bytes.  A
 // radix select over all nodes with a sort in one block took 419 us at n = 4 M,
 // k = 1000 (230 of them in global atomics on the few bins that hold most
-// bounds); these kernels take 100 us, launches included.
+// bounds); these kernels take 90 us, launches included.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 #include <stdint.h>
@@ -149,12 +149,14 @@ na_groups(NoAllocScratch* S, const double* __restrict__ lower, long long n, long
             x = max(x, __ldcg(&S->hist[s * NA_GROUPS + ((q * NA_GROUP_THREADS + tid) ^ (mix(s) % NA_GROUPS))]));
         g[q] = x;
     }
-    // the largest key that at least k groups reach, two bits a step
-    __shared__ int s_cnt[16][3];
-    if (tid < 48) (&s_cnt[0][0])[tid] = 0;
+    // a key that at least k groups reach: the largest one with its lower 10 bits
+    // 0 (a mantissa of 10 bits left), two bits a step
+    constexpr int STEPS = 11;
+    __shared__ int s_cnt[STEPS][3];
+    if (tid < 3 * STEPS) (&s_cnt[0][0])[tid] = 0;
     __syncthreads();
     unsigned int key = 0;
-    for (int step = 0; step < 16; ++step) {
+    for (int step = 0; step < STEPS; ++step) {
         const int sh = 30 - 2 * step;
         int c[3] = {0, 0, 0};
 #pragma unroll
@@ -194,6 +196,8 @@ __device__ __forceinline__ void add_candidate(NoAllocScratch* S, bool take, doub
 
 __global__ void __launch_bounds__(256)
 na_compact(NoAllocScratch* S, const double* __restrict__ lower, const double* __restrict__ upper, long long n) {
+    // no counts yet, for the radix select (the groups are done with the array)
+    for (int q = blockIdx.x * 256 + threadIdx.x; q < NA_BINS; q += gridDim.x * 256) S->hist[q] = 0;
     if (S->use_radix) return;
     const unsigned int gk = S->group_key;
     constexpr int U = 4;
@@ -296,12 +300,6 @@ na_radix(NoAllocScratch* S, const double* __restrict__ lower, long long n, int p
         if (bin < 0x10000u && lane == __ffs(peers) - 1) atomicAdd(&S->hist[bin], (unsigned)__popc(peers));
     }
     if (last_block(&S->ticket)) radix_find(S, pass);
-}
-
-// before the first pass: no counts
-__global__ void na_radix_reset(NoAllocScratch* S) {
-    if (!radix_needed(S)) return;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NA_BINS; q += gridDim.x * blockDim.x) S->hist[q] = 0;
 }
 
 // after the last pass: the candidates at or above the threshold
@@ -421,7 +419,6 @@ extern "C" katz_status katz_certify_topk_noalloc(const double* lower, const doub
     if (n > NA_CAP) {  // else every node fits
         const int rgrid = (int)((n + NA_RADIX_THREADS - 1) / NA_RADIX_THREADS < cap / 2
                                     ? (n + NA_RADIX_THREADS - 1) / NA_RADIX_THREADS : cap / 2);
-        na_radix_reset<<<64, 1024, 0, s>>>(S);
         for (int pass = 0; pass < 6; ++pass) na_radix<<<rgrid, NA_RADIX_THREADS, 0, s>>>(S, lower, nn, pass);
         na_radix_compact<<<grid, 256, 0, s>>>(S, lower, upper, nn);
     }
