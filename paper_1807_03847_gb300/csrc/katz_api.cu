@@ -1478,7 +1478,7 @@ katz_status update_swap(katz_handle* h) {
 // at once and then runs repair_finish for each.
 static katz_status repair_levels(katz_handle* h, int64_t& full_levels, int64_t& affected, bool& all_rows);
 static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_levels, int64_t affected,
-                                 bool all_rows);
+                                 bool all_rows, bool c_done = false);
 
 katz_status update_repair(katz_handle* h, katz_info* info) {
     int64_t full_levels = 0, affected = 0;
@@ -1594,8 +1594,9 @@ static katz_status repair_levels(katz_handle* h, int64_t& full_levels, int64_t& 
     return KATZ_OK;
 }
 
+// c_done: c_r of the repaired levels is in place already
 static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_levels, int64_t affected,
-                                 bool all_rows) {
+                                 bool all_rows, bool c_done) {
     const katz_handle::Pending& pd = h->rep;
     cudaError_t e;
     DeviceGraph& g = h->g;
@@ -1603,9 +1604,11 @@ static katz_status repair_finish(katz_handle* h, katz_info* info, int64_t full_l
     const int r = h->r;
     DynBuffers d = h->dyn;
     if (pd.applied) {
-        if ((e = dyn_recompute_c(g, h->b, d, h->p, r, all_rows, h->stream)) != cudaSuccess)
-            return cuda_fail(h, e, "recompute c");
-        h->launches += 1;
+        if (!c_done) {
+            if ((e = dyn_recompute_c(g, h->b, d, h->p, r, all_rows, h->stream)) != cudaSuccess)
+                return cuda_fail(h, e, "recompute c");
+            h->launches += 1;
+        }
         // FP32-certified: a row sum longer than any before widens every
         // level's error bound; the bounds of level r are re-derived with it
         if (h->p.cert && pd.depth > h->p.depth) {
@@ -1738,7 +1741,7 @@ katz_status update_pair_first(katz_handle* h, katz_info* info) {
     }
     h->pair_r = r;
     h->pair_f32_from = f32_from;
-    return repair_finish(h, info, r, n, true);
+    return repair_finish(h, info, r, n, true, true);
 }
 
 katz_status update_pair_second(katz_handle* h, katz_info* info) {
@@ -1754,7 +1757,7 @@ katz_status update_pair_second(katz_handle* h, katz_info* info) {
         return cuda_fail(h, e, "pair split");
     h->launches += 1;
     h->pair_second_used = true;
-    return repair_finish(h, info, r_pair, h->g.n, true);
+    return repair_finish(h, info, r_pair, h->g.n, true, true);
 }
 
 // the checks a handle must pass before it takes update batches

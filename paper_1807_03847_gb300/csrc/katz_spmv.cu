@@ -1374,16 +1374,27 @@ __global__ void pair_fix_hub_rows_kernel(SpmvLayout L, const int64_t* __restrict
 }
 
 // state `st` (0: A, 1: B) of levels 1..r into the handle's walk slots, and of
-// the FP32 roundings into s32
+// the FP32 roundings into s32; c_r = s_1 + ... + s_r on the way, as
+// recompute_c_kernel adds it from the slots (28 us per batch of R-MAT20)
 __global__ void pair_split_kernel(const double* __restrict__ P, int64_t pstride, int r, int f32_from, int st,
-                                  double* walk, IterParams p, const float* __restrict__ t_pair, float* s32) {
+                                  double* walk, IterParams p, const float* __restrict__ t_pair, float* s32,
+                                  double* __restrict__ c, double* __restrict__ c32) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int r64 = min(r, f32_from - 1);
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < p.n; u += stride) {
-        for (int level = 1; level <= r; ++level) {
-            const double* lv = P + (size_t)level * pstride;
-            if (level < f32_from) walk_slot(walk, p, level)[u] = lv[2 * u + st];
-            else ((float*)walk_slot(walk, p, level))[u] = ((const float*)lv)[2 * u + st];
+        double acc = 0.0, acc32 = 0.0;
+        for (int level = 1; level <= r64; ++level) {
+            const double s = (P + (size_t)level * pstride)[2 * u + st];
+            walk_slot(walk, p, level)[u] = s;
+            acc = __dadd_rn(acc, s);
         }
+        for (int level = r64 + 1; level <= r; ++level) {
+            const float s = ((const float*)(P + (size_t)level * pstride))[2 * u + st];
+            ((float*)walk_slot(walk, p, level))[u] = s;
+            acc32 = __dadd_rn(acc32, (double)s);
+        }
+        c[u] = acc;
+        if (p.cert && c32) c32[u] = acc32;
         if (s32) s32[u] = t_pair[2 * u + st];
     }
 }
@@ -1472,7 +1483,7 @@ cudaError_t launch_pair_split(const DeviceGraph& g, const IterBuffers& b, const 
                               int state, const double* P, int64_t pstride, const float* t_pair, cudaStream_t st) {
     const int64_t blocks = std::min<int64_t>(std::max<int64_t>((g.n + 255) / 256, 1), 152 * 8);
     pair_split_kernel<<<(unsigned)blocks, 256, 0, st>>>(P, pstride, r, f32_from, state, (double*)b.walk, p, t_pair,
-                                                        p.cert ? b.s32 : nullptr);
+                                                        p.cert ? b.s32 : nullptr, b.c, b.c32);
     return cudaGetLastError();
 }
 
