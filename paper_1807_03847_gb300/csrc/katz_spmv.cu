@@ -900,10 +900,10 @@ cudaError_t launch_spmv_store(const DeviceGraph& g, const IterBuffers& b, const 
     return spmv_launch(g, b, p, level, st);
 }
 
-// One warp per listed row: the row's s_level recomputed with the lane
-// partition spmv_rows_kernel uses for that row (its row mode is set by its
-// internal index) and the same merges, so a repaired level has the bits of a
-// full recomputation.  CHUNK rows are left to the two hub kernels below,
+// One warp per listed row: the row's s_level recomputed, on FP32 levels with
+// the lane partition spmv_rows_kernel uses for that row (its row mode is set by
+// its internal index) and the same merges, on FP64 levels exactly, so a repaired
+// level has the bits of a full recomputation.  CHUNK rows are left to the two hub kernels below,
 // which split them over warps as the SpMV does.
 template <typename Off>
 __global__ void rows_store_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col, SpmvLayout L,
