@@ -213,7 +213,7 @@ cudaError_t launch_iteration(katz_handle* h, cudaEvent_t* ev_pair = nullptr) {
 cudaError_t launch_first_iteration(katz_handle* h, cudaEvent_t* ev_pair = nullptr) {
     cudaError_t e;
     if (ev_pair && (e = cudaEventRecord(ev_pair[0], h->stream)) != cudaSuccess) return e;
-    if ((e = launch_degree_level(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
+    if ((e = launch_first_level(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
     if (ev_pair && (e = cudaEventRecord(ev_pair[1], h->stream)) != cudaSuccess) return e;
     if ((e = launch_select(h->g, h->b, h->p, h->stream)) != cudaSuccess) return e;
     return launch_count(h->g, h->b, h->p, h->stream);
@@ -970,11 +970,10 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->criterion = KATZ_CRIT_TOPK;
     h->b.use_cond = 0;
     h->ranked = false;
-    h->launches = h->classes_exact ? 3 : 4;  // init_walk, cert_init, theta_0 (one or two kernels)
+    h->launches = h->classes_exact ? 2 : 3;  // cert_init, theta_0 (one or two kernels)
     cudaError_t e;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
     if ((e = cudaMemsetAsync(h->b.ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess) return cuda_fail(h, e, "memset ctrl");
-    if ((e = launch_init_walk(h->g, h->b, p, h->fp32, h->stream)) != cudaSuccess) return cuda_fail(h, e, "init");
     if ((e = launch_cert_init(h->b, p, h->stream)) != cudaSuccess) return cuda_fail(h, e, "init levels");
     const bool prof = h->opts.profile != 0;
     if (h->classes_exact) {
@@ -995,7 +994,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     if (prof && (st = ensure_prof_events(h)) != KATZ_OK) return st;
     if ((e = launch_first_iteration(h, prof ? &h->sp_ev[0] : nullptr)) != cudaSuccess)
         return cuda_fail(h, e, "first iteration");
-    h->launches += 4;  // degree level, select (two), count
+    h->launches += 4;  // first level, select (two), count
     st = run_loop(h, 1);
     if (st != KATZ_OK) return st;
     float ms = 0.f;
@@ -1087,11 +1086,10 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     const int64_t spmv_kernels = iteration_kernels(h) - 3;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
     if ((e = cudaMemsetAsync(h->b.ctrl, 0, CTRL_SPAN, h->stream)) != cudaSuccess ||
-        (e = launch_init_walk(h->g, h->b, p, false, h->stream)) != cudaSuccess ||
         (e = launch_cert_init(h->b, p, h->stream)) != cudaSuccess ||
         (e = launch_crit_init(h->b, h->stream)) != cudaSuccess)
         return cuda_fail(h, e, "init");
-    h->launches += 3;
+    h->launches += 2;
     // Levels are launched four at a time (a launch after the loop stopped, or
     // paused for a sort, returns at once), the control block read in between.
     const bool ranking = criterion == KATZ_CRIT_RANKING;
@@ -1099,7 +1097,7 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     for (int it = 0;;) {
         for (int q = 0; q < 4; ++q, ++it) {
             // level 1 is the degree vector (A 1 = deg), one O(n) pass
-            e = it == 0 ? launch_degree_level(h->g, h->b, p, h->stream) : launch_spmv(h->g, h->b, p, false, h->stream);
+            e = it == 0 ? launch_first_level(h->g, h->b, p, h->stream) : launch_spmv(h->g, h->b, p, false, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "spmv");
             if (ranking)
                 e = launch_ranking_witness(h->g, h->b, p, order, h->stream);

@@ -350,8 +350,6 @@ cudaError_t build_chunk_table(const int64_t* rowptr_new, int64_t row_warp, int64
                               cudaStream_t st);
 cudaError_t launch_validate_csr(const DeviceGraph& g, unsigned long long* d_bad, int64_t* d_degmax,
                                 cudaStream_t st);
-cudaError_t launch_init_walk(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
-                             cudaStream_t st);
 // theta_0 from the kk-th largest degree among rows [a, bend) of one exact
 // degree class (degrees in (lo, lo + 2^bits])
 cudaError_t launch_theta0_class(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int64_t a,
@@ -366,8 +364,8 @@ cudaError_t launch_theta0(const DeviceGraph& g, const IterBuffers& b, const Iter
 cudaError_t launch_convert(const double* in, int64_t n, float* out, double* back, cudaStream_t st);
 // s_1 = alpha deg into its walk slot, nothing else (a full level 1 of a repair)
 cudaError_t launch_degree_store(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
-// level 1 of a ranking (s_1 = alpha deg) in one pass over the rows, fixup included
-cudaError_t launch_degree_level(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
+// the state before the loop and level 1 of a ranking (s_1 = alpha deg) in one pass over the rows
+cudaError_t launch_first_level(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
 cudaError_t launch_spmv(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
                         cudaStream_t st);
 cudaError_t launch_stage(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);

@@ -66,24 +66,6 @@ __global__ void validate_kernel(const Off* __restrict__ rowptr, const int32_t* _
     }
 }
 
-template <typename T>
-__global__ void init_walk_kernel(T* walk, double* c, double* c32, double* lb, double* ub, uint8_t* active,
-                                 IterParams p) {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = tid; v < p.n; v += stride) {
-        walk[v] = (T)1;  // s_0 = omega_0 = 1 (Alg. 1)
-        c[v] = 0.0;      // c_0 = 0
-        if (c32) c32[v] = 0.0;
-        if (lb) {
-            lb[v] = 0.0;
-            ub[v] = 1.0 / 0.0;
-        }
-        active[v] = 1;   // M = V
-    }
-    for (int64_t s = tid; s < p.slots; s += stride) walk[(size_t)s * p.stride + p.n] = (T)0;  // sentinel
-}
-
 // ---------------------------------------------------------------------------
 // theta_0: the k-th largest l_1.  l_1 is an increasing function of the degree
 // (s_1 = alpha deg), so it is l_1 evaluated at the k-th largest degree.
@@ -810,14 +792,6 @@ cudaError_t launch_validate_csr(const DeviceGraph& g, unsigned long long* d_bad,
         validate_kernel<int64_t><<<blocks, 256, 0, st>>>((const int64_t*)g.rowptr, g.col, g.n, g.nnz, d_bad, d_degmax);
     else
         validate_kernel<int32_t><<<blocks, 256, 0, st>>>((const int32_t*)g.rowptr, g.col, g.n, g.nnz, d_bad, d_degmax);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_init_walk(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, bool fp32,
-                             cudaStream_t st) {
-    (void)g;
-    (void)fp32;
-    init_walk_kernel<double><<<grid_for(p.n, 256), 256, 0, st>>>((double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, p);
     return cudaGetLastError();
 }
 

@@ -136,16 +136,25 @@ __device__ __forceinline__ double nn_min(double a, double b) {
     return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
 }
 
+// u joins the candidate list when its lower bound reaches theta_{r-1}.
+// Candidates carry the original id.
+__device__ __forceinline__ void append_candidate(int64_t u, double l, double up, const Epi& e) {
+    if (__double_as_longlong(l) < __double_as_longlong(e.theta_prev)) return;
+    // one atomic per group of lanes that append together
+    cg::coalesced_group grp = cg::coalesced_threads();
+    unsigned long long base = 0;
+    if (grp.thread_rank() == 0) base = atomicAdd(&e.ctrl->n_cand, (unsigned long long)grp.size());
+    const unsigned long long pos = grp.shfl(base, 0) + grp.thread_rank();
+    if (pos < (unsigned long long)e.cand_cap) {
+        e.cand_l[pos] = l;
+        e.cand_u[pos] = up;
+        e.cand_id[pos] = e.perm[u];
+    }
+}
+
 // Finish row u of an FP64 level: s = alpha * sum, c64 += s, bounds, candidate.
 // Finish row u of an FP32 level: s = fl32(alpha_f * sum), c32 += s, bounds, candidate.
-// Candidates carry the original id.
-// ZeroRows: rows without walks so far (sum and c both +0) skip the FP64
-// arithmetic; alpha * +0 and +0 + +0 are +0 in every rounding mode, so the
-// bits are those of the full computation.  Worth it where the FP64 pipe
-// (narrow on this GPU) bounds the pass, as in the degree pass over an R-MAT
-// graph whose rows are mostly isolated nodes; the gather levels, bound by
-// their loads, run the plain epilogue.
-template <typename Acc, bool ZeroRows = false>
+template <typename Acc>
 __device__ __forceinline__ void finish_row(int64_t u, Acc sum, const Epi& e, const IterParams& p) {
     if (e.store_only) {  // dynamic repair: the level value only (and its FP32 rounding at a transition)
         if constexpr (sizeof(Acc) == 8) {
@@ -158,22 +167,12 @@ __device__ __forceinline__ void finish_row(int64_t u, Acc sum, const Epi& e, con
         return;
     }
     double sd, c64, c32 = 0.0;
-    bool zero = false;  // ZeroRows: a node without walks so far, every value of the row is +0
     if constexpr (sizeof(Acc) == 8) {
-        const double c_prev = e.c64[u];
-        if (ZeroRows && __double_as_longlong((double)sum) == 0 && __double_as_longlong(c_prev) == 0) {
-            sd = 0.0;
-            c64 = 0.0;
-            zero = true;
-            ((double*)e.y)[u] = 0.0;
-            if (e.s32) e.s32[u] = 0.0f;
-        } else {
-            sd = __dmul_rn(p.alpha, (double)sum);
-            ((double*)e.y)[u] = sd;
-            if (e.s32) e.s32[u] = f64_to_f32_rn(sd);  // one rounding per row, not per gathered arc
-            c64 = __dadd_rn(c_prev, sd);
-            e.c64[u] = c64;
-        }
+        sd = __dmul_rn(p.alpha, (double)sum);
+        ((double*)e.y)[u] = sd;
+        if (e.s32) e.s32[u] = f64_to_f32_rn(sd);  // one rounding per row, not per gathered arc
+        c64 = __dadd_rn(e.c64[u], sd);
+        e.c64[u] = c64;
         if (e.c32) c32 = e.c32[u];
     } else {
         const float sf = __fmul_rn(p.alpha_f, (float)sum);
@@ -184,26 +183,15 @@ __device__ __forceinline__ void finish_row(int64_t u, Acc sum, const Epi& e, con
         c64 = e.c64[u];
     }
     if (e.active[u]) {
-        double l = 0.0, up = 0.0;  // zero: c = s = +0, both bounds are +0 in either mode
-        if (!ZeroRows || !zero || __double_as_longlong(c32) != 0) node_bounds(c64, c32, sd, p, e.bs, l, up);
+        double l, up;
+        node_bounds(c64, c32, sd, p, e.bs, l, up);
         if (p.cert) {  // both the new and the stored bounds are valid: keep the tighter ones
             l = nn_max(l, e.lb[u]);
             up = nn_min(up, e.ub[u]);
         }
         e.lb[u] = l;  // read by the deactivation count of this level
         e.ub[u] = up;
-        if (__double_as_longlong(l) >= __double_as_longlong(e.theta_prev)) {
-            // one atomic per group of lanes that append together
-            cg::coalesced_group grp = cg::coalesced_threads();
-            unsigned long long base = 0;
-            if (grp.thread_rank() == 0) base = atomicAdd(&e.ctrl->n_cand, (unsigned long long)grp.size());
-            const unsigned long long pos = grp.shfl(base, 0) + grp.thread_rank();
-            if (pos < (unsigned long long)e.cand_cap) {
-                e.cand_l[pos] = l;
-                e.cand_u[pos] = up;
-                e.cand_id[pos] = e.perm[u];
-            }
-        }
+        append_candidate(u, l, up, e);
     }
 }
 
@@ -662,22 +650,58 @@ __device__ __forceinline__ Epi make_epi(void* y, double* c64, double* c32, doubl
                ctrl->theta_prev, bstate(ctrl, p), 0, s32};
 }
 
-// Level 1 of a ranking as one pass over all rows, any row mode: s_0 = 1, so
-// the exact sum of a row is its length (A 1 = deg) and no walk value is read;
-// s_1 = alpha deg goes through the epilogue of every level, in a grid sized
-// for O(n) work (no chunk partials: no fixup follows).  The bits are those a
-// gather level would give: an exact sum of ones, rounded once.
+// The state of Algorithm 1 before its loop (s_0 = omega_0 = 1, c_0 = 0, M = V)
+// and level 1, as one pass over all rows, any row mode: s_0 = 1, so
+// the exact sum of a row is its length (A 1 = deg) and no walk value is read.
+// The values depend on the degree alone: those of the degrees below
+// SHORT_DEGREES, nearly all rows, are computed once per block, since the FP64
+// pipe (narrow on this GPU) bounded the pass; the bits are those a gather
+// level would give, an exact sum of ones rounded once.  Bound by its writes
+// (5.8 TB/s at n = 2^27).  In place of a pass that set the state and one that
+// read it back: 71 -> 33 us on R-MAT22, 2.40 -> 1.13 ms at n = 2^27.
+constexpr int SHORT_DEGREES = 64;
+
 template <typename Off>
-__global__ void degree_level_kernel(const Off* __restrict__ rowptr, int64_t n, double* walk, double* c64,
-                                    double* c32, double* lb, double* ub, uint8_t* active,
-                                    const int32_t* __restrict__ perm, double* cand_l, double* cand_u,
-                                    int32_t* cand_id, int64_t cand_cap, float* s32, Ctrl* ctrl, IterParams p) {
-    if (ctrl->stop) return;
+__global__ void __launch_bounds__(BLOCK)
+first_level_kernel(const Off* __restrict__ rowptr, int64_t n, double* walk, double* c64, double* c32, double* lb,
+                   double* ub, uint8_t* active, const int32_t* __restrict__ perm, double* cand_l, double* cand_u,
+                   int32_t* cand_id, int64_t cand_cap, float* s32, Ctrl* ctrl, IterParams p) {
+    __shared__ double t_s[SHORT_DEGREES], t_l[SHORT_DEGREES], t_u[SHORT_DEGREES];
     const Epi ep = make_epi(walk_slot(walk, p, 1), c64, c32, lb, ub, active, perm, cand_l, cand_u, cand_id,
                             cand_cap, ctrl, p, (p.cert && 1 < ctrl->f32_from) ? s32 : nullptr);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += stride)
-        finish_row<double, true>(u, (double)((int64_t)rowptr[u + 1] - (int64_t)rowptr[u]), ep, p);
+    // s_1 = alpha deg, c_1 = 0 + s_1, and the bounds, within [0, inf] in cert mode
+    auto level1 = [&](int64_t deg, double& s, double& l, double& u) {
+        s = __dmul_rn(p.alpha, (double)deg);
+        node_bounds(__dadd_rn(0.0, s), 0.0, s, p, ep.bs, l, u);
+        if (p.cert) {
+            l = nn_max(l, 0.0);
+            u = nn_min(u, 1.0 / 0.0);
+        }
+    };
+    if (threadIdx.x < SHORT_DEGREES) level1(threadIdx.x, t_s[threadIdx.x], t_l[threadIdx.x], t_u[threadIdx.x]);
+    __syncthreads();
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t q = t0; q < p.slots; q += stride) walk[(size_t)q * p.stride + p.n] = 0.0;  // sentinel
+    for (int64_t u = t0; u < n; u += stride) {
+        const int64_t deg = (int64_t)rowptr[u + 1] - (int64_t)rowptr[u];
+        double s, l, up;
+        if (deg < SHORT_DEGREES) {
+            s = t_s[deg];
+            l = t_l[deg];
+            up = t_u[deg];
+        } else {
+            level1(deg, s, l, up);
+        }
+        walk[u] = 1.0;  // slot 0
+        ((double*)ep.y)[u] = s;
+        if (ep.s32) ep.s32[u] = f64_to_f32_rn(s);
+        c64[u] = s;
+        if (c32) c32[u] = 0.0;
+        active[u] = 1;
+        lb[u] = l;
+        ub[u] = up;
+        append_candidate(u, l, up, ep);
+    }
 }
 
 // Six 256-thread blocks per SM (40 registers): the gathers need the warps in
@@ -882,14 +906,15 @@ cudaError_t launch_degree_store(const DeviceGraph& g, const IterBuffers& b, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_degree_level(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
-    const int64_t blocks = std::min<int64_t>(std::max<int64_t>((g.n + BLOCK - 1) / BLOCK, 1), 152 * 8);
+cudaError_t launch_first_level(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st) {
+    // one wave: six blocks of 256 threads per SM (40 registers)
+    const int64_t blocks = std::min<int64_t>(std::max<int64_t>((g.n + BLOCK - 1) / BLOCK, 1), 152 * 6);
     if (g.off64)
-        degree_level_kernel<int64_t><<<(unsigned)blocks, BLOCK, 0, st>>>(
+        first_level_kernel<int64_t><<<(unsigned)blocks, BLOCK, 0, st>>>(
             (const int64_t*)g.rowptr, g.n, (double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, g.perm, b.cand_l,
             b.cand_u, b.cand_id, b.cand_cap, b.s32, b.ctrl, p);
     else
-        degree_level_kernel<int32_t><<<(unsigned)blocks, BLOCK, 0, st>>>(
+        first_level_kernel<int32_t><<<(unsigned)blocks, BLOCK, 0, st>>>(
             (const int32_t*)g.rowptr, g.n, (double*)b.walk, b.c, b.c32, b.lb, b.ub, b.active, g.perm, b.cand_l,
             b.cand_u, b.cand_id, b.cand_cap, b.s32, b.ctrl, p);
     return cudaGetLastError();

@@ -111,3 +111,31 @@ def test_rebuilt_rows_at_the_mode_edges(seed, kinds):
         assert np.array_equal(h.walk(i), fresh.walk(i))
     h.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("top", [1, 62, 63, 64, 65, 700])
+def test_first_level_on_both_sides_of_its_table(top, precision):
+    """Level 1 is alpha deg and its bounds, of degrees in the block's table and
+    past it; FP64 bounds are the formula's bits, certified ones contain it and
+    are wider by a few dozen roundings at most (1e-13 relative)."""
+    import paper_1807_03847_gb300 as K
+
+    g = _graph({d: 400 // d + 2 for d in {1, 2, max(top - 1, 1), top}}, 5)
+    deg = np.diff(g.rowptr)
+    h = K.Katz(g.rowptr, g.col, K.katz_default_opts(r_max=1, precision=precision))
+    k = 5
+    for _ in range(2):  # the second pass finds the first one's buffers
+        info = h.rank(0.0, k, 1e-300, check=False)
+        s = info.alpha * deg.astype(np.float64)
+        low, up = s + info.alpha * s, s + (info.alpha * info.gamma) * s
+        lo, hi = h.bounds()[:2]
+        if precision:
+            assert (lo <= low * (1 + 1e-15)).all() and (hi >= up * (1 - 1e-15)).all()  # their own roundings
+            np.testing.assert_allclose(lo, low, rtol=1e-13)
+            np.testing.assert_allclose(hi, up, rtol=1e-13)
+        else:
+            assert np.array_equal(lo, low) and np.array_equal(hi, up)
+        assert np.array_equal(h.walk(1), s) and np.array_equal(h.walk(0), np.ones(g.n))
+        assert np.array_equal(h.ranking(k), np.lexsort((np.arange(g.n), -deg))[:k])
+    h.close()
