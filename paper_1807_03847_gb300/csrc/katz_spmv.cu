@@ -314,10 +314,10 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t n) {
     return r;
 }
 
-// a += the non-negative terms v (zeros add nothing)
+// a += the non-negative terms v
 template <int G>
 __device__ __forceinline__ void xacc_add_group(XAcc& a, const double (&v)[G]) {
-    uint32_t hmax = 0u, hmin = ~0u;  // of the upper words; hmin of the nonzero ones, less 1
+    uint32_t hmax = 0u, hmin = ~0u;  // of the upper words; hmin of those that are not 0, less 1
 #pragma unroll
     for (int q = 0; q < G; ++q) {
         const uint32_t hi = (uint32_t)__double2hiint(v[q]);
@@ -329,17 +329,19 @@ __device__ __forceinline__ void xacc_add_group(XAcc& a, const double (&v)[G]) {
         if (a.E) shr128(a, e - a.E);
         a.E = e;
     }
-    // common case: every nonzero term within XF binades below E, and E so far
-    // above the subnormals that one (its upper word may be 0) adds nothing
+    // common case: every term within XF binades below E, or nothing: a zero, or
+    // a subnormal so small that its upper word is 0 as well, which E > 127 puts
+    // below W's last bit
     if (a.E > 127 && hmin >= ((uint32_t)(a.E - XF) << 20) - 1u) {
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             const uint32_t hi = (uint32_t)__double2hiint(v[q]), lo = (uint32_t)__double2loint(v[q]);
-            // a zero's exponent field 0 makes t huge: all three shifts then give
-            // 0 (the last one drops the implicit bit set here)
-            const uint32_t t = (uint32_t)(a.E + 1) - (hi >> 20);  // 1..32
-            const uint32_t m1 = (hi & 0xFFFFFu) | 0x100000u;
-            add96(a, shl_clamp(lo, 32u - t), __funnelshift_lc(lo, m1, 32u - t), shr_clamp(m1, t));
+            // (m1:lo) << (32 - t).  Where hi is 0, t is above 128 and all three
+            // words are 0 whatever lo holds: 32 - t wraps far above 32, the
+            // funnel shift stops at 32 and leaves m1, which has no implicit bit then
+            const uint32_t t = (uint32_t)(a.E + 1) - (hi >> 20);  // else 1..32
+            const uint32_t m1 = (hi & 0xFFFFFu) | min(hi, 0x100000u);
+            add96(a, shl_clamp(lo, 32u - t), __funnelshift_rc(lo, m1, t), shr_clamp(m1, t));
         }
     } else {
         for (int q = 0; q < G; ++q) {
