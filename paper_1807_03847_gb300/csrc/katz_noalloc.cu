@@ -43,6 +43,7 @@ using katz::last_block;
 
 constexpr int NA_BINS = 65536;          // 16-bit digits
 constexpr int NA_CAP = KATZ_MAX_K;      // candidates held
+static_assert((NA_CAP & (NA_CAP - 1)) == 0, "a power of two: places are masked with it");
 constexpr int NA_MAX_DEVICES = 64;
 constexpr int NA_GROUPS = 8192;
 constexpr int NA_GROUP_THREADS = 512;
@@ -335,6 +336,10 @@ __global__ void __launch_bounds__(katz::RANK_THREADS) na_rank(NoAllocScratch* S,
     }
 }
 
+// the candidate that a word of the order names: within the candidate arrays
+// whatever an overlapping call wrote there
+__host__ __device__ constexpr unsigned int place_of(unsigned int word) { return word & (NA_CAP - 1u); }
+
 // every node outside the top-k must be eps-separated from the k-th (only the
 // nodes whose upper bound reaches theta need their lower bound looked at),
 // and adjacent top-k pairs from each other; the last block gives the verdict
@@ -368,7 +373,7 @@ na_cross(NoAllocScratch* S, const double* __restrict__ lower, const double* __re
     }
     const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
     for (long long r = t + 1; r < k; r += (long long)gridDim.x * 256)
-        if (__dsub_rn(S->cand_u[S->hist[r]], eps) >= bound_of(S->cand_key[S->hist[r - 1]])) ++c;
+        if (__dsub_rn(S->cand_u[place_of(S->hist[r])], eps) >= bound_of(S->cand_key[place_of(S->hist[r - 1])])) ++c;
     for (int off = 16; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&S->cross, c);
     if (last_block(&S->ticket) && threadIdx.x == 0)
