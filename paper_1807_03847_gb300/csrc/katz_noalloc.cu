@@ -29,7 +29,6 @@
 // k = 1000 (230 of them in global atomics on the few bins that hold most
 // bounds); these kernels take 90 us, launches included.
 #include <cuda_runtime.h>
-#include <math_constants.h>
 #include <stdint.h>
 
 #include <mutex>
@@ -120,7 +119,7 @@ na_groups(NoAllocScratch* S, const double* __restrict__ lower, long long n, long
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const long long v = (long long)(i + q) * T + (t ^ mix(i + q));
-            x[q] = v < n ? __ldg(lower + v) : -CUDART_INF;  // its key is below any other's
+            x[q] = v < n ? __ldg(lower + v) : __longlong_as_double(-1ll);  // key 0: no other is below it, not even a NaN's
         }
 #pragma unroll
         for (int q = 0; q < U; ++q) m = max(m, (unsigned int)(order_bits(x[q]) >> 32));
