@@ -1042,6 +1042,36 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     return KATZ_OK;
 }
 
+// The ranking criterion's buffers, all of them or none (a restored handle
+// comes with its order alone, and an earlier call may have found no memory).
+static cudaError_t ensure_sort_buffers(katz_handle* h) {
+    RadixBuffers& rs = h->rs;
+    if (h->rank_ids && rs.sums) return cudaSuccess;
+    const int64_t n = h->g.n, cnt = 256 * radix_tiles(n);
+    cudaError_t e = cudaSuccess;
+    auto A = [&](auto** p, int64_t count) {
+        if (e == cudaSuccess && !*p) e = dmalloc(h, p, (size_t)count);
+    };
+    A(&h->rank_ids, n);
+    for (int q = 0; q < 2; ++q) {
+        A(&rs.hi[q], n);
+        A(&rs.val[q], n);
+    }
+    A(&rs.counts, cnt);
+    A(&rs.offs, cnt);
+    A(&rs.sums, scan_blocks(cnt));
+    if (e == cudaSuccess) return e;
+    for (int q = 0; q < 2; ++q) {
+        dfree(h, rs.hi[q]);
+        dfree(h, rs.val[q]);
+    }
+    dfree(h, rs.counts);
+    dfree(h, rs.offs);
+    dfree(h, rs.sums);
+    rs = RadixBuffers();
+    return e;
+}
+
 katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, const int32_t* pair, double eps,
                       katz_info* info) {
     if (!h) return KATZ_EINVAL;
@@ -1068,18 +1098,8 @@ katz_status katz_rank(katz_h h, double alpha, int32_t criterion, int64_t k, cons
     if (st != KATZ_OK) return st;
     IterParams& p = h->p;
     cudaError_t e;
-    if (criterion == KATZ_CRIT_RANKING && !h->rank_ids) {
-        RadixBuffers& rs = h->rs;
-        const int64_t cnt = 256 * radix_tiles(n);
-        if ((e = dmalloc(h, &h->rank_ids, (size_t)n)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.hi[0], (size_t)n)) != cudaSuccess || (e = dmalloc(h, &rs.hi[1], (size_t)n)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.val[0], (size_t)n)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.val[1], (size_t)n)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.counts, (size_t)cnt)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.offs, (size_t)cnt)) != cudaSuccess ||
-            (e = dmalloc(h, &rs.sums, (size_t)scan_blocks(cnt))) != cudaSuccess)
-            return cuda_fail(h, e, "cudaMalloc ranking buffers");
-    }
+    if (criterion == KATZ_CRIT_RANKING && (e = ensure_sort_buffers(h)) != cudaSuccess)
+        return cuda_fail(h, e, "cudaMalloc ranking buffers");
     h->criterion = criterion;
     h->ranked = false;
     h->launches = 0;
