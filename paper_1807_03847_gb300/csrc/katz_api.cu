@@ -102,7 +102,7 @@ katz_status init_handle_runtime(katz_handle* h) {
 // Scratch of the ranking loop that does not depend on the ranking's size.
 katz_status alloc_rank_scratch(katz_handle* h) {
     cudaError_t e;
-    if ((e = dmalloc(h, &h->d_deghist, (size_t)deg_hist_top(h->D) + 1)) != cudaSuccess)
+    if ((e = dmalloc_needed(h, &h->d_deghist, (size_t)deg_hist_top(h->D) + 1)) != cudaSuccess)
         return cuda_fail(h, e, "cudaMalloc rank scratch");
     return KATZ_OK;
 }
@@ -145,18 +145,12 @@ katz_status ensure_iter_buffers(katz_handle* h) {
     const int64_t stride = ((n + 1) + 31) / 32 * 32;
     cudaError_t e;
 #define KALLOC(ptr, cnt)                                          \
-    if ((e = dmalloc(h, &(ptr), (size_t)(cnt))) != cudaSuccess) {    \
+    if ((e = dmalloc_needed(h, &(ptr), (size_t)(cnt))) != cudaSuccess) { \
         free_iter(h);                                             \
         return cuda_fail(h, e, "cudaMalloc " #ptr);               \
     }
     char* walk = nullptr;
-    if (h->g.stage.n_items > 0 && dmalloc(h, &walk, (size_t)slots * stride * esz) != cudaSuccess) {
-        // the staged gathers give their memory back before a ranking fails for it
-        cudaGetLastError();
-        stage_free(h);
-        drop_graph(h);
-    }
-    if (!walk) KALLOC(walk, (size_t)slots * stride * esz);
+    KALLOC(walk, (size_t)slots * stride * esz);
     b.walk = walk;
     KALLOC(b.c, n);
     KALLOC(b.lb, n);  // bounds of the active nodes at the last level (cert mode: monotone)
@@ -226,6 +220,13 @@ void drop_graph(katz_handle* h) {
     if (h->graph) cudaGraphDestroy(h->graph);
     h->graph_exec = nullptr;
     h->graph = nullptr;
+}
+
+// The staged gathers' memory for something that needs it more; the captured
+// loop holds their pointers.
+void stage_give_back(katz_handle* h) {
+    stage_free(h);
+    drop_graph(h);
 }
 
 // Capture one iteration as the body of a conditional while node; the
@@ -1050,7 +1051,7 @@ static cudaError_t ensure_sort_buffers(katz_handle* h) {
     const int64_t n = h->g.n, cnt = 256 * radix_tiles(n);
     cudaError_t e = cudaSuccess;
     auto A = [&](auto** p, int64_t count) {
-        if (e == cudaSuccess && !*p) e = dmalloc(h, p, (size_t)count);
+        if (e == cudaSuccess && !*p) e = dmalloc_needed(h, p, (size_t)count);
     };
     A(&h->rank_ids, n);
     for (int q = 0; q < 2; ++q) {
@@ -1200,7 +1201,7 @@ katz_status katz_get_bounds(katz_h h, double* lower, double* upper, double* err)
     double* de = err;
     if (!dev) {
         if (!h->d_scratch) {
-            if ((e = dmalloc(h, &h->d_scratch, 3 * (size_t)n)) != cudaSuccess) return cuda_fail(h, e, "cudaMalloc");
+            if ((e = dmalloc_needed(h, &h->d_scratch, 3 * (size_t)n)) != cudaSuccess) return cuda_fail(h, e, "cudaMalloc");
         }
         dl = lower ? h->d_scratch : nullptr;
         du = upper ? h->d_scratch + n : nullptr;
@@ -1230,7 +1231,8 @@ katz_status katz_get_walk(katz_h h, int32_t i, double* s_out) {
     double* dst = s_out;
     const bool dev = is_device_ptr(s_out);
     if (!dev) {
-        if (!h->d_scratch && (e = dmalloc(h, &h->d_scratch, 3 * (size_t)n)) != cudaSuccess) return cuda_fail(h, e, "cudaMalloc");
+        if (!h->d_scratch && (e = dmalloc_needed(h, &h->d_scratch, 3 * (size_t)n)) != cudaSuccess)
+            return cuda_fail(h, e, "cudaMalloc");
         dst = h->d_scratch;
     }
     if ((e = launch_walk_out(h->g, h->b, h->p, i, h->fp32, dst, h->stream)) != cudaSuccess) return cuda_fail(h, e, "walk");

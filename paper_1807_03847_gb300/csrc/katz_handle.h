@@ -173,6 +173,20 @@ inline void dfree_on(void* p, cudaStream_t st) {
 bool stage_wanted(const katz_handle* h, int64_t head_arcs);
 cudaError_t stage_build(katz_handle* h, int64_t head_arcs);
 void stage_free(katz_handle* h);
+void stage_give_back(katz_handle* h);
+
+// dmalloc for what a call cannot do without: where it finds no memory, the
+// staged gathers, which are optional, give theirs back first (the handle goes on
+// with plain gathers).  For calls with no launch of theirs queued yet.
+template <typename X>
+cudaError_t dmalloc_needed(katz_handle* h, X** p, size_t count) {
+    const cudaError_t e = dmalloc(h, p, count);
+    if (e != cudaErrorMemoryAllocation || h->g.stage.n_items == 0) return e;
+    cudaGetLastError();
+    stage_give_back(h);
+    return dmalloc(h, p, count);
+}
+
 katz_status init_handle_runtime(katz_handle* h);
 katz_status ensure_iter_buffers(katz_handle* h);
 katz_status alloc_rank_scratch(katz_handle* h);
