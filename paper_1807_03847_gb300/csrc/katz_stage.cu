@@ -188,7 +188,10 @@ cudaError_t stage_build(katz_handle* h, int64_t head_arcs) {
     const size_t cells = (size_t)windows * STAGE_BANDS;
     const int64_t band_arcs = ((g.nnz + STAGE_BANDS - 1) / STAGE_BANDS + STAGE_ASSIGN - 1) / STAGE_ASSIGN * STAGE_ASSIGN;
     unsigned int* counts = nullptr;
-    if ((e = dmalloc(h, &counts, cells)) != cudaSuccess) return e;
+    if ((e = dmalloc(h, &counts, cells)) != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    }
     std::vector<unsigned int> cnt(cells), first(cells + 1);
     e = cudaMemsetAsync(counts, 0, cells * sizeof(unsigned int), h->stream);
     if (e == cudaSuccess)
