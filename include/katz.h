@@ -113,10 +113,13 @@ typedef struct {
                               together and a line fetched from DRAM serves several gathers;
                               -1 keeps them in original-id order; 0 (default): 1 when
                               n >= 2^25 (walk vectors several times larger than L2) and the
-                              handle keeps its history, else -1: without history such a
-                              handle stages its gathers (about 4 bytes per arc and 10 per
-                              arc into the low-degree rows, at most a quarter of the free
-                              memory).  Results are the same bits either way. */
+                              handle does not stage its gathers, else -1.  Whatever the
+                              order, a handle of that size without history stages them
+                              where they would mostly miss L2 (ids not near their
+                              neighbours'): about 4 bytes per arc and 10 per arc into the
+                              low-degree rows, at most a quarter of the free memory, given
+                              back when a call on the handle finds no other.  Results are
+                              the same bits either way. */
     int32_t reserved;      /* set to 0 */
 } katz_opts;
 

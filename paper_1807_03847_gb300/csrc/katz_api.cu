@@ -845,9 +845,10 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
     // then the low-degree rows reordered inside their classes by anchor
     // (katz_opts.locality); the rows of degree > 16 keep their places, the
     // staging column array holds the old tail
-    const bool locality =
-        (h->opts.locality > 0 || (h->opts.locality == 0 && n >= ((int64_t)1 << 25) && !stage_wanted(h, head_arcs))) &&
-        n - row_thread > 1;
+    bool staged = false;
+    KCHK2(stage_pays(h, head_arcs, &staged), "staged gathers");
+    const bool locality = (h->opts.locality > 0 || (h->opts.locality == 0 && n >= ((int64_t)1 << 25) && !staged)) &&
+                          n - row_thread > 1;
     if (locality) {
         const int64_t m = n - row_thread, cnt = 256 * radix_tiles(m);
         RadixBuffers rs;
@@ -916,7 +917,7 @@ katz_status katz_create_csr(katz_h* out, int64_t n, int64_t nnz, const int64_t* 
         return KATZ_EINVAL;
     }
 #undef KCHK2
-    KCHK(stage_build(h, head_arcs), "staged gathers");
+    if (staged) KCHK(stage_build(h), "staged gathers");
     if ((st = alloc_rank_scratch(h)) != KATZ_OK) {
         katz_destroy(h);
         return st;

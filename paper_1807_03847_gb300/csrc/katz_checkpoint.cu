@@ -336,7 +336,9 @@ katz_status katz_restore(katz_h* out, const void* buf, uint64_t bytes, const kat
                     : cudaMemcpy(&narrow, (int32_t*)g.rowptr + STAGE_HOT, sizeof(int32_t), cudaMemcpyDeviceToHost);
         if (!g.off64) head_arcs = narrow;
     }
-    if (e != cudaSuccess || (e = stage_build(h, head_arcs)) != cudaSuccess) {
+    bool staged = false;
+    if (e != cudaSuccess || (e = stage_pays(h, head_arcs, &staged)) != cudaSuccess ||
+        (staged && (e = stage_build(h)) != cudaSuccess)) {
         st = cuda_fail(h, e, "staged gathers");
         katz_destroy(h);
         return st;

@@ -169,9 +169,9 @@ inline void dfree_on(void* p, cudaStream_t st) {
 }
 
 // staged gathers of the handle's graph (katz_stage.cu); head_arcs: arcs of the
-// rows below STAGE_HOT
-bool stage_wanted(const katz_handle* h, int64_t head_arcs);
-cudaError_t stage_build(katz_handle* h, int64_t head_arcs);
+// rows below STAGE_HOT.  stage_pays waits for the handle's stream.
+cudaError_t stage_pays(katz_handle* h, int64_t head_arcs, bool* pays);
+cudaError_t stage_build(katz_handle* h);
 void stage_free(katz_handle* h);
 void stage_give_back(katz_handle* h);
 

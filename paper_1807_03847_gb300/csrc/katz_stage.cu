@@ -56,6 +56,72 @@ constexpr int STAGE_ALIGN = 32;              // places of a segment start at a m
 constexpr int STAGE_MAX_WINDOWS = 1 << 15;   // 128 KB of counters in shared memory
 constexpr int STAGE_HIST_BLOCKS = 10;        // per band
 constexpr int STAGE_ASSIGN = 2048;           // arcs per block of the assignment; a band is a multiple of it
+constexpr int STAGE_CACHED = 1024;           // windows that a plain gather may find in L2 (64 MB of FP64)
+constexpr int STAGE_RUNS = 64;               // sampled runs per band, of STAGE_RUN arcs each
+constexpr int STAGE_RUN = 1024;
+
+int64_t stage_windows(int64_t n) { return (n - STAGE_HOT + STAGE_WIN - 1) / STAGE_WIN; }
+
+int64_t stage_band_arcs(int64_t nnz) {
+    return ((nnz + STAGE_BANDS - 1) / STAGE_BANDS + STAGE_ASSIGN - 1) / STAGE_ASSIGN * STAGE_ASSIGN;
+}
+
+// A sample of the arcs of one band (a block): out[0] += its cold arcs, out[1] +=
+// those outside the STAGE_CACHED windows of the vector that the band uses most.
+__global__ void __launch_bounds__(STAGE_RUN)
+stage_sample_kernel(const int32_t* __restrict__ col, int64_t nnz, int64_t band_arcs, int hot_windows, int windows,
+                    unsigned long long* out) {
+    extern __shared__ unsigned int h[];
+    __shared__ unsigned int s_cold, s_above, s_held;
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int q = tid; q < windows; q += STAGE_RUN) h[q] = 0;
+    if (tid == 0) s_cold = 0;
+    __syncthreads();
+    const int64_t begin = blockIdx.x * band_arcs, end = min(nnz, begin + band_arcs);
+    const int64_t step = max((end - begin) / STAGE_RUNS, (int64_t)STAGE_RUN);
+    unsigned int cold = 0;
+#pragma unroll 8
+    for (int r = 0; r < STAGE_RUNS; ++r) {
+        const int64_t j = begin + r * step + tid;
+        const int w = j < end ? col[j] >> STAGE_BITS : -1;
+        // lanes of one window add once: near neighbours share theirs
+        const unsigned peers = __match_any_sync(0xffffffffu, w);
+        if (w >= 0 && lane == __ffs(peers) - 1) atomicAdd(&h[w], (unsigned)__popc(peers));
+        cold += w >= hot_windows;
+    }
+    cold = __reduce_add_sync(0xffffffffu, cold);
+    if (lane == 0) atomicAdd(&s_cold, cold);
+    // the smallest count that at most STAGE_CACHED windows exceed, and the cold
+    // arcs of the windows that do
+    unsigned int lo = 0, hi = STAGE_RUNS * STAGE_RUN;
+    for (bool last = false;; last = lo == hi) {
+        if (tid == 0) s_above = s_held = 0;
+        __syncthreads();
+        const unsigned int mid = (lo + hi) / 2;
+        unsigned int above = 0, held = 0;
+        for (int q = tid; q < windows; q += STAGE_RUN)
+            if (h[q] > mid) {
+                ++above;
+                held += q >= hot_windows ? h[q] : 0u;
+            }
+        above = __reduce_add_sync(0xffffffffu, above);
+        held = __reduce_add_sync(0xffffffffu, held);
+        if (lane == 0) {
+            atomicAdd(&s_above, above);
+            atomicAdd(&s_held, held);
+        }
+        __syncthreads();
+        above = s_above;
+        __syncthreads();  // read before the next round's zeroes
+        if (last) break;
+        if (above <= STAGE_CACHED) hi = mid;
+        else lo = mid + 1;
+    }
+    if (tid == 0 && s_cold) {
+        atomicAdd(&out[0], s_cold);
+        atomicAdd(&out[1], s_cold - s_held);
+    }
+}
 
 // arcs of every band into every window (gridDim.y: the band)
 __global__ void __launch_bounds__(1024)
@@ -167,26 +233,67 @@ void stage_free(katz_handle* h) {
 // Worth it where many arcs are cold.  In a symmetric graph as many arcs lead
 // into the rows from STAGE_HOT on as leave them; for a directed one that is an
 // estimate.  The places must fit 32 bits and the windows' counters one block.
-bool stage_wanted(const katz_handle* h, int64_t head_arcs) {
+static bool stage_wanted(const katz_handle* h, int64_t head_arcs) {
     const int64_t n = h->g.n, nnz = h->g.nnz, cold = nnz - head_arcs;
     if (n < STAGE_MIN_N || h->opts.keep_history || cold < nnz / 8) return false;
-    const int64_t windows = (n - STAGE_HOT + STAGE_WIN - 1) / STAGE_WIN;
+    const int64_t windows = stage_windows(n);
     return windows <= STAGE_MAX_WINDOWS &&
            STAGE_HOT + cold + windows * STAGE_BANDS * STAGE_ALIGN <= (int64_t)0xffffffff;
+}
+
+// Whether the graph's gathers would miss: of a sample of the cold arcs, three
+// in ten or more lie outside the windows that their band uses most, as many as
+// half of L2 holds.  Where ids are near their neighbours' (rings, grids, banded
+// matrices) plain gathers hit, and a window's arcs all come from one band, so
+// that one warp does their staging and every arc's place comes from one counter.
+// At n = 2^25 + 11, 8 arcs a row (three in four of them cold), by the share of
+// sampled cold arcs that miss: us a level with plain gathers, with staged ones:
+//   ring 0: 735, 4058    grid 0: 633, 2228    neighbours within 2^20 .03: 1231,
+//   2636    2^22 .11: 1623, 1985    6 x 2^20 .37: 2250, 1787    2^24 .84: 3113,
+//   1707    ring with a tenth of its edges random .06: 1101, 3520    three tenths
+//   .22: 1954, 2832    half .40: 2603, 2374    seven tenths .58: 2936, 2069
+// G(n, m) and Chung-Lu graphs have shares of .76 to .92.  The creates of the
+// ring and the grid: 8.0 and 6.9 ms plain, 98 and 28 staged.  The sample reads
+// 2 M arcs.
+cudaError_t stage_pays(katz_handle* h, int64_t head_arcs, bool* pays) {
+    *pays = false;
+    if (!stage_wanted(h, head_arcs)) return cudaSuccess;
+    constexpr int hot_windows = (int)(STAGE_HOT / STAGE_WIN);
+    const int windows = hot_windows + (int)stage_windows(h->g.n);
+    unsigned long long* sums = nullptr;
+    unsigned long long* out = (unsigned long long*)(h->h_small + H_SMALL - 16);
+    cudaError_t e = dmalloc(h, &sums, 2);
+    if (e != cudaSuccess) {  // no memory: plain gathers
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    }
+    e = cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), h->stream);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(stage_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (hot_windows + STAGE_MAX_WINDOWS) * (int)sizeof(unsigned int));
+    if (e == cudaSuccess) {
+        stage_sample_kernel<<<STAGE_BANDS, STAGE_RUN, (size_t)windows * sizeof(unsigned int), h->stream>>>(
+            h->g.col, h->g.nnz, stage_band_arcs(h->g.nnz), hot_windows, windows, sums);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out, sums, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    dfree(h, sums);
+    if (e == cudaSuccess) *pays = out[0] > 0 && 10 * out[1] >= 3 * out[0];
+    return e;
 }
 
 // The staged gathers of the graph a handle holds (its final internal order).
 // Without the memory for them the handle goes on with plain gathers.  Waits
 // for the handle's stream.
-cudaError_t stage_build(katz_handle* h, int64_t head_arcs) {
+cudaError_t stage_build(katz_handle* h) {
     DeviceGraph& g = h->g;
-    if (!stage_wanted(h, head_arcs)) return cudaSuccess;
     const uint32_t hot = (uint32_t)STAGE_HOT;
-    const int64_t span = g.n - STAGE_HOT;
-    const int64_t windows = (span + STAGE_WIN - 1) / STAGE_WIN;
+    const int64_t windows = stage_windows(g.n);
     cudaError_t e;
     const size_t cells = (size_t)windows * STAGE_BANDS;
-    const int64_t band_arcs = ((g.nnz + STAGE_BANDS - 1) / STAGE_BANDS + STAGE_ASSIGN - 1) / STAGE_ASSIGN * STAGE_ASSIGN;
+    const int64_t band_arcs = stage_band_arcs(g.nnz);
     unsigned int* counts = nullptr;
     if ((e = dmalloc(h, &counts, cells)) != cudaSuccess) {
         cudaGetLastError();
