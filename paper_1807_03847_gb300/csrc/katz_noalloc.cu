@@ -177,11 +177,12 @@ na_groups(NoAllocScratch* S, const double* __restrict__ lower, long long n, long
 }
 
 // a candidate's place in the buffer, one atomic per warp; the buffer keeps the
-// first NA_CAP (more: the count says so, and the radix pass starts over)
-__device__ __forceinline__ void add_candidate(NoAllocScratch* S, bool take, double l, const double* upper,
+// first NA_CAP (more: the count says so, and the radix pass starts over).  False
+// once the buffer was full before this warp's.
+__device__ __forceinline__ bool add_candidate(NoAllocScratch* S, bool take, double l, const double* upper,
                                               long long v) {
     const unsigned m = __ballot_sync(0xffffffffu, take);
-    if (!m) return;
+    if (!m) return true;
     const int lane = threadIdx.x & 31;
     unsigned long long base = 0;
     if (lane == __ffs(m) - 1) base = atomicAdd(&S->cand_count, (unsigned long long)__popc(m));
@@ -192,6 +193,7 @@ __device__ __forceinline__ void add_candidate(NoAllocScratch* S, bool take, doub
         S->cand_u[pos] = upper[v];
         S->cand_id[pos] = (int)v;
     }
+    return base < (unsigned long long)NA_CAP;
 }
 
 __global__ void __launch_bounds__(256)
@@ -212,7 +214,8 @@ na_compact(NoAllocScratch* S, const double* __restrict__ lower, const double* __
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const long long v = base + q * 256 + threadIdx.x;
-            add_candidate(S, v < n && (unsigned int)(order_bits(l[q]) >> 32) >= gk, l[q], upper, v);
+            if (!add_candidate(S, v < n && (unsigned int)(order_bits(l[q]) >> 32) >= gk, l[q], upper, v))
+                return;  // the radix select counts them all again
         }
     }
 }
@@ -222,44 +225,66 @@ __device__ __forceinline__ bool radix_needed(const NoAllocScratch* S) {
 }
 
 // pick the bucket that holds the k-th key (one block); stop once all keys from
-// that bucket up fit the candidate buffer
+// that bucket up fit the candidate buffer.  A warp sums 128 bins a load, and one
+// warp looks through the 128 that hold the key: with a thread per 128 bins, each
+// walking its own one load at a time, na_radix of 9000 nodes took 60 us, 11 so.
 __device__ void radix_find(NoAllocScratch* S, int pass) {
-    __shared__ unsigned long long part[NA_RADIX_THREADS];
-    __shared__ int sel;
-    __shared__ unsigned long long cum_sel;
-    const int tid = threadIdx.x;
-    constexpr int per = NA_BINS / NA_RADIX_THREADS;
-    // thread tid owns bins [NA_BINS-1 - tid*per - (per-1), NA_BINS-1 - tid*per], visited from the top
-    unsigned long long s = 0;
-    for (int q = 0; q < per; ++q) s += __ldcg(&S->hist[NA_BINS - 1 - tid * per - q]);
-    part[tid] = s;
-    if (tid == 0) sel = -1;
-    __syncthreads();
-    for (int off = 1; off < NA_RADIX_THREADS; off <<= 1) {
-        const unsigned long long a = tid >= off ? part[tid - off] : 0ull;
-        __syncthreads();
-        part[tid] += a;
-        __syncthreads();
+    constexpr int SLICES = NA_BINS / 128, WARPS = NA_RADIX_THREADS / 32;
+    static_assert(SLICES == NA_RADIX_THREADS, "a thread per slice in the scan");
+    __shared__ unsigned int part[SLICES], warp_sum[WARPS];  // a digit's counts stay below 2^31
+    __shared__ int s_slice, s_bin;
+    __shared__ unsigned int s_cum, s_count;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const uint4* h4 = (const uint4*)S->hist;
+    // slice i: the 128 bins from NA_BINS - 128 (i + 1) on; slices count from the top
+    auto slice_load = [&](int i, int l) { return __ldcg(h4 + (NA_BINS / 4 - 32 * (i + 1) + l)); };
+#pragma unroll 8
+    for (int q = 0; q < SLICES / WARPS; ++q) {
+        const int i = q * WARPS + wid;
+        const uint4 v = slice_load(i, lane);
+        const unsigned int sum = __reduce_add_sync(0xffffffffu, v.x + v.y + v.z + v.w);
+        if (lane == 0) part[i] = sum;
     }
-    const unsigned long long k = S->k_rem;
-    unsigned long long cum = tid ? part[tid - 1] : 0ull;
-    if (cum < k && part[tid] >= k) {
-        for (int q = 0; q < per; ++q) {
-            const int b = NA_BINS - 1 - tid * per - q;
-            const unsigned long long h = __ldcg(&S->hist[b]);
-            if (cum + h >= k) {
-                sel = b;
-                cum_sel = cum;
-                break;
-            }
-            cum += h;
+    if (tid == 0) s_slice = s_bin = -1;
+    __syncthreads();
+    const unsigned int k = (unsigned int)S->k_rem;
+    auto scan = [&](unsigned int x) {  // inclusive, over the lanes
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned int y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        return x;
+    };
+    const unsigned int mine = part[tid];
+    unsigned int upto = scan(mine);
+    if (lane == 31) warp_sum[wid] = upto;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) upto += warp_sum[w];
+    if (upto - mine < k && upto >= k) {
+        s_slice = tid;
+        s_cum = upto - mine;
+    }
+    __syncthreads();
+    if (wid == 0 && s_slice >= 0) {
+        const uint4 v = slice_load(s_slice, 31 - lane);  // lane 0: the top four bins, w the first
+        const unsigned int before = s_cum;
+        const unsigned int four = v.x + v.y + v.z + v.w, in = before + scan(four);
+        unsigned int cum = in - four;
+        if (cum < k && in >= k) {
+            const unsigned int h[4] = {v.w, v.z, v.y, v.x};
+            int q = 0;
+            while (cum + h[q] < k) cum += h[q++];
+            s_bin = NA_BINS - 1 - 128 * s_slice - 4 * lane - q;
+            s_count = h[q];
+            s_cum = cum;
         }
     }
     __syncthreads();
-    const int b = sel;
-    const unsigned long long hb = b >= 0 ? __ldcg(&S->hist[b]) : 0ull;
-    __syncthreads();
-    for (int q = tid; q < NA_BINS; q += NA_RADIX_THREADS) S->hist[q] = 0;  // ready for the next pass
+    const int b = s_bin;
+    const unsigned long long hb = s_count, cum_sel = s_cum;
+    for (int q = tid; q < NA_BINS / 4; q += NA_RADIX_THREADS)  // ready for the next pass
+        ((uint4*)S->hist)[q] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0 && b >= 0) {
         const int shift = 80 - 16 * pass;
         const u128 pre = (((u128)S->pre_hi << 32) | S->pre_lo) | ((u128)(unsigned)b << shift);
