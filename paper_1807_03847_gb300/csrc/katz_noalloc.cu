@@ -13,7 +13,9 @@
 //
 // Its work is the selection and checking half of an iteration of the
 // library's main loop, run over all n nodes:
-//   groups   the nodes fall into 8192 groups by a hash of their id; the k-th
+//   begin    where groups are not needed: every node fits the candidate buffer, or
+//            k is above 4096;
+//   groups   else: the nodes fall into 8192 groups by a hash of their id; the k-th
 //            largest of the groups' largest lower bounds, cut to its upper 22
 //            bits, is reached by at least k nodes, and by few more (about 1660
 //            for k = 1500, wherever the large bounds lie);
@@ -97,6 +99,26 @@ __device__ __forceinline__ u128 key_of(double l, int v) {
     return ((u128)order_bits(l) << 32) | (u128)(0xffffffffu ^ (unsigned)v);
 }
 
+// what a call starts from
+__device__ __forceinline__ void begin_call(NoAllocScratch* S, long long k, int use_radix) {
+    S->cand_count = 0;
+    S->cross = 0;
+    S->above = 0;
+    S->k_rem = (unsigned long long)k;
+    S->pre_hi = 0;
+    S->pre_lo = 0;
+    S->done = 0;
+    S->use_radix = use_radix;
+    S->group_key = 0;  // unless the groups give one: every node is taken
+}
+
+// the start of a call that needs no groups: every node fits the buffer, or k is
+// too large for them
+__global__ void na_begin(NoAllocScratch* S, long long k, int use_radix) {
+    S->ticket = 0;
+    begin_call(S, k, use_radix);
+}
+
 // The largest lower bound (upper 32 key bits; 0: no node) of thread t's nodes
 // i 65536 + (t ^ mix(i)), i = 0, 1, ...; the last block takes the k-th largest
 // over the groups of eight threads s 8192 + (g ^ mix(s)).  Neighbouring large
@@ -126,19 +148,7 @@ na_groups(NoAllocScratch* S, const double* __restrict__ lower, long long n, long
     }
     S->hist[t] = m;
     if (!last_block(&S->ticket)) return;
-    if (tid == 0) {
-        S->cand_count = 0;
-        S->cross = 0;
-        S->above = 0;
-        S->k_rem = (unsigned long long)k;
-        S->pre_hi = 0;
-        S->pre_lo = 0;
-        S->done = 0;
-        S->use_radix = k > NA_GROUP_MAX_K && n > NA_CAP;
-        S->group_key = 0;  // unless the groups give one below: every node is taken
-    }
-    if (k > NA_GROUP_MAX_K || n <= NA_CAP) return;
-    __syncthreads();
+    if (tid == 0) begin_call(S, k, 0);  // and the key below
     constexpr int PER = NA_GROUPS / NA_GROUP_THREADS;
     unsigned int g[PER];
 #pragma unroll
@@ -443,13 +453,17 @@ extern "C" katz_status katz_certify_topk_noalloc(const double* lower, const doub
     const long long nn = (long long)n, kk = (long long)k;
     const long long cap = 8LL * sms;  // eight 256-thread blocks per multiprocessor, grid-stride beyond
     const int grid = (int)((n + 1023) / 1024 < cap ? (n + 1023) / 1024 : cap);
-    // calls that overlapped may have left a count behind: it would make every
-    // later call wrong (2 us of 92 at n = 4 M)
-    if (cudaMemsetAsync(&S->ticket, 0, sizeof(S->ticket), s) != cudaSuccess) {
-        cudaGetLastError();
-        return KATZ_ECUDA;
+    // either start clears the count of finished blocks: calls that overlapped may
+    // have left one behind, which would make every later call wrong
+    if (n <= NA_CAP || k > NA_GROUP_MAX_K) {
+        na_begin<<<1, 1, 0, s>>>(S, kk, n > NA_CAP);
+    } else {
+        if (cudaMemsetAsync(&S->ticket, 0, sizeof(S->ticket), s) != cudaSuccess) {
+            cudaGetLastError();
+            return KATZ_ECUDA;
+        }
+        na_groups<<<NA_GROUP_BLOCKS, NA_GROUP_THREADS, 0, s>>>(S, lower, nn, kk);
     }
-    na_groups<<<NA_GROUP_BLOCKS, NA_GROUP_THREADS, 0, s>>>(S, lower, nn, kk);
     na_compact<<<grid, 256, 0, s>>>(S, lower, upper, nn);
     if (n > NA_CAP) {  // else every node fits
         const int rgrid = (int)((n + NA_RADIX_THREADS - 1) / NA_RADIX_THREADS < cap / 2
