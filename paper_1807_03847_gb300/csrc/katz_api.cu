@@ -33,10 +33,18 @@ katz_status fail(katz_handle* h, katz_status s, const std::string& msg) {
     return s;
 }
 
+// The status of a failed CUDA call.  One that found no memory leaves nothing
+// behind but its error, which would fail the next call's first launch check.
+static katz_status status_of(cudaError_t e) {
+    if (e != cudaErrorMemoryAllocation) return KATZ_ECUDA;
+    cudaGetLastError();
+    return KATZ_ENOMEM;
+}
+
 katz_status cuda_fail(katz_handle* h, cudaError_t e, const char* what) {
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     if (h) h->err = m;
-    return e == cudaErrorMemoryAllocation ? KATZ_ENOMEM : KATZ_ECUDA;
+    return status_of(e);
 }
 
 bool is_device_ptr(const void* p) {
@@ -1288,8 +1296,7 @@ katz_status update_prepare(katz_handle* h, const int32_t* src, const int32_t* ds
         return st;
     };
     auto cuda_done = [&](cudaError_t ce, const char* what) {
-        return done(ce == cudaErrorMemoryAllocation ? KATZ_ENOMEM : KATZ_ECUDA,
-                    (std::string(what) + ": " + cudaGetErrorString(ce)).c_str());
+        return done(status_of(ce), (std::string(what) + ": " + cudaGetErrorString(ce)).c_str());
     };
     // the spare buffers held the graph before the current one: the repair
     // that read it is queued on the handle's stream before ev_committed
