@@ -426,40 +426,41 @@ katz_status dyn_reserve(katz_handle* h, int64_t m, int64_t nnz_cap, cudaStream_t
     const int64_t n = g.n;
 #define DALLOC(ptr, cnt)                                                      \
     if ((e = dmalloc_on(h, &(ptr), (size_t)(cnt), st)) != cudaSuccess) return cuda_fail(h, e, "cudaMalloc " #ptr);
+#define DALLOC_ONCE(ptr, cnt) \
+    if (!(ptr)) DALLOC(ptr, cnt)
     if (!h->stream_a) {
         if ((e = cudaStreamCreateWithFlags(&h->stream_a, cudaStreamNonBlocking)) != cudaSuccess ||
             (e = cudaEventCreateWithFlags(&h->ev_prepared, cudaEventDisableTiming)) != cudaSuccess ||
             (e = cudaEventCreateWithFlags(&h->ev_committed, cudaEventDisableTiming)) != cudaSuccess)
             return cuda_fail(h, e, "update stream");
     }
-    if (!d.delta) {
-        DALLOC(d.delta, n);
-        DALLOC(d.ins_cnt, n);
-        DALLOC(d.cursor, n);
-        DALLOC(d.touched, (n + 3) / 4 * 4);  // whole words: rows are claimed with word atomics
-        DALLOC(d.ins_start, n);
-        DALLOC(d.vbits, (n + 31) / 32);
-        DALLOC(d.frontier, n);
-        DALLOC(d.fsize, 2);
-        DALLOC(d.hub_epoch, std::max<int64_t>(g.layout.row_warp, 1));
-        DALLOC(d.n_ins_rows, 1);
-        DALLOC(d.err, 2);
-        DALLOC(d.mode_dmax, 4);
-        DALLOC(h->rp_new, n + 1);
-        DALLOC(h->deg_tmp, n + 1);
-        DALLOC(h->scan_sums, scan_blocks(n + 1));
-        if (g.off64) {
-            int64_t* rp = nullptr;
-            DALLOC(rp, n + 1);
-            h->rowptr_spare = rp;
-        } else {
-            int32_t* rp = nullptr;
-            DALLOC(rp, n + 1);
-            h->rowptr_spare = rp;
-        }
-        DALLOC(h->chunk_first_spare, g.layout.row_warp + 1);
+    if (!h->dyn_ready) {
+        // what an earlier call left allocated when it found no memory is kept; its
+        // allocations may have been ordered on the other stream
+        if (d.delta && ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess ||
+                        (e = cudaStreamSynchronize(h->stream_a)) != cudaSuccess))
+            return cuda_fail(h, e, "update scratch");
+        DALLOC_ONCE(d.delta, n);
+        DALLOC_ONCE(d.ins_cnt, n);
+        DALLOC_ONCE(d.cursor, n);
+        DALLOC_ONCE(d.touched, (n + 3) / 4 * 4);  // whole words: rows are claimed with word atomics
+        DALLOC_ONCE(d.ins_start, n);
+        DALLOC_ONCE(d.vbits, (n + 31) / 32);
+        DALLOC_ONCE(d.frontier, n);
+        DALLOC_ONCE(d.fsize, 2);
+        DALLOC_ONCE(d.hub_epoch, std::max<int64_t>(g.layout.row_warp, 1));
+        DALLOC_ONCE(d.n_ins_rows, 1);
+        DALLOC_ONCE(d.err, 2);
+        DALLOC_ONCE(d.mode_dmax, 4);
+        DALLOC_ONCE(h->rp_new, n + 1);
+        DALLOC_ONCE(h->deg_tmp, n + 1);
+        DALLOC_ONCE(h->scan_sums, scan_blocks(n + 1));
+        char* rp = (char*)h->rowptr_spare;
+        DALLOC_ONCE(rp, (n + 1) * (g.off64 ? sizeof(int64_t) : sizeof(int32_t)));
+        h->rowptr_spare = rp;
+        DALLOC_ONCE(h->chunk_first_spare, g.layout.row_warp + 1);
         const int64_t chunk_cap = h->chunk_row_cap + h->chunk_row_cap / 8 + 16;  // batches may add chunks
-        DALLOC(h->chunk_row_spare, chunk_cap);
+        DALLOC_ONCE(h->chunk_row_spare, chunk_cap);
         h->chunk_row_spare_cap = chunk_cap;
         if ((e = cudaMemsetAsync(d.delta, 0, (size_t)n * sizeof(int32_t), st)) != cudaSuccess ||
             (e = cudaMemsetAsync(d.ins_cnt, 0, (size_t)n * sizeof(int32_t), st)) != cudaSuccess ||
@@ -469,6 +470,7 @@ katz_status dyn_reserve(katz_handle* h, int64_t m, int64_t nnz_cap, cudaStream_t
                 cudaSuccess)
             return cuda_fail(h, e, "memset dynamic scratch");
         h->col_cap = g.nnz;
+        h->dyn_ready = true;
     }
     if (m > h->bcap) {  // both batch sets (called before any batch is in flight, or for the first one)
         for (int q = 0; q < 2; ++q) {
@@ -515,6 +517,7 @@ katz_status dyn_reserve(katz_handle* h, int64_t m, int64_t nnz_cap, cudaStream_t
         DALLOC(h->col_spare, nnz_cap);
         h->col_spare_cap = nnz_cap;
     }
+#undef DALLOC_ONCE
 #undef DALLOC
     return KATZ_OK;
 }

@@ -60,6 +60,7 @@ struct katz_handle {
     cudaStream_t stream_a = nullptr;
     cudaEvent_t ev_prepared = nullptr;   // stream_a: the prepared graph is complete
     cudaEvent_t ev_committed = nullptr;  // stream: work on the previous graph is queued before this
+    bool dyn_ready = false;              // the update scratch that does not depend on the batch is allocated
     void* rowptr_spare = nullptr;        // [n+1], the offset type of g.rowptr
     // a batch that takes n + nnz past the int32 offset range: the new int64
     // offsets and the int64 spare that replace the two int32 arrays at its swap

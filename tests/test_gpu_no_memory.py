@@ -79,7 +79,7 @@ def child(kind):
     assert np.array_equal(h.ranking(100), ref.ranking(100))
 
 
-@pytest.mark.parametrize("kind", ["rank"])
+@pytest.mark.parametrize("kind", ["rank", "update"])
 def test_call_without_memory_then_with_it(kind):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     p = subprocess.run([sys.executable, os.path.abspath(__file__), kind], capture_output=True, text=True, timeout=300,
