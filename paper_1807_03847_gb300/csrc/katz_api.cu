@@ -1466,6 +1466,19 @@ katz_status update_swap(katz_handle* h) {
         return pd.status != KATZ_OK ? fail(h, pd.status, pd.err) : KATZ_OK;
     }
     {
+        // before anything is swapped: without this memory the graph stays as it was
+        if (pd.chunks > h->chunk_part_cap) {
+            const int64_t cap = pd.chunks + pd.chunks / 8 + 16;
+            double* part = nullptr;
+            if ((e = dmalloc(h, &part, 3 * (size_t)cap)) != cudaSuccess) {
+                h->rep.applied = false;
+                cudaEventRecord(h->ev_committed, h->stream);
+                return cuda_fail(h, e, "cudaMalloc chunk sums");
+            }
+            dfree(h, g.chunk_part);
+            g.chunk_part = part;
+            h->chunk_part_cap = cap;
+        }
         std::swap(g.col, h->col_spare);
         std::swap(h->col_cap, h->col_spare_cap);
         if (pd.promote) {  // int32 -> int64 offsets; the old arrays are released after the work queued on them
@@ -1483,15 +1496,6 @@ katz_status update_swap(katz_handle* h) {
         std::swap(g.chunk_row, h->chunk_row_spare);
         std::swap(h->chunk_row_cap, h->chunk_row_spare_cap);
         g.nnz = pd.nnz;
-        if (pd.chunks > h->chunk_part_cap) {
-            dfree(h, g.chunk_part);
-            g.chunk_part = nullptr;
-            h->chunk_part_cap = 0;
-            const int64_t cap = pd.chunks + pd.chunks / 8 + 16;
-            if ((e = dmalloc(h, &g.chunk_part, 3 * (size_t)cap)) != cudaSuccess)
-                return cuda_fail(h, e, "cudaMalloc chunk sums");
-            h->chunk_part_cap = cap;
-        }
         g.layout = make_layout(n, g.layout.row_warp, g.layout.row_octet, g.layout.row_thread, pd.chunks);
         h->classes_exact = false;  // rows keep their place while their degrees change
         drop_graph(h);             // captured launches hold the old arrays and layout
