@@ -157,13 +157,14 @@ __global__ void new_degree_kernel(const Off* __restrict__ rowptr, const int32_t*
 constexpr unsigned FULL_MASK = 0xffffffffu;
 
 constexpr int REMAP_UNROLL = 4;  // arcs per lane in flight
-constexpr int REMAP_TILE = 1024;  // rows plus arcs per warp
+constexpr int REMAP_TILE = 1024;  // rows plus arcs per warp, at most
+constexpr int REMAP_MIN = 128;    // and at least
 
 // Arcs [a0, a1) of the original rows [v0, v1), renamed, into their new rows
 // inv[v].  The work is cut along the merge of rows and arcs: one warp takes
-// REMAP_TILE consecutive items, row v sitting just before its arcs, so a warp
-// meets at most REMAP_TILE arcs whatever the degrees (R-MAT keeps its hubs at
-// neighbouring ids) and at most REMAP_TILE rows where most are empty.  A warp
+// tile_items consecutive items, row v sitting just before its arcs, so a warp
+// meets at most so many arcs whatever the degrees (R-MAT keeps its hubs at
+// neighbouring ids) and at most so many rows where most are empty.  A warp
 // per 32 rows left the few groups of hub rows running alone: 321 us per slice
 // of 8.4 M arcs of R-MAT21, against 64 us with the tiles.  The lanes
 // scan the lengths of 32 rows, clipped to the tile, then walk their arcs
@@ -174,15 +175,15 @@ constexpr int REMAP_TILE = 1024;  // rows plus arcs per warp
 template <typename Off>
 __global__ void remap_rows_kernel(const Off* __restrict__ rowptr, const int32_t* __restrict__ col,
                                   const int32_t* __restrict__ inv, const int64_t* __restrict__ rowptr_new, int64_t v0,
-                                  int64_t v1, int64_t a0, int64_t a1, int64_t n, int32_t* __restrict__ col_new,
-                                  unsigned long long* bad) {
+                                  int64_t v1, int64_t a0, int64_t a1, int64_t n, int tile_items,
+                                  int32_t* __restrict__ col_new, unsigned long long* bad) {
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
     const int lane = threadIdx.x & 31;
     const int64_t items = (v1 - v0) + (a1 - a0);
-    const int64_t tiles = (items + REMAP_TILE - 1) / REMAP_TILE;
+    const int64_t tiles = (items + tile_items - 1) / tile_items;
     unsigned long long nb = 0;
     for (int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; tile < tiles; tile += warps) {
-        const int64_t d0 = tile * REMAP_TILE, d1 = min(d0 + REMAP_TILE, items);
+        const int64_t d0 = tile * tile_items, d1 = min(d0 + tile_items, items);
         // the last row that sits at or before item d0: 32 rows probed at a time
         int64_t lo = v0, hi = v1;  // row lo sits at or before d0, row hi after it (or is the end)
         while (hi - lo > 1) {
@@ -469,9 +470,14 @@ cudaError_t remap_rows(const int64_t* rowptr64, const int32_t* col, const int32_
                        int64_t v0, int64_t v1, int64_t a0, int64_t a1, int64_t n, int32_t* col_new,
                        unsigned long long* bad, cudaStream_t st) {
     if (v1 <= v0 || a1 <= a0) return cudaSuccess;
-    const int64_t tiles = ((v1 - v0) + (a1 - a0) + REMAP_TILE - 1) / REMAP_TILE;
+    // smaller tiles where there are too few for the warps of the chip: a create of
+    // 2^22 rows of degree 4 from host slices 758 -> 713 us, of R-MAT18 512 -> 411
+    const int64_t items = (v1 - v0) + (a1 - a0);
+    int tile = REMAP_TILE;
+    while (tile > REMAP_MIN && items < (int64_t)tile * 152 * 48) tile /= 2;
+    const int64_t tiles = (items + tile - 1) / tile;
     remap_rows_kernel<int64_t><<<grid_for(tiles * 32, 256, 152 * 32), 256, 0, st>>>(
-        rowptr64, col, inv, rowptr_new, v0, v1, a0, a1, n, col_new, bad);
+        rowptr64, col, inv, rowptr_new, v0, v1, a0, a1, n, tile, col_new, bad);
     return cudaGetLastError();
 }
 
