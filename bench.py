@@ -510,8 +510,9 @@ def spmv_roofline(infos, n, nnz, off64, fp32_run, hbm_peak, hbm_src, tr):
             "peak_source": f"{hbm_src} hbm_gbs (burst copy)",
             "algorithmic_bytes_per_launch": bytes_alg, "spmv_ms_per_launch": t_launch * 1e3,
             "gathers_per_s": nnz / t_launch, "launches": launches,
-            "limiter": "random gathers of s_{r-1} (one L1 request per arc; beyond L2 one DRAM sector per "
-                       "missed gather) and, for FP64 levels, the integer adds of the exact row sums"}
+            "limiter": ("staged gathers: L2 requests of the staged values and the latency of the short rows, "
+                        "then the staging pass" if n >= 1 << 25 else
+                        "random gathers of s_{r-1}: one L1 request per arc, L2 behind it")}
 
 
 def deviation_stats(lo, up, err, l_ref, u_ref):

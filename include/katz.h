@@ -455,12 +455,13 @@ void katz_server_destroy(katz_server_h s);
  *
  * The work is queued on cuda_stream (NULL: the default stream) and the call
  * returns without waiting for it.  The first call on a device, with that
- * device current, looks up the array's device address and raises the sort
- * kernel's shared-memory limit; make that first call before any stream
- * capture begins on that device.  Every call on a device uses the same
+ * device current, looks up the array's device address and the device's
+ * multiprocessor count; make that first call before any stream capture
+ * begins on that device.  Every call on a device uses the same
  * array, which keeps the contents of the last call; each call clears what
  * must start at zero.  Calls whose work overlaps on the GPU (streams with no
- * ordering between them) race on the array and give wrong results.
+ * ordering between them) race on the array and give wrong results; a later
+ * call that overlaps with none is right again.
  * No handle: errors are reported by the return value alone.
  * Errors: KATZ_EINVAL (NULL pointer, sizes above the limits), KATZ_ECUDA
  * (device lookup or a launch failed).

@@ -312,12 +312,6 @@ katz_status take_trace(katz_handle* h) {
     return e == cudaSuccess ? KATZ_OK : cuda_fail(h, e, "copy trace");
 }
 
-// Run iterations until the device sets ctrl.stop (converged or r_max).
-// Graph mode: one graph launch runs the whole loop on the device; the host
-// only steps in when the candidate set outgrows the one-CTA select.
-// Host mode: iterations are launched in batches and ctrl is read between
-// batches (launches after a stop return at once).  done: iterations already
-// enqueued by the caller (profile events of the loop's launches follow theirs).
 // one pair of timing events per iteration up to r_max (profile mode)
 katz_status ensure_prof_events(katz_handle* h) {
     cudaError_t e;
@@ -330,6 +324,11 @@ katz_status ensure_prof_events(katz_handle* h) {
     return KATZ_OK;
 }
 
+// Run iterations until the device sets ctrl.stop (converged or r_max).
+// Graph mode: one graph launch runs the whole loop on the device.
+// Host mode: iterations are launched in batches and ctrl is read between
+// batches (launches after a stop return at once).  done: iterations already
+// enqueued by the caller (profile events of the loop's launches follow theirs).
 katz_status run_loop(katz_handle* h, int done) {
     cudaError_t e;
     const bool graph_mode = h->opts.use_graph && !h->opts.profile;
@@ -1023,7 +1022,7 @@ static katz_status rank_static_once(katz_h h, double alpha, int64_t k, double ep
     h->last_ms = ms;
     if ((st = take_trace(h)) != KATZ_OK) return st;
     if (h->opts.use_graph && !h->opts.profile)
-        // loop bodies that did work: all finalize runs but the first iteration's
+        // loop bodies that did work: all levels closed but the first
         h->launches += iteration_kernels(h) * std::max<int64_t>(0, (int64_t)hc.body_runs - 1);
     double spmv_ms = 0.0;
     if (h->opts.profile) {  // levels 2..r: level 1 reads no walk values

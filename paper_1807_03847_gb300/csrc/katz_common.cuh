@@ -47,7 +47,7 @@ struct Ctrl {
     int32_t theta_id;    // original id of the k-th node (ties of l broken by smaller id)
     int32_t k_eff;       // entries in the top-k list
     double tau;          // candidate filter used by the select (diagnostic)
-    unsigned long long body_runs;  // loop bodies executed (finalize calls that did work)
+    unsigned long long body_runs;  // levels closed by a count
     // FP32-certified mode (unused in FP64 mode): levels >= f32_from are FP32
     int32_t f32_from;    // first FP32 level (INT32_MAX: none yet)
     int32_t stall;       // 1: rounding widening dominates; more iterations cannot certify
@@ -150,12 +150,12 @@ __device__ __forceinline__ double walk_value(const double* walk, const IterParam
 
 // ---- launchers (katz_kernels.cu) -------------------------------------------
 
-// Internal row ranges of the SpMV row modes and their block ranges.
 // Staged gathers (katz_stage.cu): from this many vertices, with this many of
 // the vector's first entries (64 MB of FP64, half of L2) gathered directly
 constexpr int64_t STAGE_MIN_N = (int64_t)1 << 25;
 constexpr int64_t STAGE_HOT = (int64_t)1 << 23;
 
+// Internal row ranges of the SpMV row modes and their block ranges.
 struct SpmvLayout {
     int64_t n;
     int64_t row_warp;    // rows [0, row_warp): CHUNK mode (degree > 2048)
@@ -371,14 +371,14 @@ cudaError_t launch_spmv(const DeviceGraph& g, const IterBuffers& b, const IterPa
 cudaError_t launch_stage(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, cudaStream_t st);
 cudaError_t launch_spmv_store(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int level,
                               cudaStream_t st);
-// s_level recomputed for the listed rows (CHUNK rows excepted) and for the
-// CHUNK rows whose visit bit is set, with the lane partition of the SpMV
 cudaError_t launch_pair_levels(const DeviceGraph& ga, const DeviceGraph& gb, const int32_t* bsrc,
                                const int32_t* bdst, int64_t m, const IterParams& p, int r, int f32_from,
                                int t_level, double* P, int64_t pstride, float* t_pair, double* part,
                                uint32_t* vbits, int32_t* rows, unsigned long long* nrows, cudaStream_t st);
 cudaError_t launch_pair_split(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int r, int f32_from,
                               int state, const double* P, int64_t pstride, const float* t_pair, cudaStream_t st);
+// s_level recomputed for the listed rows (CHUNK rows excepted) and for the
+// CHUNK rows whose visit bit is set, with the lane partition of the SpMV
 cudaError_t launch_rows_store(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, const int32_t* rows,
                               const unsigned long long* nrows_dev, int64_t nrows_max, const uint32_t* vbits,
                               int level, cudaStream_t st);
@@ -394,7 +394,5 @@ int sum_depth_of(int64_t deg_thread, int64_t deg_octet, int64_t deg_warp, bool h
                  int64_t max_chunks_per_row);
 cudaError_t launch_walk_out(const DeviceGraph& g, const IterBuffers& b, const IterParams& p, int level, bool fp32,
                             double* out, cudaStream_t st);
-// radix select over candidates (large candidate sets): one pass of 8-bit digits
-
 
 }  // namespace katz

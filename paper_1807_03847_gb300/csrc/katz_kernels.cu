@@ -551,7 +551,7 @@ __device__ __noinline__ void finalize_level(const double* __restrict__ topk_l, c
 // M is read from a compact list of its nodes: the first count after all
 // nodes became active scans the flags of all of V instead.  Either way the
 // survivors are written, in tiles, to the other list buffer (one atomic per
-// tile for its place), which finalize then makes current.  The order of a
+// tile for its place), which the level's end then makes current.  The order of a
 // list is arbitrary; nothing computed from it depends on the order.
 //
 // The block that finishes last closes the level (finalize_level): as a kernel
@@ -733,7 +733,7 @@ __global__ void cert_init_kernel(Ctrl* ctrl, IterParams p) {
 // FP32-certified handles whose summation depth grew (an update batch made a
 // row longer than its row mode's nominal limit): the error state of level r
 // replayed from level 1 with the new depth.  This is the recursion the
-// ranking ran level by level (cert_init, then finalize), with the switch
+// ranking ran level by level (cert_init, then each level's end), with the switch
 // level it chose; the repaired levels satisfy the larger bounds, and so do
 // the levels left as they were.
 __global__ void cert_replay_kernel(Ctrl* ctrl, IterParams p, int r) {
