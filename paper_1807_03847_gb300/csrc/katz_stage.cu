@@ -24,16 +24,18 @@
 // + 4 and 4) in place of 128.  The values and the order of every row sum are
 // those of the plain gather, so the results are the same bits.
 //
-// Measured on that graph, FP64: a level 17.1 -> 11.4 ms (2.3 of it step 1), the
-// ranking 193 -> 131 ms; n = 6e7: 63.2 -> 54.9 ms, FP32-certified 57.3 -> 53.1;
-// n = 4e7: 38.2 -> 36.1; G(3.6e7, 4 n): 48.8 -> 27.9.  Building it takes no more of
-// a create than the anchor order (katz_relabel.cu), which it replaces: 61 against
-// 77 ms at 2^27.  Below 2^25 vertices the gain (2.68 -> 2.54 ms a level at 2^25 - 39)
-// does not pay for a create three times as long.
+// Measured on that graph, FP64: a level 17.1 -> 11.4 ms when it came, 10.6 now with
+// fewer rows per warp (1.8 of it step 1; 37.4 GB read and 7.8 written by both
+// steps).  Rankings before it and now, the SpMV's row batches included: 185 -> 121
+// ms; Chung-Lu n = 6e7: 64.7 -> 48.6, FP32-certified 59.4 -> 47.6; n = 4e7: 39.1 ->
+// 32.0; G(3.6e7, 4 n): 50.3 -> 27.9.  Building it takes no more of a create than the
+// anchor order (katz_relabel.cu), which it replaces: 59 against 75 ms at 2^27.
+// Below 2^25 vertices the gain (2.68 -> 2.54 ms a level at 2^25 - 39) does not pay
+// for a create three times as long.
 //
-// 2^23 hot entries, 8192 per window: with 2^22 the level took 11.6 ms, 2^21 12.5,
-// 2^24 12.3 (the hot part then contends for L2); 64 or 128 bands changed nothing;
-// windows of 16384 (one block per SM) 16.1 ms with 16 bands.
+// 2^23 hot entries, 8192 per window: against 11.4 ms a level then, 2^22 took 11.6 ms,
+// 2^21 12.5, 2^24 12.3 (the hot part contends for L2); 64 or 128 bands changed
+// nothing; windows of 16384 (one block per SM) 16.1 ms with 16 bands.
 #include <stdint.h>
 
 #include <algorithm>
